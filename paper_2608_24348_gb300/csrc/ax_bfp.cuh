@@ -287,14 +287,18 @@ __device__ __forceinline__ float bfp_two_sum(float a, float b, float &err)
 // One element.  load(p) -> double (u at local node p), store(p, double).
 // geo: the element's float-pair factors [7][NP^3].  slab: 3 slabs; red: 8
 // words (the exponent reduction).  after_load() runs on every thread after
-// the first block barrier, when no thread reads u any more.  All threads of
-// the block call it (barriers are block-wide).
-template <int NP, bool PAIR, class Load, class Store, class After>
+// the first barrier, when no thread reads u any more.  All threads of
+// the element's group call it; sync() is the group's barrier (block-wide by default).
+struct BlockSync {
+    __device__ __forceinline__ void operator()() const { __syncthreads(); }
+};
+
+template <int NP, bool PAIR, class Load, class Store, class After, class Sync = BlockSync>
 __device__ __forceinline__ void ax_bfp_element(const Load &load, const Store &store,
                                                const dfp *__restrict__ geo, dfp h1, dfp h2,
                                                const BfpTabs &T, dfp *__restrict__ slab,
                                                unsigned *red, int tid, bool active,
-                                               const After &after_load)
+                                               const After &after_load, const Sync &sync = Sync())
 {
     using Cf = BfpCfg<NP>;
     constexpr int NP2 = Cf::NP2, NP3 = Cf::NP3, LS = Cf::LS, SL = Cf::SLAB;
@@ -312,7 +316,7 @@ __device__ __forceinline__ void ax_bfp_element(const Load &load, const Store &st
         }
     }
     bfp_group_max_write<NP>(m, red, tid);
-    __syncthreads();
+    sync();
     after_load();
     const unsigned bmax = bfp_group_max_read<NP>(red);
     // u 2^-E has |.| < 1
@@ -328,7 +332,7 @@ __device__ __forceinline__ void ax_bfp_element(const Load &load, const Store &st
             su[(k * NP + j) * LS + i] = ru[k];
         }
     }
-    __syncthreads();
+    sync();
     // the atomic form of the reduction starts the next element from zero
     bfp_group_max_clear<NP>(red, tid);
 
@@ -356,7 +360,7 @@ __device__ __forceinline__ void ax_bfp_element(const Load &load, const Store &st
         }
         bfp_line_sel<NP, 0, PAIR>(ru, gt, off, T);
     }
-    __syncthreads();
+    sync();
 
     // ---- geometric factors (column owner): v_a = sum_b G_ab g_b, each node on
     // its own quantum; h2 B u as a Dekker pair for the last stage
@@ -400,7 +404,7 @@ __device__ __forceinline__ void ax_bfp_element(const Load &load, const Store &st
             bu[k] = {p3, e3};
         }
     }
-    __syncthreads();
+    sync();
 
     // ---- transpose: each line re-quantised to its largest value, then folded;
     // r lines in place in sA, s lines in place in sB, t in registers
@@ -428,7 +432,7 @@ __device__ __forceinline__ void ax_bfp_element(const Load &load, const Store &st
         const float C3 = bfp_offset(__fmul_rn(T.kt, bfp_requantise<NP>(gt)));
         bfp_line_sel<NP, 1, PAIR>(gt, wt, [&](int) { return C3; }, T);
     }
-    __syncthreads();
+    sync();
 
     // ---- h1 (w_r + w_s + w_t) + h2 B u, rounded to FP64 and scaled by 2^E
     if (active) {

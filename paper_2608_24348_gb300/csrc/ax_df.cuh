@@ -242,7 +242,7 @@ __device__ __forceinline__ void ax_df_element(const Load &load, const Store &sto
     __syncthreads();
 }
 
-// Low-register variant (one thread per node, strided; every contraction read
+// Low-register variant (nthreads threads, one node each in turn; every contraction read
 // from shared memory): the FP64-accurate residual inside mixed-precision
 // refinement, where the kernel's register budget belongs to the FP32 phases.
 template <int NP>
@@ -251,30 +251,31 @@ __host__ __device__ constexpr size_t ax_df_lowreg_smem_bytes()
     return sizeof(dfp) * (2 * NP * NP + 4 * (size_t)NP * NP * NP) + 16;
 }
 
-template <int NP, class Load, class Store>
+template <int NP, class Load, class Store, class Sync>
 __device__ __forceinline__ void ax_df_element_lowreg(const Load &load, const Store &store,
                                                      const dfp *__restrict__ geo, dfp h1, dfp h2,
-                                                     const dfp *__restrict__ D, unsigned char *smem)
+                                                     const dfp *__restrict__ D, unsigned char *smem, int tid,
+                                                     int nthreads, const Sync &sync)
 {
     constexpr int NP2 = NP * NP, NP3 = NP2 * NP;
     dfp *sD = reinterpret_cast<dfp *>(smem), *sDT = sD + NP2;
     dfp *su = sDT + NP2, *svr = su + NP3, *svs = svr + NP3, *svt = svs + NP3;
     int *sexp = reinterpret_cast<int *>(svt + NP3);
-    for (int t = threadIdx.x; t < NP2; t += blockDim.x) {
+    for (int t = tid; t < NP2; t += nthreads) {
         const int a = t / NP, b = t - a * NP;
         sD[t] = D[t];
         sDT[b * NP + a] = D[t];
     }
-    if (threadIdx.x == 0) *sexp = 0;
-    __syncthreads();
+    if (tid == 0) *sexp = 0;
+    sync();
     int m = 0;
-    for (int q = threadIdx.x; q < NP3; q += blockDim.x) m = max(m, df_bexp(load(q)));
+    for (int q = tid; q < NP3; q += nthreads) m = max(m, df_bexp(load(q)));
     atomicMax(sexp, m);
-    __syncthreads();
+    sync();
     const int E = *sexp > 0 ? *sexp - 1023 : 0;
-    for (int q = threadIdx.x; q < NP3; q += blockDim.x) su[q] = df_split_scaled(load(q), E);
-    __syncthreads();
-    for (int q = threadIdx.x; q < NP3; q += blockDim.x) {
+    for (int q = tid; q < NP3; q += nthreads) su[q] = df_split_scaled(load(q), E);
+    sync();
+    for (int q = tid; q < NP3; q += nthreads) {
         const int i = q % NP, j = (q / NP) % NP, k = q / NP2;
         dfacc ar = df_mul(sDT[i], su[(k * NP + j) * NP]);
         dfacc as = df_mul(sDT[j], su[k * NP2 + i]);
@@ -295,8 +296,8 @@ __device__ __forceinline__ void ax_df_element_lowreg(const Load &load, const Sto
         svs[q] = df_raw(vs);
         svt[q] = df_raw(vt);
     }
-    __syncthreads();
-    for (int q = threadIdx.x; q < NP3; q += blockDim.x) {
+    sync();
+    for (int q = tid; q < NP3; q += nthreads) {
         const int i = q % NP, j = (q / NP) % NP, k = q / NP2;
         dfacc ar = df_mul(sD[i], svr[(k * NP + j) * NP]);
         dfacc as = df_mul(sD[j], svs[k * NP2 + i]);
@@ -313,5 +314,5 @@ __device__ __forceinline__ void ax_df_element_lowreg(const Load &load, const Sto
         df_mad(o, h2, df_raw(bu));
         store(q, df_join_scaled(df_raw(o), E));
     }
-    __syncthreads();
+    sync();
 }

@@ -20,13 +20,13 @@
 
 GsDesc sem_gs_desc(const sem_ctx *c);  // ops.cu
 
-#define SEM_DECL_NP(NPV) int sem_solve_launch_np##NPV(const SolveParams<8> &, int, int, long long, cudaStream_t);
+#define SEM_DECL_NP(NPV) int sem_solve_launch_np##NPV(const SolveParams<8> &, int, int, cudaStream_t);
 SEM_DECL_NP(2) SEM_DECL_NP(3) SEM_DECL_NP(4) SEM_DECL_NP(5) SEM_DECL_NP(6) SEM_DECL_NP(7)
 SEM_DECL_NP(8) SEM_DECL_NP(9) SEM_DECL_NP(10) SEM_DECL_NP(11) SEM_DECL_NP(12) SEM_DECL_NP(13)
 SEM_DECL_NP(14) SEM_DECL_NP(15) SEM_DECL_NP(16)
 #undef SEM_DECL_NP
 
-typedef int (*noalloc_launch_fn)(const SolveParams<8> &, int, int, long long, cudaStream_t);
+typedef int (*noalloc_launch_fn)(const SolveParams<8> &, int, int, cudaStream_t);
 static const noalloc_launch_fn k_noalloc_launch[17] = {
     nullptr, nullptr, sem_solve_launch_np2, sem_solve_launch_np3, sem_solve_launch_np4,
     sem_solve_launch_np5, sem_solve_launch_np6, sem_solve_launch_np7, sem_solve_launch_np8,
@@ -34,7 +34,7 @@ static const noalloc_launch_fn k_noalloc_launch[17] = {
     sem_solve_launch_np13, sem_solve_launch_np14, sem_solve_launch_np15, sem_solve_launch_np16};
 
 // Scratch layout (bytes from the start of the array):
-//   [0, HEAD)             solver state: SyncState, PState[8], schedule
+//   [0, HEAD)             solver state: SyncState, PState[8]
 //   [HEAD, HEAD + PART)   per-CTA partial sums
 //   [.., + TAB)           derivative matrix D (FP64) and the mass sum
 //   then 4 FP64 vectors of nL entries: r, p, w, minv
@@ -50,7 +50,6 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[NA_BYTES];
 struct NaStateHost {
     SyncState sync;
     PState st[8];
-    int sched[8 * 2 + 2];
 };
 static_assert(sizeof(NaStateHost) <= NA_HEAD, "solver state exceeds its scratch slot");
 
@@ -212,8 +211,8 @@ extern "C" int sem_pcg_solve_noalloc(int N, int nelx, int nely, int nelz, const 
     prm.timeout_ns = (long long)((o.wait_timeout_s > 0 ? o.wait_timeout_s : 10.0) * 1e9);
     prm.sync = &state->sync;
     prm.st = state->st;
-    prm.sched = state->sched;
     prm.partials = partials;
+    prm.partials_cap = (long long)(NA_PART / sizeof(double));
     ProbDesc &d = prm.prob[0];
     d.n = n;
     d.NE = (256 / (n * n)) > 0 ? 256 / (n * n) : 1;
@@ -222,7 +221,8 @@ extern "C" int sem_pcg_solve_noalloc(int N, int nelx, int nely, int nelz, const 
     d.E = E;
     d.nL = nL;
     d.nG = shape.nG;
-    d.gs = sem_gs_desc(&shape);
+    d.mesh = uq_mesh(sem_gs_desc(&shape));
+    d.dn3 = fast_div((unsigned)(d.n * d.n * d.n));
     d.volume = volume;
     d.h1 = h1;
     d.h2 = h2;
@@ -237,7 +237,7 @@ extern "C" int sem_pcg_solve_noalloc(int N, int nelx, int nely, int nelz, const 
 
     // the array keeps the previous call's contents: the solver state must start at zero
     SEM_CUDA(cudaMemsetAsync(state, 0, sizeof(NaStateHost), s));
-    rc = k_noalloc_launch[n](prm, MODE_F64N, sms, (nL + SEM_SOLVE_THREADS - 1) / SEM_SOLVE_THREADS, s);
+    rc = k_noalloc_launch[n](prm, MODE_F64N, sms, s);
     if (rc) return rc;
     NaStateHost h;
     SEM_CUDA(cudaMemcpyAsync(&h, state, sizeof(NaStateHost), cudaMemcpyDeviceToHost, s));

@@ -10,38 +10,53 @@ GsDesc sem_gs_desc(const sem_ctx *c);  // ops.cu
 int sem_alloc_ws(sem_ctx *c, int slot);  // setup.cu
 
 // Per-order kernels (solve_npXX.cu), up to 8 problems of one order.
-#define SEM_DECL_NP(NPV) int sem_solve_launch_np##NPV(const SolveParams<8> &, int, int, long long, cudaStream_t);
+#define SEM_DECL_NP(NPV) int sem_solve_launch_np##NPV(const SolveParams<8> &, int, int, cudaStream_t);
 SEM_DECL_NP(2) SEM_DECL_NP(3) SEM_DECL_NP(4) SEM_DECL_NP(5) SEM_DECL_NP(6) SEM_DECL_NP(7)
 SEM_DECL_NP(8) SEM_DECL_NP(9) SEM_DECL_NP(10) SEM_DECL_NP(11) SEM_DECL_NP(12) SEM_DECL_NP(13)
 SEM_DECL_NP(14) SEM_DECL_NP(15) SEM_DECL_NP(16)
 #undef SEM_DECL_NP
 // Mixed-order kernel for N in {5, 7, 9} (solve_multi.cu), up to 64 problems.
-int sem_solve_launch_multi(const SolveParams<SEM_MAXP> &, int, int, long long, cudaStream_t);
+int sem_solve_launch_multi(const SolveParams<SEM_MAXP> &, int, int, cudaStream_t);
 
-#define SEM_DECL_TAB(NPV) int sem_solve_tables_np##NPV(const void *);
-SEM_DECL_TAB(2) SEM_DECL_TAB(4) SEM_DECL_TAB(6) SEM_DECL_TAB(8) SEM_DECL_TAB(10) SEM_DECL_TAB(12)
-SEM_DECL_TAB(14) SEM_DECL_TAB(16)
+#define SEM_DECL_TAB(NPV) int sem_solve_tables_np##NPV(const double *);
+SEM_DECL_TAB(2) SEM_DECL_TAB(3) SEM_DECL_TAB(4) SEM_DECL_TAB(5) SEM_DECL_TAB(6) SEM_DECL_TAB(7)
+SEM_DECL_TAB(8) SEM_DECL_TAB(9) SEM_DECL_TAB(10) SEM_DECL_TAB(11) SEM_DECL_TAB(12) SEM_DECL_TAB(13)
+SEM_DECL_TAB(14) SEM_DECL_TAB(15) SEM_DECL_TAB(16)
 #undef SEM_DECL_TAB
-int sem_solve_tables_multi(int np, const void *tabs);
+int sem_solve_tables_multi(int np, const double *D);
 
-// Copies the block-floating-point tables of the context's order into the
-// constant memory of the solver kernels that serve it (the per-order unit and,
-// for N + 1 in {6, 8, 10}, the mixed-order unit), on the current device.
+// The ordered solver of Taylor-Green steps (solver_ordered.cuh), N + 1 <= 10.
+#define SEM_DECL_ORD(U)                                                        \
+    int sem_solve_ordered_##U(const SolveParams<8> &, int, int, cudaStream_t); \
+    int sem_solve_ordered_tables_##U(int, const double *);
+SEM_DECL_ORD(a) SEM_DECL_ORD(b) SEM_DECL_ORD(c)
+#undef SEM_DECL_ORD
+typedef int (*ordered_fn)(const SolveParams<8> &, int, int, cudaStream_t);
+typedef int (*ordered_tab_fn)(int, const double *);
+static const ordered_fn k_ordered[3] = {sem_solve_ordered_c, sem_solve_ordered_a, sem_solve_ordered_b};  // n % 3
+static const ordered_tab_fn k_ordered_tab[3] = {sem_solve_ordered_tables_c, sem_solve_ordered_tables_a,
+                                                sem_solve_ordered_tables_b};
+
+// Fills the constant memory of the solver kernels that serve the context's
+// order (the per-order unit, for N + 1 in {6, 8, 10} the mixed-order unit and
+// for even N + 1 <= 10 the ordered solver's) with the tables made from its derivative matrix, on the current device.
 int sem_solve_upload_tables(const sem_ctx *c)
 {
-    if (!c->bfp_tabs) return SEM_OK;  // odd N+1: no such tables
-    typedef int (*tab_fn)(const void *);
-    static const tab_fn f[17] = {nullptr, nullptr, sem_solve_tables_np2, nullptr, sem_solve_tables_np4,
-                                 nullptr, sem_solve_tables_np6, nullptr, sem_solve_tables_np8, nullptr,
-                                 sem_solve_tables_np10, nullptr, sem_solve_tables_np12, nullptr,
-                                 sem_solve_tables_np14, nullptr, sem_solve_tables_np16};
-    if (c->n < 2 || c->n > 16 || !f[c->n]) return SEM_ERR_ARG;
-    int rc = f[c->n](c->bfp_tabs);
-    if (rc == SEM_OK && (c->n == 6 || c->n == 8 || c->n == 10)) rc = sem_solve_tables_multi(c->n, c->bfp_tabs);
+    typedef int (*tab_fn)(const double *);
+    static const tab_fn f[17] = {nullptr, nullptr, sem_solve_tables_np2, sem_solve_tables_np3,
+                                 sem_solve_tables_np4, sem_solve_tables_np5, sem_solve_tables_np6,
+                                 sem_solve_tables_np7, sem_solve_tables_np8, sem_solve_tables_np9,
+                                 sem_solve_tables_np10, sem_solve_tables_np11, sem_solve_tables_np12,
+                                 sem_solve_tables_np13, sem_solve_tables_np14, sem_solve_tables_np15,
+                                 sem_solve_tables_np16};
+    if (c->n < 2 || c->n > 16) return SEM_ERR_ARG;
+    int rc = f[c->n](c->hD);
+    if (rc == SEM_OK && (c->n == 6 || c->n == 8 || c->n == 10)) rc = sem_solve_tables_multi(c->n, c->hD);
+    if (rc == SEM_OK && c->n % 2 == 0 && c->n <= 10) rc = k_ordered_tab[c->n % 3](c->n, c->hD);
     return rc;
 }
 
-typedef int (*launch8_fn)(const SolveParams<8> &, int, int, long long, cudaStream_t);
+typedef int (*launch8_fn)(const SolveParams<8> &, int, int, cudaStream_t);
 static const launch8_fn k_launch8[17] = {
     nullptr, nullptr, sem_solve_launch_np2, sem_solve_launch_np3, sem_solve_launch_np4,
     sem_solve_launch_np5, sem_solve_launch_np6, sem_solve_launch_np7, sem_solve_launch_np8,
@@ -51,7 +66,6 @@ static const launch8_fn k_launch8[17] = {
 struct SolveStateHost {
     SyncState sync;
     PState st[SEM_MAXP];
-    int sched[SEM_MAXP * 2 + 2];
 };
 
 int sem_solve_state_bytes() { return (int)sizeof(SolveStateHost); }
@@ -96,11 +110,26 @@ static int inner_tc_of(sem_dtype inner, int n)
     }
 }
 
+// Problem p on the same context and coefficients as an earlier problem q of the
+// launch takes q's Jacobi inverse instead of making (and keeping) its own.
+static bool share_jacobi(const ProbDesc &q, ProbDesc &d, const sem_ctx *cq, const sem_ctx *c)
+{
+    if (cq != c || q.h1 != d.h1 || q.h2 != d.h2) return false;
+    d.minv = q.minv;
+    d.minv32 = q.minv32;
+    d.jac_cached = q.jac_cached;
+    d.jac_shared = !q.jac_cached;
+    return true;
+}
+
 // Fills d for a solve on workspace ws; the Jacobi inverse is recomputed unless
 // ws still holds the one of (h1, h2) (and its FP32 copy when mixed), and ws
-// records what the launch leaves in minv / minv32.
+// records what the launch leaves in minv / minv32.  first .. first + nfirst:
+// the launch's earlier problems and their contexts, one of which may share its
+// Jacobi inverse.
 static void fill_desc(const sem_ctx *c, sem_ws &ws, const double *b, double *x, double h1,
-                      double h2, bool mixed, int tc, ProbDesc &d)
+                      double h2, bool mixed, int tc, ProbDesc &d, const ProbDesc *first = nullptr,
+                      sem_ctx *const *fctx = nullptr, int nfirst = 0)
 {
     memset(&d, 0, sizeof(d));
     d.n = c->n;
@@ -111,7 +140,8 @@ static void fill_desc(const sem_ctx *c, sem_ws &ws, const double *b, double *x, 
     d.E = c->E;
     d.nL = c->nL;
     d.nG = c->nG;
-    d.gs = sem_gs_desc(c);
+    d.mesh = uq_mesh(sem_gs_desc(c));
+    d.dn3 = fast_div((unsigned)(d.n * d.n * d.n));
     d.volume = c->volume;
     d.h1 = h1;
     d.h2 = h2;
@@ -121,26 +151,29 @@ static void fill_desc(const sem_ctx *c, sem_ws &ws, const double *b, double *x, 
     d.D64 = c->tab64 + 2 * c->n;
     d.D32 = c->tab32 + 2 * c->n;
     d.Ddf = (const dfp *)c->tabdf;
-    d.Ddfeo = (const dfp *)c->tabdfeo;
     d.b = b;
     d.x = x;
     d.r = ws.r;
     d.p = ws.p;
     d.w = ws.w;
     d.minv = ws.minv;
-    d.jac_cached = ws.jac_ok && ws.jac_h1 == h1 && ws.jac_h2 == h2 && (!mixed || ws.jac32_ok);
-    if (!d.jac_cached) {
-        ws.jac_ok = 1;
-        ws.jac_h1 = h1;
-        ws.jac_h2 = h2;
-        ws.jac32_ok = mixed;
-    }
+    d.y = ws.b;
+    d.vec = ((uintptr_t)b | (uintptr_t)x) % 32 == 0;
     if (mixed) {
         d.r32 = ws.r32;
         d.p32 = ws.p32;
         d.w32 = ws.w32;
         d.d32 = ws.d32;
         d.minv32 = ws.minv32;
+    }
+    for (int q = 0; q < nfirst; ++q)
+        if (share_jacobi(first[q], d, fctx[q], c)) return;
+    d.jac_cached = ws.jac_ok && ws.jac_h1 == h1 && ws.jac_h2 == h2 && (!mixed || ws.jac32_ok);
+    if (!d.jac_cached) {
+        ws.jac_ok = 1;
+        ws.jac_h1 = h1;
+        ws.jac_h2 = h2;
+        ws.jac32_ok = mixed;
     }
 }
 
@@ -160,18 +193,8 @@ static void fill_common(SolveParams<MAXP> &p, sem_ctx *owner, const sem_solve_op
     SolveStateHost *S = (SolveStateHost *)owner->solve_dev;
     p.sync = &S->sync;
     p.st = S->st;
-    p.sched = S->sched;
     p.partials = (double *)owner->partials;
-}
-
-static long long max_items(const ProbDesc *d, int np)
-{
-    long long m = 1;
-    for (int p = 0; p < np; ++p) {
-        long long a = (d[p].nL + SEM_SOLVE_THREADS - 1) / SEM_SOLVE_THREADS;
-        if (a > m) m = a;
-    }
-    return m;
+    p.partials_cap = (long long)(sem_partials_bytes(owner->num_sms) / sizeof(double));
 }
 
 static int validate_opts(const sem_solve_opts &o)
@@ -183,20 +206,22 @@ static int validate_opts(const sem_solve_opts &o)
     return SEM_OK;
 }
 
+// Plain FP64 PCG to a relative tolerance below 1e-11 runs on the native
+// FP64 operator: the float-pair and block-floating-point operators of
+// SEM_F64 carry a relative error of a few 1e-13 per application, the size
+// of such a residual, and on a singular (periodic Poisson) problem their
+// error on the constant mode can end the solve with <p,Ap> <= 0.
+static bool tight_f64(const sem_solve_opts &o) { return o.inner == SEM_F64 && !o.abs_tol && o.tol < 1e-11; }
+
 // Enqueue one launch for problems `idx` (all on owner's state buffers).
+// ordered: with the solver of solver_ordered.cuh.
 static int enqueue(sem_ctx *owner, const sem_solve_opts &o, const ProbDesc *d, int np,
-                   cudaStream_t s)
+                   cudaStream_t s, bool ordered = false)
 {
     SEM_CUDA(cudaMemsetAsync(owner->solve_dev, 0, sizeof(SolveStateHost), s));
-    const long long mi = max_items(d, np);
     bool any_tc = false;
     for (int p = 0; p < np; ++p) any_tc |= (d[p].tc != 0);
-    // Plain FP64 PCG to a relative tolerance below 1e-11 runs on the native
-    // FP64 operator: the float-pair and block-floating-point operators of
-    // SEM_F64 carry a relative error of a few 1e-13 per application, the size
-    // of such a residual, and on a singular (periodic Poisson) problem their
-    // error on the constant mode can end the solve with <p,Ap> <= 0.
-    const bool tight = o.inner == SEM_F64 && !o.abs_tol && o.tol < 1e-11;
+    const bool tight = tight_f64(o);
     const int mode = tight ? MODE_F64N
                      : o.inner == SEM_F64 ? MODE_F64
                      : o.inner == SEM_F64_NATIVE ? MODE_F64N
@@ -208,13 +233,20 @@ static int enqueue(sem_ctx *owner, const sem_solve_opts &o, const ProbDesc *d, i
         SolveParams<8> prm;
         memset(&prm, 0, sizeof(prm));
         fill_common(prm, owner, o, np);
-        for (int p = 0; p < np; ++p) prm.prob[p] = d[p];
-        rc = k_launch8[d[0].n](prm, mode, owner->num_sms, mi, s);
+        for (int p = 0; p < np; ++p) {
+            prm.prob[p] = d[p];
+            prm.order[p] = (unsigned char)p;
+        }
+        rc = ordered ? k_ordered[d[0].n % 3](prm, d[0].n, owner->num_sms, s)
+                     : k_launch8[d[0].n](prm, mode, owner->num_sms, s);
     } else {
         SolveParams<SEM_MAXP> *prm = new SolveParams<SEM_MAXP>();
         fill_common(*prm, owner, o, np);
         for (int p = 0; p < np; ++p) prm->prob[p] = d[p];
-        rc = sem_solve_launch_multi(*prm, mode, owner->num_sms, mi, s);
+        for (int n = 2, o = 0; n <= SEM_NPMAX; ++n)
+            for (int p = 0; p < np; ++p)
+                if (d[p].n == n) prm->order[o++] = (unsigned char)p;
+        rc = sem_solve_launch_multi(*prm, mode, owner->num_sms, s);
         delete prm;
     }
     if (rc) return rc;
@@ -264,9 +296,10 @@ int sem_pcg_solve_dev(sem_ctx *c, int slot, const double *b, double *x, double h
     return jac_forget(c, enqueue(c, o, &d, 1, s));
 }
 
-// Several device-pointer solves on one context (workspace slots 0..np-1) in one launch.
+// Several device-pointer solves on one context (workspace slots slot0 and up) in
+// one launch.  ordered: FP64 solves take solver_ordered.cuh.
 int sem_pcg_solve_dev_batch(sem_ctx *c, int np, const double *const *b, double *const *x, double h1,
-                            double h2, const sem_solve_opts &o, cudaStream_t s, int slot0)
+                            double h2, const sem_solve_opts &o, cudaStream_t s, int slot0, bool ordered)
 {
     if (np < 1 || np > 4 || slot0 < 0 || slot0 + np > 8) return SEM_ERR_ARG;
     for (int p = 0; p < np; ++p)
@@ -276,9 +309,13 @@ int sem_pcg_solve_dev_batch(sem_ctx *c, int np, const double *const *b, double *
                     o.inner == SEM_BF16X3_TC;  // a tensor-core path was asked for
     const int tc_nmax = (o.inner == SEM_F16X2_TC || o.inner == SEM_BF16X3_TC) ? 8 : 10;
     if (tc && c->n > tc_nmax) return SEM_ERR_ARG;
+    ordered = ordered && o.inner == SEM_F64 && !tight_f64(o) && c->n <= 10;
     ProbDesc d[8];
-    for (int p = 0; p < np; ++p) fill_desc(c, c->ws[slot0 + p], b[p], x[p], h1, h2, mixed, inner_tc_of(o.inner, c->n), d[p]);
-    return jac_forget(c, enqueue(c, o, d, np, s));
+    sem_ctx *const cs[8] = {c, c, c, c, c, c, c, c};
+    for (int p = 0; p < np; ++p)  // (the ordered solver's problems make a Jacobi inverse each)
+        fill_desc(c, c->ws[slot0 + p], b[p], x[p], h1, h2, mixed, inner_tc_of(o.inner, c->n), d[p], d, cs,
+                  ordered ? 0 : p);
+    return jac_forget(c, enqueue(c, o, d, np, s, ordered));
 }
 
 // Device address of the solver state of problem p of the last launch (iters, status).
@@ -357,7 +394,8 @@ extern "C" int sem_pcg_solve_batched(int nprob, sem_ctx *const *ctxs, const doub
             rc = sem_alloc_ws(c, slot[p]);
             if (rc) return rc;
         }
-        fill_desc(c, c->ws[slot[p]], b[p], x[p], h1[p], h2[p], mixed, inner_tc_of(o.inner, c->n), d[p]);
+        fill_desc(c, c->ws[slot[p]], b[p], x[p], h1[p], h2[p], mixed, inner_tc_of(o.inner, c->n), d[p],
+                  d.data(), ctxs, p);
     }
     sem_ctx *owner = ctxs[0];
     bool multi_ok = true, same = true;

@@ -1,13 +1,15 @@
 // solve_np03.cu -- persistent solver kernels for order N = 2 (up to 8 problems).
 #include "solver.cuh"
 
-int sem_solve_launch_np3(const SolveParams<8> &p, int mode, int sms, long long mi, cudaStream_t s)
+int sem_solve_launch_np3(const SolveParams<8> &p, int mode, int sms, cudaStream_t s)
 {
     switch (mode) {
-        case MODE_F64: return launch_solve<8, MODE_F64, 3>(p, sms, mi, s);
-        case MODE_F64N: return launch_solve<8, MODE_F64N, 3>(p, sms, mi, s);
-        case MODE_F32: return launch_solve<8, MODE_F32, 3>(p, sms, mi, s);
-        case MODE_TC: return launch_solve<8, MODE_TC, 3>(p, sms, mi, s);
+        case MODE_F64: return launch_solve<8, MODE_F64, 3>(p, sms, s);
+        case MODE_F64N: return launch_solve<8, MODE_F64N, 3>(p, sms, s);
+        case MODE_F32: return launch_solve<8, MODE_F32, 3>(p, sms, s);
+        case MODE_TC: return launch_solve<8, MODE_TC, 3>(p, sms, s);
         default: return SEM_ERR_ARG;
     }
 }
+
+int sem_solve_tables_np3(const double *D) { return solver_upload_tables(3, D); }

@@ -1,13 +1,15 @@
 // solve_np11.cu -- persistent solver kernels for order N = 10 (up to 8 problems).
 #include "solver.cuh"
 
-int sem_solve_launch_np11(const SolveParams<8> &p, int mode, int sms, long long mi, cudaStream_t s)
+int sem_solve_launch_np11(const SolveParams<8> &p, int mode, int sms, cudaStream_t s)
 {
     switch (mode) {
-        case MODE_F64: return launch_solve<8, MODE_F64, 11>(p, sms, mi, s);
-        case MODE_F64N: return launch_solve<8, MODE_F64N, 11>(p, sms, mi, s);
-        case MODE_F32: return launch_solve<8, MODE_F32, 11>(p, sms, mi, s);
+        case MODE_F64: return launch_solve<8, MODE_F64, 11>(p, sms, s);
+        case MODE_F64N: return launch_solve<8, MODE_F64N, 11>(p, sms, s);
+        case MODE_F32: return launch_solve<8, MODE_F32, 11>(p, sms, s);
         case MODE_TC: return SEM_ERR_ARG;
         default: return SEM_ERR_ARG;
     }
 }
+
+int sem_solve_tables_np11(const double *D) { return solver_upload_tables(11, D); }

@@ -1,13 +1,15 @@
 // solve_np13.cu -- persistent solver kernels for order N = 12 (up to 8 problems).
 #include "solver.cuh"
 
-int sem_solve_launch_np13(const SolveParams<8> &p, int mode, int sms, long long mi, cudaStream_t s)
+int sem_solve_launch_np13(const SolveParams<8> &p, int mode, int sms, cudaStream_t s)
 {
     switch (mode) {
-        case MODE_F64: return launch_solve<8, MODE_F64, 13>(p, sms, mi, s);
-        case MODE_F64N: return launch_solve<8, MODE_F64N, 13>(p, sms, mi, s);
-        case MODE_F32: return launch_solve<8, MODE_F32, 13>(p, sms, mi, s);
+        case MODE_F64: return launch_solve<8, MODE_F64, 13>(p, sms, s);
+        case MODE_F64N: return launch_solve<8, MODE_F64N, 13>(p, sms, s);
+        case MODE_F32: return launch_solve<8, MODE_F32, 13>(p, sms, s);
         case MODE_TC: return SEM_ERR_ARG;
         default: return SEM_ERR_ARG;
     }
 }
+
+int sem_solve_tables_np13(const double *D) { return solver_upload_tables(13, D); }

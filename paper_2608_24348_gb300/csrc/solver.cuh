@@ -3,28 +3,30 @@
 // One launch runs a whole solve (or a batch of independent solves).  Every
 // problem carries a small state machine; all problems advance together in
 // "grid steps".  In a step each problem executes the work items of its
-// current phase (element groups, chunks of unique nodes or chunks of local
-// nodes), every CTA adds its FP64 partial sums, and a reducing grid barrier
-// ends the step: the last CTA to arrive sums the partials of every problem in
-// a fixed order (deterministic), advances each state machine, publishes the
-// next schedule and releases the others.  Every wait is bounded in time; a
-// CTA that gives up raises SEM_ERR_TIMEOUT and the whole grid exits.
+// current phase (element groups, unique nodes or local nodes), every CTA
+// publishes its FP64 partial sums, and a grid barrier ends the step.  Behind
+// the barrier every CTA sums the published partials in the same fixed order
+// and advances its own copy of every state machine (in shared memory), so the
+// decision costs one exchange and is the same everywhere (deterministic).
+// Every wait is bounded in time; a CTA that gives up raises SEM_ERR_TIMEOUT
+// and the whole grid exits.
 //
 // Phases of one problem (Sec. 1.1: CG with Jacobi; Sec. 2: dot products and
 // norms reduced in fp64):
 //   JAC    local   minv = local diagonal of A
 //   JACGS  unique  minv = 1/dssum(minv);  sum b  (mean removal when h2 == 0)
 //   AX0    element w = A x                                      (FP64)
-//   R0     unique  r = b' - dssum(w); <r,r>, <r,z>, <b',b'>      (plain PCG)
-//   A      element x += alpha p (previous step); p = z + beta p; w = A p; <p,w>
-//   C      unique  r -= alpha dssum(w); <r,r>, <r,z>
-//   XUPD   local   x += alpha p (the last step, after convergence)
+//   R0     unique  r = b' - dssum(w); w <- z = minv r; <r,r>, <r,z>, <b',b'>
+//   A      element p = z + beta p; w <- A p; <p,w>
+//   C      unique  r -= alpha dssum(w); y += alpha p (x += alpha p in the first
+//                  X_DIRECT iterations); w <- z = minv r; <r,r>, <r,z>
+//   XUPD   unique  x += y                                       (after the last C)
 //   R64    unique  r = b' - dssum(w); <r,r>, <b',b'>            (refinement)
-//   INIT32 unique  r32 = r / ||r||; d = 0; <r32,r32>, <r32,z32>
-//   A32    element d += alpha p32; p32 = z32 + beta p32; w32 = A32 p32; <p32,w32>
-//   C32    unique  r32 -= alpha dssum(w32); <r32,r32>, <r32,z32>
-//   UPD    local   p = x (kept until the next FP64 residual accepts the step);
-//                  x += ||r|| (d + alpha p32 when that last step is pending)
+//   INIT32 unique  r32 = r / ||r||; d = 0; w32 <- z32; <r32,r32>, <r32,z32>
+//   A32    element p32 = z32 + beta p32; w32 <- A32 p32; <p32,w32>
+//   C32    unique  r32 -= alpha dssum(w32); d += alpha p32; w32 <- z32; <r32,r32>, <r32,z32>
+//   UPD    unique  p = x (kept until the next FP64 residual accepts the step);
+//                  x += ||r|| d
 //   XREST  local   x = p: a refinement step that raised the FP64 residual is
 //                  undone, so a solve never returns an iterate worse than the
 //                  one it had before that step
@@ -33,48 +35,47 @@
 // The inner product <a,b> = sum_local a b / mult is evaluated over unique
 // nodes, where it is a plain sum; <p, dssum(Ap)> equals sum_local p (Ap)
 // for a continuous p, which lets the element phase produce it directly.
-// Unique-node items are a chunk of 256 consecutive gx on SEM_UQ_ROWS rows
-// (gy, gz): the y/z copies are computed once per row, the x copies once per
-// thread, and all loads of a thread are issued before any store.
+//
+// Where each vector lives: z and A p share one E-vector (w): the unique phase
+// gathers every copy of A p and puts z in their place, the element phase reads
+// its element's z and puts A p there.  r, y (the sum of the corrections; d in
+// FP32) and the preconditioner are read and written at the first copy of every
+// unique node only.  So the element phase, whose arithmetic dominates, has two
+// input streams (z, p) instead of the four of a fused x and p update, and the
+// solution's update rides in the streaming phase: 144 bytes a node and
+// iteration in FP64.
+//
+// Element phases copy the next element's two input columns into shared memory
+// with asynchronous copies (cp.async; every thread copies and reads only its
+// own column, so no barrier guards them) while the current element is in
+// flight, and synchronise per element group (a named barrier over the group's
+// warps), so the groups of a CTA do not move in step.  Unique phases map one
+// thread to a few consecutive nodes of one element's row.  A CTA of the line
+// phases fills its multiprocessor (512 threads of 128 registers in FP64, 768 of
+// 80 in FP32), so a barrier has 152 arrivals and the redundant sums behind it
+// run once a multiprocessor.
 #pragma once
 
-#include <type_traits>
+#include <string.h>
 
 #include "ax.cuh"
 #include "ax_bfp.cuh"
 #include "ax_df.cuh"
-#include "ax_dfeo.cuh"
+#include "ax_dfl.cuh"
+#include "ax_line32.cuh"
 #include "ax_tc.cuh"
 #include "common.cuh"
-#include "gs.cuh"
 #include "tma.cuh"
+#include "uniq.cuh"
 
 #define SEM_MAXP 64
+// Threads of a CTA whose element phases are not line phases (see solve_threads).
 #define SEM_SOLVE_THREADS 256
-#define SEM_UQ_ROWS 4
-#ifndef SEM_SOLVE_F64_MINB
-#define SEM_SOLVE_F64_MINB 2
-#endif
-#ifndef SEM_SOLVE_F32_MINB
-#define SEM_SOLVE_F32_MINB 3
-#endif
-// Element phases prefetch their group's geometric factors into L2.
-#ifndef SEM_SOLVE_GEO_PREFETCH
-#define SEM_SOLVE_GEO_PREFETCH 1
-#endif
-// FP64-accurate element phases of even orders use the folded operator.
-#ifndef SEM_SOLVE_DF_FOLDED
-#define SEM_SOLVE_DF_FOLDED 1
-#endif
-// ... and, for even N+1 <= 12, the block-floating-point operator.
-#ifndef SEM_SOLVE_BFP
-#define SEM_SOLVE_BFP 1
-#endif
 
 // Which element operators a solver kernel carries (keeps each kernel's
 // register budget to what its mode needs).
-// MODE_F64 evaluates the FP64 operator on the FP32 pipes (float pairs,
-// ax_df.cuh); MODE_F64N uses native FP64 arithmetic.
+// MODE_F64 evaluates the FP64 operator on the FP32 pipes (block-floating-point
+// or float pairs); MODE_F64N uses native FP64 arithmetic.
 enum SolveMode { MODE_F64 = 0, MODE_F32 = 1, MODE_TC = 2, MODE_F64N = 3 };
 
 enum SolvePhase {
@@ -87,8 +88,11 @@ struct ProbDesc {
     int tc;                     // inner path of a MODE_TC launch: 0 FP32 CUDA cores, 1 BF16, 2 FP16,
                                 // 3 FP16 x2, 4 BF16 x3 tensor cores
     int jac_cached;             // minv (and minv32 if mixed) already hold this problem's Jacobi inverse
+    int vec;                    // b and x are aligned for vector accesses
+    int jac_shared;             // an earlier problem of the launch makes the Jacobi inverse in minv
     int64_t E, nL, nG;
-    GsDesc gs;
+    UqMesh mesh;
+    FastDiv dn3;
     double volume, h1, h2;
     const double *geo64;
     const float *geo32;
@@ -96,15 +100,15 @@ struct ProbDesc {
     const double *D64;
     const float *D32;
     const dfp *Ddf;
-    const dfp *Ddfeo;   // folded half tables (even orders)
     const double *b;
     double *x;
     double *r, *p, *w, *minv;
+    double *y;          // the sum of the corrections; null: x is updated in every iteration instead
     float *r32, *p32, *w32, *d32, *minv32;
 };
 
 struct PState {
-    int phase, iters, outer, inner_iters, status, first, nvals, pending;
+    int phase, iters, outer, inner_iters, status, first;
     double rz, alpha, beta, bnorm, rnorm, target, bmean, scale, prev_rnorm, inner_target, shift;
 };
 
@@ -120,8 +124,9 @@ struct SolveParams {
     long long timeout_ns;
     SyncState *sync;
     PState *st;
-    double *partials;   // [gridDim][MAXP][3]
-    int *sched;         // phase[MAXP], then offsets[MAXP + 1]
+    double *partials;       // two buffers of [MAXP * 3][gridDim]
+    long long partials_cap; // doubles that fit
+    unsigned char order[MAXP]; // the problems by polynomial order
     ProbDesc prob[MAXP];
 };
 
@@ -143,7 +148,18 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p)
     return v;
 }
 
-__device__ __forceinline__ int phase_nvals(int ph)
+__device__ __forceinline__ void red_release_add_u32(unsigned *p, unsigned v)
+{
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// Phases whose sums are gathered in float pairs.
+__device__ __forceinline__ bool phase_pairs(int ph)
+{
+    return ph == PH_A32 || ph == PH_C32 || ph == PH_INIT32;
+}
+
+__host__ __device__ __forceinline__ int phase_nvals(int ph)
 {
     switch (ph) {
         case PH_JACGS: return 1;
@@ -152,25 +168,6 @@ __device__ __forceinline__ int phase_nvals(int ph)
         case PH_C: case PH_C32: case PH_R64: case PH_INIT32: return 2;
         case PH_FINAL: return 1;
         default: return 0;
-    }
-}
-
-__device__ __forceinline__ int64_t phase_items(const ProbDesc &P, int ph)
-{
-    switch (ph) {
-        case PH_JAC: case PH_UPD: case PH_FINAL: case PH_SHIFT: case PH_XUPD: case PH_XREST:
-            return (P.nL + SEM_SOLVE_THREADS - 1) / SEM_SOLVE_THREADS;
-        case PH_JACGS: case PH_R0: case PH_C: case PH_R64: case PH_INIT32: case PH_C32: {
-            const int64_t nxch = (P.gs.ngx + SEM_SOLVE_THREADS - 1) / SEM_SOLVE_THREADS;
-            const int64_t rows = (int64_t)P.gs.ngy * P.gs.ngz;
-            return nxch * ((rows + SEM_UQ_ROWS - 1) / SEM_UQ_ROWS);
-        }
-        case PH_AX0: case PH_A:
-            return (P.E + P.NE - 1) / P.NE;
-        case PH_A32:
-            return (P.E + P.NE32 - 1) / P.NE32;
-        default:
-            return 0;
     }
 }
 
@@ -200,120 +197,364 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// Adds the block sum of v[0..2] into dst[0..2] (thread 0); all threads call.
-__device__ __forceinline__ void block_accumulate(double v[3], double *s_red, double *dst)
+// The sum of a warp's float pairs (two-sums, the errors gathered as in dot2_acc).
+__device__ __forceinline__ dfacc warp_sum_pair(dfacc A)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        double s = warp_sum(v[k]);
-        if (lane == 0) s_red[warp * 3 + k] = s;
-        v[k] = 0.0;
+    for (int o = 16; o > 0; o >>= 1) {
+        const float b = __shfl_xor_sync(0xffffffffu, A.s, o), be = __shfl_xor_sync(0xffffffffu, A.e, o);
+        const float s = __fadd_rn(A.s, b), bv = __fsub_rn(s, A.s);
+        const float t = __fadd_rn(__fsub_rn(A.s, __fsub_rn(s, bv)), __fsub_rn(b, bv));
+        A.s = s;
+        A.e = __fadd_rn(__fadd_rn(A.e, be), t);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < 3; ++k) {
-            double s = 0.0;
-            for (int w = 0; w < SEM_SOLVE_THREADS / 32; ++w) s += s_red[w * 3 + k];
-            dst[k] += s;
-        }
-    }
-    __syncthreads();
+    return A;
 }
 
-// Thread 0 asks L2 for the geometric factors of the element group this block
-// is about to work on (bytes [e0, e1) elements of a [E][7][NP^3] array of
-// `wb`-byte words): the operator reads them after its gradient stage, about
+// The sum of a thread's values by halves: the additions of one level are
+// independent, and FP64 additions are slow to return on this part.
+template <int N>
+__device__ __forceinline__ double tree_sum(double (&t)[N])
+{
+#pragma unroll
+    for (int m = N; m > 1; m = (m + 1) / 2)
+#pragma unroll
+        for (int j = 0; j < m / 2; ++j) t[j] += t[j + (m + 1) / 2];
+    return t[0];
+}
+
+// A lane's L2 prefetch of the geometric factors of the element group it is
+// about to work on (elements [e0, e0 + ne) of a [E][7][NP^3] array of
+// wb-byte words): the operator reads them after its gradient stage, about
 // half an element phase later.  (A whole group ahead let L2 evict the element
 // phase's output before the gather read it.)
 template <int NP>
 __device__ __forceinline__ void geo_prefetch(const void *geo, int64_t e0, int ne, int64_t E, int wb)
 {
     constexpr int64_t N3 = NP * NP * NP;
-    if (!SEM_SOLVE_GEO_PREFETCH || threadIdx.x != 0 || e0 >= E) return;
+    if (e0 >= E) return;
     const int64_t e1 = e0 + ne < E ? e0 + ne : E;
     l2_prefetch_span(geo, e0 * 7 * N3 * wb, e1 * 7 * N3 * wb);
 }
 
 // ---------------------------------------------------------------------------
-// element items
+// element phases
 // ---------------------------------------------------------------------------
 
-// kind 0: w64 = A64 x;  kind 1: FP64 p-update + w = A p + <p,w>;
-// kind 2: FP32 p32-update + w32 = A32 p32 + <p32,w32>.
-template <int NP, int KIND>
-__device__ __forceinline__ void elem_item(const ProbDesc &P, double alpha, double beta, int first,
-                                          int64_t g, unsigned char *smem, double &acc)
+// Element groups of the staged phases: GE elements on GT threads (whole
+// warps), the smallest GT that keeps about 80 % of its lanes busy.
+__host__ __device__ constexpr int grp_threads(int np)
 {
-    using C = AxCfg<NP>;
-    using T = typename std::conditional<KIND == 2, float, double>::type;
-    T *sm = reinterpret_cast<T *>(smem);
-    T *sD = sm, *sDT = sm + NP * NP;
-    const int grp = threadIdx.x / C::NP2;
-    const int tid = threadIdx.x - grp * C::NP2;
-    const bool inrange = grp < C::NE;
-    const int64_t e = g * C::NE + grp;
-    const bool active = inrange && e < P.E;
-    T *su = sm + 2 * NP * NP + (size_t)(inrange ? grp : 0) * 3 * C::NP3;
-    T *svr = su + C::NP3, *svs = svr + C::NP3;
-    const int64_t off = (active ? e : 0) * C::NP3;
-    const T *D = KIND == 2 ? (const T *)P.D32 : (const T *)P.D64;
-    const T *geo = (KIND == 2 ? (const T *)P.geo32 : (const T *)P.geo64) + (active ? e : 0) * 7 * C::NP3;
-    if (KIND == 2) geo_prefetch<NP>(P.geo32, g * C::NE, C::NE, P.E, 4);  // (native FP64: no gain)
-    ax_load_D<NP, T>(D, sD, sDT);
-    if (KIND == 0) {
-        const double *x = P.x + off;
-        double *w = P.w + off;
-        auto load = [&](int q) { return (T)__ldcg(x + q); };
-        auto store = [&](int q, T v, T) { w[q] = v; };
-        ax_element<NP, T>(load, store, geo, (T)P.h1, (T)P.h2, sD, sDT, su, svr, svs, tid, active);
-    } else if (KIND == 1) {
-        const double *r = P.r + off, *mi = P.minv + off;
-        double *p = P.p + off, *w = P.w + off, *x = P.x + off;
-        auto load = [&](int q) {
-            double pn = __ldcg(mi + q) * __ldcg(r + q);
-            if (!first) {
-                const double po = __ldcg(p + q);
-                x[q] = fma(alpha, po, __ldcg(x + q));
-                pn = fma(beta, po, pn);
-            }
-            p[q] = pn;
-            return (T)pn;
+    return np <= 4 ? 32 : np == 8 ? 64 : (np == 5 || np == 6 || np == 10 || np == 11) ? 128 : 256;
+}
+__host__ __device__ constexpr int grp_elems(int np) { return grp_threads(np) / (np * np); }
+
+template <int NP, int TH>
+struct GrpCfg {
+    static constexpr int GT = grp_threads(NP), GE = grp_elems(NP);
+    static constexpr int NG = TH / GT;  // groups per CTA
+    static constexpr int NE = NG * GE;  // elements per CTA
+};
+
+// Barrier over one element group of a CTA of TH threads.
+template <int GT, int TH>
+struct GrpSync {
+    int grp;
+    __device__ __forceinline__ void operator()() const
+    {
+        if constexpr (GT == TH)
+            __syncthreads();
+        else if constexpr (GT == 32)
+            __syncwarp();
+        else
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(GT) : "memory");
+    }
+};
+
+// The calling thread's place in its element group.
+template <int NP>
+struct GrpThread {
+    int grp, ge, tid;  // tid: column owner 0 .. NP^2 - 1, or -1 (takes part in the barriers only)
+    __device__ __forceinline__ GrpThread()
+    {
+        constexpr int GT = grp_threads(NP), GE = grp_elems(NP);
+        grp = threadIdx.x / GT;
+        const int lt = threadIdx.x - grp * GT;
+        ge = lt / (NP * NP);
+        tid = ge < GE ? lt - ge * NP * NP : -1;
+        if (tid < 0) ge = 0;
+    }
+};
+
+// One problem's place in a step: its portions are dealt to slots, a slot being
+// one group of warps, slot k on CTA k % ncta: a problem smaller than the
+// machine spreads over the multiprocessors before it fills any of them, and the
+// last round of a larger one leaves every multiprocessor about as many busy
+// groups.  The next problem of the step goes on where the last one ended: rot
+// counts slots of one warp.
+struct Deal {
+    unsigned cta, ncta, rot;
+    // the first portion of group grp of a CTA that has ng groups of wpg warps;
+    // the group's next ones follow ncta * ng apart
+    __device__ __forceinline__ unsigned first(unsigned grp, unsigned wpg, unsigned ng) const
+    {
+        const unsigned n = ncta * ng;
+        unsigned s = grp * ncta + cta;
+        if (rot) s += n - (rot % ncta + ncta * (rot / ncta / wpg)) % n;
+        return s < n ? s : s - n;
+    }
+    // the next problem's start after this one dealt out `portions`
+    __device__ __forceinline__ unsigned after(unsigned portions, unsigned wpg, unsigned ng, unsigned nw) const
+    {
+        const unsigned n = ncta * ng;
+        const unsigned s = (rot % ncta + ncta * (rot / ncta / wpg) + portions) % n;
+        return (s % ncta + (s / ncta) * wpg * ncta) % (ncta * nw);
+    }
+};
+
+// FP64-accurate phases stage two columns (z, p) per thread and keep the new p
+// for the inner product in a third where the shared memory allows it.
+template <int NP>
+constexpr bool stage_keep_p()
+{
+    return NP <= 8;
+}
+
+template <int NP, int TH>
+__host__ __device__ constexpr size_t stage64_bytes()
+{
+    return sizeof(double) * (stage_keep_p<NP>() ? 3 : 2) * NP * TH;
+}
+
+template <int NP, int TH>
+__host__ __device__ constexpr size_t elem32_smem_bytes()
+{
+    return sizeof(float) * ((size_t)GrpCfg<NP, TH>::NE * 3 * Line32Cfg<NP>::SLAB + 2 * NP * TH);
+}
+
+// Shared memory of one low-register element, a multiple of 16 bytes.
+template <int NP>
+__host__ __device__ constexpr size_t lowreg_smem_bytes()
+{
+    return (ax_df_lowreg_smem_bytes<NP>() + 15) / 16 * 16;
+}
+
+// Tables of the line operators, one copy per translation unit and order
+// (constant-bank operands in the unrolled contractions): the FP32 operator's, and
+// the FP64-accurate one's for the order's parity.  Filled at context setup,
+// outside any stream capture, by solver_upload_tables.
+struct SolveTabs {
+    LineTab32 l;
+    union {
+        BfpTabs bfp;
+        DflTabs dfl;
+    };
+};
+static __constant__ SolveTabs c_tabs[SEM_NPMAX + 1];
+
+// A32: p32 = z32 + beta p32, w32 <- A32 p32, <p32, w32>, by whole lines.
+template <int NP, int TH>
+__device__ __forceinline__ void phase_a32(const ProbDesc &P, double beta, int first, const Deal &deal,
+                                          unsigned char *smem, dfacc &dot)
+{
+    using G = GrpCfg<NP, TH>;
+    constexpr int NP2 = NP * NP, NP3 = NP2 * NP;
+    const GrpThread<NP> th;
+    const GrpSync<G::GT, TH> sync{th.grp};
+    float *slabs = reinterpret_cast<float *>(smem);
+    float *slab = slabs + (size_t)(th.grp * G::GE + th.ge) * 3 * Line32Cfg<NP>::SLAB;
+    float *sz = slabs + (size_t)G::NE * 3 * Line32Cfg<NP>::SLAB + threadIdx.x;
+    float *sp = sz + NP * TH;
+    const float b32 = (float)beta, h1 = (float)P.h1, h2 = (float)P.h2;
+    const int E = (int)P.E, ngr = (E + G::GE - 1) / G::GE;
+    auto fetch = [&](int g) {
+        const int e = g * G::GE + th.ge;
+        if (g < ngr && th.tid >= 0 && e < E) {
+            const size_t off = (size_t)e * NP3 + th.tid;
+#pragma unroll
+            for (int k = 0; k < NP; ++k) cp_async4(sz + k * TH, P.w32 + off + k * NP2);
+            if (!first)
+#pragma unroll
+                for (int k = 0; k < NP; ++k) cp_async4(sp + k * TH, P.p32 + off + k * NP2);
+        }
+    };
+    const int stride = (int)deal.ncta * G::NG;
+    int g = th.grp < G::NG ? (int)deal.first(th.grp, G::GT / 32, G::NG) : ngr;
+    fetch(g);
+    for (; g < ngr; g += stride) {
+        const int e = g * G::GE + th.ge;
+        const bool active = th.tid >= 0 && e < E;
+        if (threadIdx.x % G::GT == 0) geo_prefetch<NP>(P.geo32, (int64_t)g * G::GE, G::GE, E, 4);
+        const size_t off = (size_t)(active ? e : 0) * NP3 + th.tid;
+        cp_async_wait_all();
+        auto load = [&](int k) {
+            float pn = sz[k * TH];
+            if (!first) pn = fmaf(b32, sp[k * TH], pn);
+            P.p32[off + k * NP2] = pn;
+            return pn;
         };
-        auto store = [&](int q, T v, T u) {
-            w[q] = v;
-            acc = fma((double)u, (double)v, acc);
-        };
-        ax_element<NP, T>(load, store, geo, (T)P.h1, (T)P.h2, sD, sDT, su, svr, svs, tid, active);
-    } else {
-        const float *r = P.r32 + off, *mi = P.minv32 + off;
-        float *p = P.p32 + off, *w = P.w32 + off, *d = P.d32 + off;
-        const float b32 = (float)beta, a32 = (float)alpha;
-        auto load = [&](int q) {
-            float pn = __ldcg(mi + q) * __ldcg(r + q);
-            if (!first) {
-                const float po = __ldcg(p + q);
-                d[q] = fmaf(a32, po, __ldcg(d + q));
-                pn = fmaf(b32, po, pn);
-            }
-            p[q] = pn;
-            return (T)pn;
-        };
-        dfacc dot = {0.f, 0.f};
-        auto store = [&](int q, T v, T u) {
-            w[q] = v;
+        auto store = [&](int k, float v, float u) {
+            P.w32[off + k * NP2] = v;
             dot2_acc(dot, u, v);
         };
-        ax_element<NP, T>(load, store, geo, (T)P.h1, (T)P.h2, sD, sDT, su, svr, svs, tid, active);
-        acc += dfacc_value(dot);
+        ax_line32_element<NP>(load, store, P.geo32 + (size_t)(active ? e : 0) * 7 * NP3, h1, h2,
+                              c_tabs[NP].l, slab, th.tid, active, [&] { fetch(g + stride); }, sync);
     }
 }
 
-// FP64-accurate element phases on the FP32 pipes (float pairs):
-// kind 0: w = A x;  kind 1: x += alpha p, p = z + beta p, w = A p, <p,w>.
-template <int NP, int KIND>
-__device__ __forceinline__ void elem_item_df(const ProbDesc &P, double alpha, double beta, int first,
-                                             int64_t g, unsigned char *smem, double &acc)
+// D: the FP64 derivative matrix, np x np row-major (host).
+static inline int solver_upload_tables(int np, const double *D)
+{
+    if (np < 2 || np > SEM_NPMAX || !D) return SEM_ERR_ARG;
+    SolveTabs T;
+    memset(&T, 0, sizeof(T));
+    for (int t = 0; t < np * np; ++t) T.l.d[t] = (float)D[t];
+    if (np % 2 == 0) ax_bfp_tables(np, D, &T.bfp);
+    else if (np <= 11) ax_dfl_tables(np, D, &T.dfl);
+    SEM_CUDA(cudaMemcpyToSymbol(c_tabs, &T, sizeof(T), (size_t)np * sizeof(T)));
+    return SEM_OK;
+}
+
+// Dynamic shared memory of an FP64-accurate line phase: eight reduction words
+// an element (the first zeroed at the start of every phase), the slabs, the
+// staged columns.
+template <int NP, int TH>
+constexpr size_t line64_red_bytes()
+{
+    return 8 * sizeof(unsigned) * GrpCfg<NP, TH>::NE;
+}
+
+template <int NP>
+constexpr bool solve_bfp()
+{
+    return BfpCfg<NP>::OK && NP <= 12;
+}
+template <int NP>
+constexpr bool solve_dfl()
+{
+    return DflCfg<NP>::OK;
+}
+template <int NP>
+constexpr size_t line64_slab_pairs()
+{
+    return 3 * (size_t)(solve_bfp<NP>() ? BfpCfg<NP>::SLAB : NP * NP * NP);
+}
+template <int NP, int TH>
+constexpr size_t line64_smem_bytes()
+{
+    return line64_red_bytes<NP, TH>() + sizeof(dfp) * GrpCfg<NP, TH>::NE * line64_slab_pairs<NP>() + stage64_bytes<NP, TH>();
+}
+
+// FP64-accurate element phases on the FP32 pipes by whole lines
+// (block-floating-point pairs for even N+1 <= 12, float pairs for odd N+1 <=
+// 11).  AX0: w = A x;  A: p = z + beta p, w <- A p, <p, w>.
+template <int NP, int TH>
+__device__ __forceinline__ void phase_a64(const ProbDesc &P, bool ax0, double beta, int first, const Deal &deal,
+                                          unsigned char *smem, double &acc)
+{
+    using G = GrpCfg<NP, TH>;
+    constexpr int NP2 = NP * NP, NP3 = NP2 * NP;
+    const GrpThread<NP> th;
+    const GrpSync<G::GT, TH> sync{th.grp};
+    const int slot = th.grp * G::GE + th.ge;
+    unsigned *red = reinterpret_cast<unsigned *>(smem) + 8 * slot;
+    dfp *slabs = reinterpret_cast<dfp *>(smem + line64_red_bytes<NP, TH>());
+    dfp *slab = slabs + (size_t)slot * line64_slab_pairs<NP>();
+    double *sz = reinterpret_cast<double *>(slabs + G::NE * line64_slab_pairs<NP>()) + threadIdx.x;
+    double *sp = sz + NP * TH;
+    double *sn = sp + NP * TH;  // the new p (stage_keep_p)
+    const float h1h = (float)P.h1, h2h = (float)P.h2;
+    const dfp H1 = {h1h, (float)(P.h1 - (double)h1h)}, H2 = {h2h, (float)(P.h2 - (double)h2h)};
+    const int E = (int)P.E, ngr = (E + G::GE - 1) / G::GE;
+    const double *zsrc = ax0 ? P.x : P.w;
+    const bool add_p = !ax0 && !first;
+    auto fetch = [&](int g) {
+        const int e = g * G::GE + th.ge;
+        if (g < ngr && th.tid >= 0 && e < E) {
+            const size_t off = (size_t)e * NP3 + th.tid;
+#pragma unroll
+            for (int k = 0; k < NP; ++k) cp_async8(sz + k * TH, zsrc + off + k * NP2);
+            if (add_p)
+#pragma unroll
+                for (int k = 0; k < NP; ++k) cp_async8(sp + k * TH, P.p + off + k * NP2);
+        }
+    };
+    if (th.tid == 0 && th.grp < G::NG) *red = 0u;
+    if (th.grp < G::NG) sync();
+    const int stride = (int)deal.ncta * G::NG;
+    int g = th.grp < G::NG ? (int)deal.first(th.grp, G::GT / 32, G::NG) : ngr;
+    fetch(g);
+    for (; g < ngr; g += stride) {
+        const int e = g * G::GE + th.ge;
+        const bool active = th.tid >= 0 && e < E;
+        if (threadIdx.x % G::GT == 0) geo_prefetch<NP>(P.geodf, (int64_t)g * G::GE, G::GE, E, 8);
+        const size_t off = (size_t)(active ? e : 0) * NP3;
+        const dfp *geo = P.geodf + (size_t)(active ? e : 0) * 7 * NP3;
+        cp_async_wait_all();
+        auto load = [&](int q) {
+            const int k = (q - th.tid) / NP2;  // a constant after unrolling
+            double pn = sz[k * TH];
+            if (ax0) return pn;
+            if (add_p) pn = fma(beta, sp[k * TH], pn);
+            if (stage_keep_p<NP>()) sn[k * TH] = pn;
+            P.p[off + q] = pn;
+            return pn;
+        };
+        auto store = [&](int q, double v) {
+            P.w[off + q] = v;
+            if (!ax0) {
+                const int k = (q - th.tid) / NP2;
+                acc = fma(stage_keep_p<NP>() ? sn[k * TH] : __ldcg(P.p + off + q), v, acc);
+            }
+        };
+        auto next = [&] { fetch(g + stride); };
+        if constexpr (solve_bfp<NP>())
+            ax_bfp_element<NP, false>(load, store, geo, H1, H2, c_tabs[NP].bfp, slab, red, th.tid, active,
+                                      next, sync);
+        else
+            ax_dfl_element<NP>(load, store, geo, H1, H2, c_tabs[NP].dfl, slab, red, th.tid, active, next,
+                               sync);
+    }
+}
+
+// FP64-accurate w = A x with the low-register float-pair operator (mixed
+// modes: the FP64 residual of each refinement step), one element per 256
+// threads of the CTA.
+template <int NP, int TH>
+__device__ __forceinline__ void phase_ax0_lowreg(const ProbDesc &P, const Deal &deal, unsigned char *smem)
+{
+    constexpr int NP3 = NP * NP * NP, NG = TH / SEM_SOLVE_THREADS;
+    const float h1h = (float)P.h1, h2h = (float)P.h2;
+    const dfp H1 = {h1h, (float)(P.h1 - (double)h1h)}, H2 = {h2h, (float)(P.h2 - (double)h2h)};
+    const int grp = threadIdx.x / SEM_SOLVE_THREADS;
+    const GrpSync<SEM_SOLVE_THREADS, TH> sync{grp};
+    smem += grp * lowreg_smem_bytes<NP>();
+    for (int64_t e = deal.first(grp, SEM_SOLVE_THREADS / 32, NG); e < P.E; e += deal.ncta * NG) {
+        const double *x = P.x + e * NP3;
+        double *w = P.w + e * NP3;
+        auto load = [&](int q) { return __ldcg(x + q); };
+        auto store = [&](int q, double v) { w[q] = v; };
+        ax_df_element_lowreg<NP>(load, store, P.geodf + e * 7 * NP3, H1, H2, P.Ddf, smem,
+                                 threadIdx.x % SEM_SOLVE_THREADS, SEM_SOLVE_THREADS, sync);
+    }
+}
+
+// Loads of a phase without staging: the input of node q (z + beta p, kept as
+// the new p, in phase A; x in AX0).
+__device__ __forceinline__ double a_input(const ProbDesc &P, bool ax0, double beta, int first, size_t q)
+{
+    if (ax0) return __ldcg(P.x + q);
+    double pn = __ldcg(P.w + q);
+    if (!first) pn = fma(beta, __ldcg(P.p + q), pn);
+    P.p[q] = pn;
+    return pn;
+}
+
+// FP64-accurate element phases of the largest orders (float pairs, D in shared
+// memory), one group of 256/NP^2 elements per CTA.
+template <int NP>
+__device__ __forceinline__ void elem_item_df(const ProbDesc &P, bool ax0, double beta, int first, int64_t g,
+                                             unsigned char *smem, double &acc)
 {
     using C = AxDfCfg<NP>;
     dfp *sm = reinterpret_cast<dfp *>(smem);
@@ -326,213 +567,60 @@ __device__ __forceinline__ void elem_item_df(const ProbDesc &P, double alpha, do
     const bool active = inrange && e < P.E;
     dfp *su = sm + 2 * NP * NP + (size_t)(inrange ? grp : 0) * 3 * C::NP3;
     dfp *svr = su + C::NP3, *svs = svr + C::NP3;
-    const int64_t off = (active ? e : 0) * C::NP3;
+    const size_t off = (size_t)(active ? e : 0) * C::NP3;
     const dfp *geo = P.geodf + (active ? e : 0) * 7 * C::NP3;
     const float h1h = (float)P.h1, h2h = (float)P.h2;
     const dfp H1 = {h1h, (float)(P.h1 - (double)h1h)}, H2 = {h2h, (float)(P.h2 - (double)h2h)};
-    geo_prefetch<NP>(P.geodf, g * C::NE, C::NE, P.E, 8);
+    if (threadIdx.x == 0) geo_prefetch<NP>(P.geodf, g * C::NE, C::NE, P.E, 8);
     ax_df_load_D<NP>(P.Ddf, sD, sDT);
     int *myexp = sexp + (inrange ? grp : 0);
-    if (KIND == 0) {
-        const double *x = P.x + off;
-        double *w = P.w + off;
-        auto load = [&](int q) { return __ldcg(x + q); };
-        auto store = [&](int q, double v) { w[q] = v; };
-        ax_df_element<NP>(load, store, geo, H1, H2, sD, sDT, su, svr, svs, myexp, tid, active);
-    } else {
-        const double *r = P.r + off, *mi = P.minv + off;
-        double *p = P.p + off, *w = P.w + off, *x = P.x + off;
-        auto load = [&](int q) {
-            double pn = __ldcg(mi + q) * __ldcg(r + q);
-            if (!first) {
-                const double po = __ldcg(p + q);
-                x[q] = fma(alpha, po, __ldcg(x + q));
-                pn = fma(beta, po, pn);
-            }
-            p[q] = pn;
-            return pn;
-        };
-        auto store = [&](int q, double v) {
-            w[q] = v;
-            acc = fma(__ldcg(p + q), v, acc);
-        };
-        ax_df_element<NP>(load, store, geo, H1, H2, sD, sDT, su, svr, svs, myexp, tid, active);
-    }
+    auto load = [&](int q) { return a_input(P, ax0, beta, first, off + q); };
+    auto store = [&](int q, double v) {
+        P.w[off + q] = v;
+        if (!ax0) acc = fma(__ldcg(P.p + off + q), v, acc);
+    };
+    ax_df_element<NP>(load, store, geo, H1, H2, sD, sDT, su, svr, svs, myexp, tid, active);
 }
 
-// The same phases with the folded (even-odd) float-pair operator, even orders.
+// Native FP64 element phases.
 template <int NP>
-constexpr bool df_folded()
+__device__ __forceinline__ void elem_item_native(const ProbDesc &P, bool ax0, double beta, int first,
+                                                 int64_t g, unsigned char *smem, double &acc)
 {
-    // (and only while two blocks still fit on an SM)
-    return SEM_SOLVE_DF_FOLDED && AxEoCfg<NP>::OK && AxEoCfg<NP>::THREADS <= SEM_SOLVE_THREADS &&
-           ax_dfeo_smem_bytes<NP>() <= 112 * 1024;
-}
-
-template <int NP, int KIND>
-__device__ __forceinline__ void elem_item_dfeo(const ProbDesc &P, double alpha, double beta, int first,
-                                               int64_t g, unsigned char *smem, double &acc)
-{
-    using C = AxEoCfg<NP>;
-    constexpr int HH = (NP / 2) * (NP / 2);
-    dfp *sm = reinterpret_cast<dfp *>(smem);
-    dfp *stab = sm;
-    int *sexp = reinterpret_cast<int *>(sm + 4 * HH + (size_t)C::NE * 5 * C::SLAB);
+    using C = AxCfg<NP>;
+    double *sm = reinterpret_cast<double *>(smem);
+    double *sD = sm, *sDT = sm + NP * NP;
     const int grp = threadIdx.x / C::NP2;
     const int tid = threadIdx.x - grp * C::NP2;
     const bool inrange = grp < C::NE;
     const int64_t e = g * C::NE + grp;
     const bool active = inrange && e < P.E;
-    dfp *slab = sm + 4 * HH + (size_t)(inrange ? grp : 0) * 5 * C::SLAB;
-    const int64_t off = (active ? e : 0) * C::NP3;
-    const dfp *geo = P.geodf + (active ? e : 0) * 7 * C::NP3;
-    const float h1h = (float)P.h1, h2h = (float)P.h2;
-    const dfp H1 = {h1h, (float)(P.h1 - (double)h1h)}, H2 = {h2h, (float)(P.h2 - (double)h2h)};
-    geo_prefetch<NP>(P.geodf, g * C::NE, C::NE, P.E, 8);
-    for (int t = threadIdx.x; t < 4 * HH; t += blockDim.x) stab[t] = P.Ddfeo[t];
-    int *myexp = sexp + (inrange ? grp : 0);
-    if (KIND == 0) {
-        const double *x = P.x + off;
-        double *w = P.w + off;
-        auto load = [&](int q) { return __ldcg(x + q); };
-        auto store = [&](int q, double v) { w[q] = v; };
-        ax_dfeo_element<NP>(load, store, geo, H1, H2, stab, slab, myexp, tid, active);
-    } else {
-        const double *r = P.r + off, *mi = P.minv + off;
-        double *p = P.p + off, *w = P.w + off, *x = P.x + off;
-        auto load = [&](int q) {
-            double pn = __ldcg(mi + q) * __ldcg(r + q);
-            if (!first) {
-                const double po = __ldcg(p + q);
-                x[q] = fma(alpha, po, __ldcg(x + q));
-                pn = fma(beta, po, pn);
-            }
-            p[q] = pn;
-            return pn;
-        };
-        auto store = [&](int q, double v) {
-            w[q] = v;
-            acc = fma(__ldcg(p + q), v, acc);
-        };
-        ax_dfeo_element<NP>(load, store, geo, H1, H2, stab, slab, myexp, tid, active);
-    }
-}
-
-// The block-floating-point operator's tables for each even order, one copy
-// per translation unit (constant-bank operands in the unrolled contractions);
-// filled at context setup, outside any stream capture, by
-// solver_upload_bfp_tables.
-static __constant__ BfpTabs c_bfp_tabs[SEM_NPMAX / 2 + 1];
-
-static inline int solver_upload_bfp_tables(int np, const void *tabs)
-{
-    if (np < 2 || np > SEM_NPMAX || np % 2 || !tabs) return SEM_ERR_ARG;
-    SEM_CUDA(cudaMemcpyToSymbol(c_bfp_tabs, tabs, sizeof(BfpTabs), (size_t)(np / 2) * sizeof(BfpTabs)));
-    return SEM_OK;
-}
-
-// Dynamic shared memory of a block-floating-point element phase: 2 KB of
-// reduction words (zeroed at kernel start; each element leaves them zero),
-// then the slabs.
-#define SEM_BFP_RED_BYTES 2048
-
-template <int NP>
-constexpr bool solve_bfp()
-{
-    return SEM_SOLVE_BFP && BfpCfg<NP>::OK && NP <= 12 && BfpCfg<NP>::THREADS <= SEM_SOLVE_THREADS &&
-           ax_bfp_smem_bytes_ne<NP, BfpCfg<NP>::NE>() + SEM_BFP_RED_BYTES <= 112 * 1024;
-}
-
-
-// FP64-accurate element phases with the block-floating-point operator:
-// kind 0: w = A x;  kind 1: x += alpha p, p = z + beta p, w = A p, <p,w>.
-template <int NP, int KIND>
-__device__ __forceinline__ void elem_item_bfp(const ProbDesc &P, double alpha, double beta, int first,
-                                              int64_t g, unsigned char *smem, double &acc)
-{
-    using C = BfpCfg<NP>;
-    static_assert(8 * C::NE * sizeof(unsigned) <= SEM_BFP_RED_BYTES, "reduction words");
-    unsigned *red = reinterpret_cast<unsigned *>(smem);
-    dfp *slabs = reinterpret_cast<dfp *>(smem + SEM_BFP_RED_BYTES);
-    const int grp = threadIdx.x / C::NP2;
-    const bool inrange = grp < C::NE;
-    // threads beyond the last whole element take part in the barriers only
-    const int tid = inrange ? (int)threadIdx.x - grp * C::NP2 : -1;
-    const int gs = inrange ? grp : 0;
-    const int64_t e = g * C::NE + grp;
-    const bool active = inrange && e < P.E;
-    const int64_t off = (active ? e : 0) * C::NP3;
-    const dfp *geo = P.geodf + (active ? e : 0) * 7 * C::NP3;
-    const float h1h = (float)P.h1, h2h = (float)P.h2;
-    const dfp H1 = {h1h, (float)(P.h1 - (double)h1h)}, H2 = {h2h, (float)(P.h2 - (double)h2h)};
-    geo_prefetch<NP>(P.geodf, g * C::NE, C::NE, P.E, 8);
-    const BfpTabs &T = c_bfp_tabs[NP / 2];
-    dfp *slab = slabs + (size_t)gs * 3 * C::SLAB;
-    if (KIND == 0) {
-        const double *x = P.x + off;
-        double *w = P.w + off;
-        auto load = [&](int q) { return __ldcg(x + q); };
-        auto store = [&](int q, double v) { w[q] = v; };
-        ax_bfp_element<NP, false>(load, store, geo, H1, H2, T, slab, red + gs * 8, tid, active, [] {});
-    } else {
-        const double *r = P.r + off, *mi = P.minv + off;
-        double *p = P.p + off, *w = P.w + off, *x = P.x + off;
-        auto load = [&](int q) {
-            double pn = __ldcg(mi + q) * __ldcg(r + q);
-            if (!first) {
-                const double po = __ldcg(p + q);
-                x[q] = fma(alpha, po, __ldcg(x + q));
-                pn = fma(beta, po, pn);
-            }
-            p[q] = pn;
-            return pn;
-        };
-        auto store = [&](int q, double v) {
-            w[q] = v;
-            acc = fma(__ldcg(p + q), v, acc);
-        };
-        ax_bfp_element<NP, false>(load, store, geo, H1, H2, T, slab, red + gs * 8, tid, active, [] {});
-    }
-}
-
-// FP64-accurate w = A x with the low-register float-pair operator (mixed
-// modes: the FP64 residual of each refinement step); the NE elements of
-// group g one after another.
-template <int NP>
-__device__ __forceinline__ void elem_item_lowreg(const ProbDesc &P, int64_t g, unsigned char *smem)
-{
-    constexpr int NP3 = NP * NP * NP;
-    const float h1h = (float)P.h1, h2h = (float)P.h2;
-    const dfp H1 = {h1h, (float)(P.h1 - (double)h1h)}, H2 = {h2h, (float)(P.h2 - (double)h2h)};
-    for (int t = 0; t < P.NE; ++t) {
-        const int64_t e = g * P.NE + t;
-        if (e >= P.E) break;  // uniform across the block
-        const double *x = P.x + e * NP3;
-        double *w = P.w + e * NP3;
-        auto load = [&](int q) { return __ldcg(x + q); };
-        auto store = [&](int q, double v) { w[q] = v; };
-        ax_df_element_lowreg<NP>(load, store, P.geodf + e * 7 * NP3, H1, H2, P.Ddf, smem);
-    }
+    double *su = sm + 2 * NP * NP + (size_t)(inrange ? grp : 0) * 3 * C::NP3;
+    double *svr = su + C::NP3, *svs = svr + C::NP3;
+    const size_t off = (size_t)(active ? e : 0) * C::NP3;
+    const double *geo = P.geo64 + (active ? e : 0) * 7 * C::NP3;
+    ax_load_D<NP, double>(P.D64, sD, sDT);
+    auto load = [&](int q) { return a_input(P, ax0, beta, first, off + q); };
+    auto store = [&](int q, double v, double u) {
+        P.w[off + q] = v;
+        if (!ax0) acc = fma(u, v, acc);
+    };
+    ax_element<NP, double>(load, store, geo, P.h1, P.h2, sD, sDT, su, svr, svs, tid, active);
 }
 
 // TC inner operator (16-bit tensor-core contractions, FP32 vectors).  tc: 1
 // BF16, 2 FP16 (plain rounding); 3 FP16 x2, 4 BF16 x3 (split operands, N+1 <= 8).
 template <int NP>
-__device__ __forceinline__ void elem_item_tc(const ProbDesc &P, double alpha, double beta, int first,
-                                             int64_t g, int tc, unsigned char *smem, double &acc)
+__device__ __forceinline__ void elem_item_tc(const ProbDesc &P, double beta, int first, int64_t g, int tc,
+                                             unsigned char *smem, dfacc &dot)
 {
-    const float b32 = (float)beta, a32 = (float)alpha;
+    const float b32 = (float)beta;
     auto load = [&](int64_t q) {
-        float pn = __ldcg(P.minv32 + q) * __ldcg(P.r32 + q);
-        if (!first) {
-            const float po = __ldcg(P.p32 + q);
-            P.d32[q] = fmaf(a32, po, __ldcg(P.d32 + q));
-            pn = fmaf(b32, po, pn);
-        }
+        float pn = __ldcg(P.w32 + q);
+        if (!first) pn = fmaf(b32, __ldcg(P.p32 + q), pn);
         P.p32[q] = pn;
         return pn;
     };
-    dfacc dot = {0.f, 0.f};
     auto store = [&](int64_t q, float v, float u) {
         P.w32[q] = v;
         dot2_acc(dot, u, v);
@@ -543,268 +631,215 @@ __device__ __forceinline__ void elem_item_tc(const ProbDesc &P, double alpha, do
         ax_tc_split_group<NP, false>(load, store, P.geo32, P.D32, (float)P.h1, (float)P.h2, P.E, g, smem);
     else
         ax_tc_group<NP>(load, store, P.geo32, P.D32, (float)P.h1, (float)P.h2, P.E, g, tc == 2, smem);
-    acc += dfacc_value(dot);
 }
 
+// Whether the element phases of order NP in MODE are line phases (A32 always is).
 template <int NP, int MODE>
-__device__ __forceinline__ void elem_dispatch_np(const ProbDesc &P, int ph, double alpha, double beta,
-                                                 int first, int64_t g, int tc, unsigned char *smem,
-                                                 double &acc)
+constexpr bool line_mode()
 {
-    if constexpr (MODE == MODE_F64 && solve_bfp<NP>()) {
-        if (ph == PH_AX0)
-            elem_item_bfp<NP, 0>(P, alpha, beta, first, g, smem, acc);
-        else
-            elem_item_bfp<NP, 1>(P, alpha, beta, first, g, smem, acc);
-    } else if constexpr (MODE == MODE_F64 && df_folded<NP>()) {
-        if (ph == PH_AX0)
-            elem_item_dfeo<NP, 0>(P, alpha, beta, first, g, smem, acc);
-        else
-            elem_item_dfeo<NP, 1>(P, alpha, beta, first, g, smem, acc);
-    } else if constexpr (MODE == MODE_F64) {
-        if (ph == PH_AX0)
-            elem_item_df<NP, 0>(P, alpha, beta, first, g, smem, acc);
-        else
-            elem_item_df<NP, 1>(P, alpha, beta, first, g, smem, acc);
-    } else if constexpr (MODE == MODE_F64N) {
-        if (ph == PH_AX0)
-            elem_item<NP, 0>(P, alpha, beta, first, g, smem, acc);
-        else
-            elem_item<NP, 1>(P, alpha, beta, first, g, smem, acc);
+    return MODE == MODE_F32 || (MODE == MODE_F64 && (solve_bfp<NP>() || solve_dfl<NP>()));
+}
+
+// This CTA's share of an element phase; returns the next problem's rot.
+template <int NP, int MODE, int TH>
+__device__ __forceinline__ unsigned phase_elem_np(const ProbDesc &P, int ph, double beta, int first,
+                                                  const Deal &deal, unsigned char *smem, double &acc, dfacc &dot)
+{
+    const bool ax0 = ph == PH_AX0;
+    if constexpr (MODE == MODE_F64 && (solve_bfp<NP>() || solve_dfl<NP>())) {
+        phase_a64<NP, TH>(P, ax0, beta, first, deal, smem, acc);
+    } else if (MODE == MODE_F32 && !ax0) {
+        if constexpr (MODE == MODE_F32) phase_a32<NP, TH>(P, beta, first, deal, smem, dot);
+    } else if (MODE == MODE_TC && !ax0 && P.tc == 0) {  // each problem of the launch has its own inner path
+        if constexpr (MODE == MODE_TC) phase_a32<NP, TH>(P, beta, first, deal, smem, dot);
+    } else if ((MODE == MODE_F32 || MODE == MODE_TC) && ax0) {
+        if constexpr (MODE == MODE_F32 || MODE == MODE_TC) phase_ax0_lowreg<NP, TH>(P, deal, smem);
+        constexpr int NG = TH / SEM_SOLVE_THREADS;
+        return deal.after((unsigned)P.E, SEM_SOLVE_THREADS / 32, NG, TH / 32);
     } else {
-        if (ph == PH_AX0) {
-            elem_item_lowreg<NP>(P, g, smem);
-        } else if constexpr (MODE == MODE_TC) {
-            // each problem of the launch has its own inner path
-            if (P.tc == 0)
-                elem_item<NP, 2>(P, alpha, beta, first, g, smem, acc);
-            else
-                elem_item_tc<NP>(P, alpha, beta, first, g, P.tc, smem, acc);
-        } else
-            elem_item<NP, 2>(P, alpha, beta, first, g, smem, acc);
+        // whole CTAs take groups of elements in turn
+        const int ne = MODE == MODE_TC ? P.NE32 : P.NE;
+        const int64_t items = (P.E + ne - 1) / ne;
+        for (int64_t g = deal.first(0, 1, 1); g < items; g += deal.ncta) {
+            if constexpr (MODE == MODE_F64) elem_item_df<NP>(P, ax0, beta, first, g, smem, acc);
+            if constexpr (MODE == MODE_F64N) elem_item_native<NP>(P, ax0, beta, first, g, smem, acc);
+            if constexpr (MODE == MODE_TC) elem_item_tc<NP>(P, beta, first, g, P.tc, smem, dot);
+        }
+        return deal.after((unsigned)(items % deal.ncta), 1, 1, TH / 32);
     }
+    using G = GrpCfg<NP, TH>;
+    return deal.after((unsigned)((P.E + G::GE - 1) / G::GE), G::GT / 32, G::NG, TH / 32);
 }
 
-template <int MODE, int... NPs>
-struct ElemDispatch;
-
-template <int MODE>
-struct ElemDispatch<MODE> {
-    __device__ static void run(const ProbDesc &, int, double, double, int, int64_t, int,
-                               unsigned char *, double &) {}
-};
-
-template <int MODE, int NP0, int... NPs>
-struct ElemDispatch<MODE, NP0, NPs...> {
-    __device__ static void run(const ProbDesc &P, int ph, double alpha, double beta, int first,
-                               int64_t g, int tc, unsigned char *smem, double &acc)
-    {
-        if (P.n == NP0)
-            elem_dispatch_np<NP0, MODE>(P, ph, alpha, beta, first, g, tc, smem, acc);
-        else
-            ElemDispatch<MODE, NPs...>::run(P, ph, alpha, beta, first, g, tc, smem, acc);
-    }
-};
-
 // ---------------------------------------------------------------------------
-// unique-node and local-node items (one node per thread)
+// unique-node and local-node phases
 // ---------------------------------------------------------------------------
 
-// y/z copies of one row (gy, gz) of unique nodes: local offsets without the x part.
-struct RowCopies {
-    int m;
-    int64_t off[4];
-};
+// Iterations that update x themselves (FP64 modes); later ones gather their
+// corrections in y, at the owned nodes alone, and x += y follows once at the end
+// (740 iterations at 16^3 elements, N = 7: 31 us a C phase against 37).  A solve
+// of few iterations saves that last pass.
+constexpr int X_DIRECT = 4;
 
-__device__ __forceinline__ void row_copies(const GsDesc &d, int row, RowCopies &R)
+// Chunk t of a unique phase.  v: FP64 sums; d: the sums of the FP32 phases, in
+// float pairs (converting them once a chunk cost more FP64 operations than an
+// FP64 phase has).
+template <int NP, int MODE>
+__device__ __forceinline__ void uniq_item(const ProbDesc &P, const PState &S, int ph, unsigned t, double v[3],
+                                          dfacc d[2])
 {
-    const int gy = row % d.ngy, gz = row / d.ngy;
-    int ey[2], iy[2], ez[2], iz[2];
-    const int my = gs_copies_1d(gy, d.N, d.nely, d.py, ey, iy);
-    const int mz = gs_copies_1d(gz, d.N, d.nelz, d.pz, ez, iz);
-    const int64_t n3 = (int64_t)d.n * d.n * d.n;
-    R.m = 0;
-    for (int c = 0; c < mz; ++c)
-        for (int b = 0; b < my; ++b)
-            R.off[R.m++] = ((int64_t)ey[b] + (int64_t)d.nely * ez[c]) * d.nelx * n3 +
-                           (int64_t)(iz[c] * d.n + iy[b]) * d.n;
-}
-
-// Copy k (y/z part) x a (x part) of a unique node; valid when k < R.m, a < mx.
-#define UQ_FOR_COPIES(R, mx, xo, BODY)                              \
-    _Pragma("unroll") for (int k_ = 0; k_ < 4; ++k_)                \
-        _Pragma("unroll") for (int a_ = 0; a_ < 2; ++a_)            \
-            if (k_ < (R).m && a_ < (mx)) {                          \
-                const int64_t cp = (R).off[k_] + (xo)[a_];          \
-                BODY;                                               \
-            }
-
-__device__ __forceinline__ void uniq_item(const ProbDesc &P, const PState &S, int ph, int64_t item,
-                                          double v[3])
-{
-    const GsDesc &d = P.gs;
-    const int nxch = (d.ngx + SEM_SOLVE_THREADS - 1) / SEM_SOLVE_THREADS;
-    const int it32 = (int)item;  // unique-node items fit in 32 bits (checked at setup)
-    const int rg = it32 / nxch;
-    const int gx = (it32 - rg * nxch) * SEM_SOLVE_THREADS + threadIdx.x;
-    const int rows = d.ngy * d.ngz;
-    if (gx >= d.ngx) return;
-    const int64_t n3 = (int64_t)d.n * d.n * d.n;
-    int ex[2], ix[2];
-    const int mx = gs_copies_1d(gx, d.N, d.nelx, d.px, ex, ix);
-    const int64_t xo[2] = {ex[0] * n3 + ix[0], mx > 1 ? ex[1] * n3 + ix[1] : 0};
-    constexpr int RU = SEM_UQ_ROWS;
-    RowCopies R[RU];
-    bool ok[RU];
+    constexpr int CH = UqCfg<NP>::CH;
+    constexpr bool MIXED = MODE == MODE_F32 || MODE == MODE_TC;
+    const UqChunk U = uq_chunk<NP>(P.mesh, t);
+    if constexpr (!MIXED) {
+        if (ph == PH_C || ph == PH_R0) {
+            // C: r -= alpha dssum(w), y += alpha p;  R0: r = (b - mean) - dssum(w)
+            const bool c = ph == PH_C;
+            const double alpha = c ? S.alpha : 1.0, shift = S.bmean;
+            double s[CH], r0[CH], mv[CH], po[CH], yo[CH];
 #pragma unroll
-    for (int r = 0; r < RU; ++r) {
-        const int row = rg * RU + r;
-        ok[r] = row < rows;
-        if (ok[r]) row_copies(d, row, R[r]);
-        else R[r].m = 0;
-    }
-    switch (ph) {
-        case PH_JACGS: {
-            if (P.jac_cached) {  // the Jacobi inverse is kept from an earlier solve: only sum b
-#pragma unroll
-                for (int r = 0; r < RU; ++r)
-                    if (ok[r]) v[0] += __ldcg(P.b + R[r].off[0] + xo[0]);
-                break;
-            }
-            double s[RU], bv[RU];
-#pragma unroll
-            for (int r = 0; r < RU; ++r) {
-                s[r] = 0.0;
-                bv[r] = 0.0;
-                if (!ok[r]) continue;
-                UQ_FOR_COPIES(R[r], mx, xo, s[r] += __ldcg(P.minv + cp));
-                bv[r] = __ldcg(P.b + R[r].off[0] + xo[0]);
-            }
-#pragma unroll
-            for (int r = 0; r < RU; ++r) {
-                if (!ok[r]) continue;
-                const double rinv = 1.0 / s[r];
-                UQ_FOR_COPIES(R[r], mx, xo, {
-                    P.minv[cp] = rinv;
-                    if (P.minv32) P.minv32[cp] = (float)rinv;
-                });
-                v[0] += bv[r];
-            }
-        } break;
-        case PH_R0:
-        case PH_R64: {
-            double s[RU], bv[RU], mv[RU];
-#pragma unroll
-            for (int r = 0; r < RU; ++r) {
-                s[r] = 0.0;
-                bv[r] = mv[r] = 0.0;
-                if (!ok[r]) continue;
-                UQ_FOR_COPIES(R[r], mx, xo, s[r] += __ldcg(P.w + cp));
-                const int64_t f = R[r].off[0] + xo[0];
-                bv[r] = __ldcg(P.b + f) - S.bmean;
-                if (ph == PH_R0) mv[r] = __ldcg(P.minv + f);
-            }
-#pragma unroll
-            for (int r = 0; r < RU; ++r) {
-                if (!ok[r]) continue;
-                const double rv = bv[r] - s[r];
-                UQ_FOR_COPIES(R[r], mx, xo, P.r[cp] = rv);
-                v[0] = fma(rv, rv, v[0]);
-                if (ph == PH_R0) {
-                    v[1] = fma(rv, mv[r] * rv, v[1]);
-                    v[2] = fma(bv[r], bv[r], v[2]);
+            for (int i = 0; i < CH; ++i) r0[i] = yo[i] = po[i] = 0.0;
+            uq_gather(P.w, U, s, [&] {
+                uq_ldv(P.minv + U.f, mv);
+                if (c) {
+                    uq_ldv(P.r + U.f, r0);
+                    uq_ldv(P.p + U.f, po);
+                    if (P.y && S.iters > X_DIRECT) uq_ldv(P.y + U.f, yo);
                 } else {
-                    v[1] = fma(bv[r], bv[r], v[1]);
+                    uq_ldu(P.b + U.f, r0, U.own, P.vec);
+                }
+            });
+            if (!c)
+#pragma unroll
+                for (int i = 0; i < CH; ++i) r0[i] -= shift;
+            // (slots past the owned nodes carry junk; nothing reads them)
+#pragma unroll
+            for (int i = 0; i < CH; ++i) {
+                if (!c && i < U.own) v[2] = fma(r0[i], r0[i], v[2]);
+                r0[i] = fma(-alpha, s[i], r0[i]);
+                s[i] = mv[i] * r0[i];
+                yo[i] = fma(alpha, po[i], yo[i]);
+                if (i < U.own) {
+                    v[0] = fma(r0[i], r0[i], v[0]);
+                    v[1] = fma(r0[i], s[i], v[1]);
                 }
             }
-        } break;
-        case PH_C: {
-            double s[RU], r0[RU], mv[RU];
-#pragma unroll
-            for (int r = 0; r < RU; ++r) {
-                s[r] = r0[r] = mv[r] = 0.0;
-                if (!ok[r]) continue;
-                UQ_FOR_COPIES(R[r], mx, xo, s[r] += __ldcg(P.w + cp));
-                const int64_t f = R[r].off[0] + xo[0];
-                r0[r] = __ldcg(P.r + f);
-                mv[r] = __ldcg(P.minv + f);
-            }
-#pragma unroll
-            for (int r = 0; r < RU; ++r) {
-                if (!ok[r]) continue;
-                const double rv = r0[r] - S.alpha * s[r];
-                UQ_FOR_COPIES(R[r], mx, xo, P.r[cp] = rv);
-                v[0] = fma(rv, rv, v[0]);
-                v[1] = fma(rv, mv[r] * rv, v[1]);
-            }
-        } break;
-        case PH_INIT32: {
-            double r0[RU];
-            float mv[RU];
-#pragma unroll
-            for (int r = 0; r < RU; ++r) {
-                r0[r] = 0.0;
-                mv[r] = 0.f;
-                if (!ok[r]) continue;
-                const int64_t f = R[r].off[0] + xo[0];
-                r0[r] = __ldcg(P.r + f);
-                mv[r] = __ldcg(P.minv32 + f);
-            }
-            dfacc d0 = {0.f, 0.f}, d1 = {0.f, 0.f};
-#pragma unroll
-            for (int r = 0; r < RU; ++r) {
-                if (!ok[r]) continue;
-                const float rv = (float)(r0[r] / S.scale);
-                UQ_FOR_COPIES(R[r], mx, xo, {
-                    P.r32[cp] = rv;
-                    P.d32[cp] = 0.0f;
-                });
-                dot2_acc(d0, rv, rv);
-                dot2_acc(d1, rv, mv[r] * rv);
-            }
-            v[0] += dfacc_value(d0);
-            v[1] += dfacc_value(d1);
-        } break;
-        case PH_C32: {
-            float s[RU], r0[RU], mv[RU];
-#pragma unroll
-            for (int r = 0; r < RU; ++r) {
-                s[r] = r0[r] = mv[r] = 0.f;
-                if (!ok[r]) continue;
-                UQ_FOR_COPIES(R[r], mx, xo, s[r] += __ldcg(P.w32 + cp));
-                const int64_t f = R[r].off[0] + xo[0];
-                r0[r] = __ldcg(P.r32 + f);
-                mv[r] = __ldcg(P.minv32 + f);
-            }
+            uq_stv(P.r + U.f, r0, CH);
+            uq_scatter(P.w, U, s);
+            if (c && P.y && S.iters >= X_DIRECT)
+                uq_stv(P.y + U.f, yo, CH);
+            else if (c)
+                uq_update<CH>(P.x, U, P.vec, [&](int i, double xv) { return fma(alpha, po[i], xv); });
+            return;
+        }
+        if (ph == PH_XUPD) {
+            double yv[CH];
+            uq_ldv(P.y + U.f, yv);
+            uq_update<CH>(P.x, U, P.vec, [&](int i, double xv) { return xv + yv[i]; });
+            return;
+        }
+    } else {
+        if (ph == PH_C32) {
             const float a = (float)S.alpha;
-            dfacc d0 = {0.f, 0.f}, d1 = {0.f, 0.f};
+            float s[CH], r0[CH], mv[CH], po[CH], dv[CH];
+            uq_gather(P.w32, U, s, [&] {
+                uq_ldv(P.r32 + U.f, r0);
+                uq_ldv(P.minv32 + U.f, mv);
+                uq_ldv(P.p32 + U.f, po);
+                uq_ldv(P.d32 + U.f, dv);
+            });
 #pragma unroll
-            for (int r = 0; r < RU; ++r) {
-                if (!ok[r]) continue;
-                const float rv = r0[r] - a * s[r];
-                UQ_FOR_COPIES(R[r], mx, xo, P.r32[cp] = rv);
-                dot2_acc(d0, rv, rv);
-                dot2_acc(d1, rv, mv[r] * rv);
+            for (int i = 0; i < CH; ++i) {
+                r0[i] = r0[i] - a * s[i];
+                s[i] = mv[i] * r0[i];
+                dv[i] = fmaf(a, po[i], dv[i]);
+                if (i < U.own) {
+                    dot2_acc(d[0], r0[i], r0[i]);
+                    dot2_acc(d[1], r0[i], s[i]);
+                }
             }
-            v[0] += dfacc_value(d0);
-            v[1] += dfacc_value(d1);
-        } break;
-        default: break;
+            uq_stv(P.r32 + U.f, r0, CH);
+            uq_stv(P.d32 + U.f, dv, CH);
+            uq_scatter(P.w32, U, s);
+            return;
+        }
+        if (ph == PH_R64) {
+            double s[CH], bv[CH];
+            uq_gather(P.w, U, s, [&] { uq_ldu(P.b + U.f, bv, U.own, P.vec); });
+#pragma unroll
+            for (int i = 0; i < CH; ++i) {
+                bv[i] -= S.bmean;
+                s[i] = bv[i] - s[i];
+                if (i < U.own) {
+                    v[0] = fma(s[i], s[i], v[0]);
+                    v[1] = fma(bv[i], bv[i], v[1]);
+                }
+            }
+            uq_stv(P.r + U.f, s, CH);
+            return;
+        }
+        if (ph == PH_INIT32) {
+            double r[CH];
+            float mv[CH], z[CH], rv[CH], zero[CH];
+            uq_ldv(P.r + U.f, r);
+            uq_ldv(P.minv32 + U.f, mv);
+#pragma unroll
+            for (int i = 0; i < CH; ++i) {
+                rv[i] = (float)(r[i] / S.scale);
+                z[i] = mv[i] * rv[i];
+                zero[i] = 0.f;
+                if (i < U.own) {
+                    dot2_acc(d[0], rv[i], rv[i]);
+                    dot2_acc(d[1], rv[i], z[i]);
+                }
+            }
+            uq_stv(P.r32 + U.f, rv, CH);
+            uq_stv(P.d32 + U.f, zero, CH);
+            uq_scatter(P.w32, U, z);
+            return;
+        }
+        if (ph == PH_UPD) {
+            // the FP64 p vector is unused by refinement: it keeps x until the
+            // next residual accepts the step
+            float dv[CH];
+            uq_ldv(P.d32 + U.f, dv);
+            uq_each<CH>(U, [&](unsigned q, int i) {
+                const double xv = __ldcg(P.x + q);
+                P.p[q] = xv;
+                P.x[q] = fma(S.scale, (double)dv[i], xv);
+            });
+            return;
+        }
+    }
+    if (ph == PH_JACGS) {
+        if (P.singular)
+#pragma unroll
+            for (int i = 0; i < CH; ++i)
+                if (i < U.own) v[0] += __ldcg(P.b + U.f + i);
+        if (P.jac_cached || P.jac_shared) return;  // only the sum of b
+        double s[CH];
+        uq_gather(P.minv, U, s, [] {});
+#pragma unroll
+        for (int i = 0; i < CH; ++i) s[i] = 1.0 / s[i];
+        uq_scatter(P.minv, U, s);
+        if (P.minv32) {
+            float f[CH];
+#pragma unroll
+            for (int i = 0; i < CH; ++i) f[i] = (float)s[i];
+            uq_scatter(P.minv32, U, f);
+        }
     }
 }
 
-__device__ __forceinline__ void local_item(const ProbDesc &P, const PState &S, int ph, int64_t chunk,
-                                           double v[3])
+__device__ __forceinline__ void local_item(const ProbDesc &P, const PState &S, int ph, unsigned q, double v[3])
 {
-    const int64_t q = chunk * SEM_SOLVE_THREADS + threadIdx.x;
-    if (q >= P.nL) return;
-    const int n = P.n, n3 = n * n * n;
-    const int64_t e = q / n3;
+    const int n = P.n, n3 = (int)P.dn3.d;
+    const unsigned e = fd_div(q, P.dn3);
     const int l = (int)(q - e * n3);
     switch (ph) {
         case PH_JAC: {
             const int i = l % n, j = (l / n) % n, k = l / (n * n);
-            const double *g = P.geo64 + e * 7 * n3;
+            const double *g = P.geo64 + (size_t)e * 7 * n3;
             const double *D = P.D64;
             double s = 0.0;
             for (int t = 0; t < n; ++t) {
@@ -817,23 +852,11 @@ __device__ __forceinline__ void local_item(const ProbDesc &P, const PState &S, i
             s += 2.0 * (di * dj * g[3 * n3 + l] + di * dk * g[4 * n3 + l] + dj * dk * g[5 * n3 + l]);
             P.minv[q] = P.h1 * s + P.h2 * g[6 * n3 + l];
         } break;
-        case PH_UPD: {
-            // the FP64 p vector is unused by refinement: it keeps x until the
-            // next residual accepts the step
-            float dv = __ldcg(P.d32 + q);
-            if (S.pending) dv = fmaf((float)S.alpha, __ldcg(P.p32 + q), dv);
-            const double xo = __ldcg(P.x + q);
-            P.p[q] = xo;
-            P.x[q] = fma(S.scale, (double)dv, xo);
-        } break;
         case PH_XREST:
             P.x[q] = __ldcg(P.p + q);
             break;
-        case PH_XUPD:
-            P.x[q] = fma(S.alpha, __ldcg(P.p + q), __ldcg(P.x + q));
-            break;
         case PH_FINAL:
-            v[0] = fma(P.geo64[(e * 7 + 6) * n3 + l], __ldcg(P.x + q), v[0]);
+            v[0] = fma(P.geo64[((size_t)e * 7 + 6) * n3 + l], __ldcg(P.x + q), v[0]);
             break;
         case PH_SHIFT:
             P.x[q] = __ldcg(P.x + q) - S.shift;
@@ -843,21 +866,30 @@ __device__ __forceinline__ void local_item(const ProbDesc &P, const PState &S, i
 }
 
 // ---------------------------------------------------------------------------
-// per-problem state machine (run by one thread of the last CTA of a step)
+// per-problem state machine (run by one thread of every CTA between steps)
 // ---------------------------------------------------------------------------
+
+// Whether sqrt(rr) <= target; the square root is only taken near the target.
+__device__ __forceinline__ bool norm_met(double rr, double target)
+{
+    const double t2 = target * target;
+    if (t2 > 1e-290 && rr > t2 * (1.0 + 1e-12)) return false;
+    return sqrt(rr) <= target;
+}
 
 template <int MAXP>
 __device__ void advance(const SolveParams<MAXP> &prm, const ProbDesc &P, PState &S, const double *red)
 {
     const int ph = S.phase;
+    const int tail = P.singular ? PH_FINAL : PH_DONE;
     auto finish = [&](int status) {
         S.status = status;
-        S.phase = P.singular ? PH_FINAL : PH_DONE;
+        S.phase = tail;
     };
-    // after a C phase the last alpha p is not yet in x
-    auto finish_pending = [&](int status) {
+    // after C phases past the first X_DIRECT the correction y is not yet in x
+    auto finish_y = [&](int status) {
         S.status = status;
-        S.phase = PH_XUPD;
+        S.phase = (P.y && S.iters > X_DIRECT) ? PH_XUPD : tail;
     };
     switch (ph) {
         case PH_JAC: S.phase = PH_JACGS; break;
@@ -880,16 +912,24 @@ __device__ void advance(const SolveParams<MAXP> &prm, const ProbDesc &P, PState 
         } break;
         case PH_A: {
             const double pw = red[0];
-            if (!(pw > 0.0) || !isfinite(pw)) { finish(SEM_ERR_BREAKDOWN); break; }
+            if (!(pw > 0.0) || !isfinite(pw)) {
+                if (S.iters > 0) S.rnorm = sqrt(S.rnorm);  // (phase C keeps its square)
+                finish_y(SEM_ERR_BREAKDOWN);
+                break;
+            }
             S.alpha = S.rz / pw;
             S.phase = PH_C;
         } break;
         case PH_C: {
             S.iters += 1;
-            S.rnorm = sqrt(red[0]);
-            if (!isfinite(S.rnorm)) { finish_pending(SEM_ERR_BREAKDOWN); break; }
-            if (S.rnorm <= S.target) { finish_pending(SEM_OK); break; }
-            if (S.iters >= prm.maxit) { finish_pending(SEM_ERR_NOT_CONVERGED); break; }
+            const double rr = red[0];
+            const bool met = norm_met(rr, S.target);
+            if (!isfinite(rr) || met || S.iters >= prm.maxit) {
+                S.rnorm = sqrt(rr);
+                finish_y(!isfinite(rr) ? SEM_ERR_BREAKDOWN : met ? SEM_OK : SEM_ERR_NOT_CONVERGED);
+                break;
+            }
+            S.rnorm = rr;  // squared until the solve ends
             S.beta = red[1] / S.rz;
             S.rz = red[1];
             S.first = 0;
@@ -930,21 +970,18 @@ __device__ void advance(const SolveParams<MAXP> &prm, const ProbDesc &P, PState 
             S.first = 1;
             S.beta = 0.0;
             S.inner_iters = 0;
-            S.pending = 0;
             S.phase = (red[0] > 0.0) ? PH_A32 : PH_UPD;
         } break;
         case PH_A32: {
             const double pw = red[0];
-            if (!(pw > 0.0) || !isfinite(pw)) { S.pending = 0; S.phase = PH_UPD; break; }
+            if (!(pw > 0.0) || !isfinite(pw)) { S.phase = PH_UPD; break; }
             S.alpha = S.rz / pw;
             S.phase = PH_C32;
         } break;
         case PH_C32: {
             S.iters += 1;
             S.inner_iters += 1;
-            const double rn = sqrt(red[0]);
-            if (!isfinite(rn) || rn <= S.inner_target || S.iters >= prm.maxit) {
-                S.pending = 1;
+            if (!isfinite(red[0]) || norm_met(red[0], S.inner_target) || S.iters >= prm.maxit) {
                 S.phase = PH_UPD;
                 break;
             }
@@ -956,208 +993,290 @@ __device__ void advance(const SolveParams<MAXP> &prm, const ProbDesc &P, PState 
         case PH_UPD: S.outer += 1; S.phase = PH_AX0; break;
         case PH_FINAL: S.shift = red[0] / P.volume; S.phase = PH_SHIFT; break;
         case PH_SHIFT: S.phase = PH_DONE; break;
-        case PH_XUPD: case PH_XREST: S.phase = P.singular ? PH_FINAL : PH_DONE; break;
+        case PH_XUPD: case PH_XREST: S.phase = tail; break;
         default: S.phase = PH_DONE; break;
     }
-    S.nvals = phase_nvals(S.phase);
 }
 
 // ---------------------------------------------------------------------------
 // the persistent kernel
 // ---------------------------------------------------------------------------
 
-template <int MAXP, int MODE, int... NPs>
-__global__ void __launch_bounds__(SEM_SOLVE_THREADS, MODE == MODE_F32 ? SEM_SOLVE_F32_MINB : SEM_SOLVE_F64_MINB)
-    k_solve(const __grid_constant__ SolveParams<MAXP> prm)
+enum PhaseKind { KIND_ELEM, KIND_UNIQ, KIND_LOCAL };
+
+__host__ __device__ __forceinline__ int phase_kind(int ph)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ double s_part[MAXP][3];
-    __shared__ double s_red[SEM_SOLVE_THREADS / 32 * 3];
-    __shared__ int s_phase[MAXP];
-    __shared__ long long s_offs[MAXP + 1];
-    __shared__ double s_alpha[MAXP], s_beta[MAXP], s_bmean[MAXP], s_scale[MAXP], s_shift[MAXP];
-    __shared__ int s_first[MAXP], s_pending[MAXP];
-    __shared__ int s_last, s_stop;
-    __shared__ unsigned s_gen;
-    const int np = prm.nprob;
-    SyncState *sync = prm.sync;
-    if constexpr (MODE == MODE_F64)  // reduction words of the block-floating-point element phases
-        for (int t = threadIdx.x; t < SEM_BFP_RED_BYTES / 4; t += blockDim.x)
-            reinterpret_cast<unsigned *>(smem)[t] = 0u;
-
-    for (int step = 0;; ++step) {
-        // ---- schedule of this step
-        if (threadIdx.x == 0) {
-            long long o = 0;
-            for (int p = 0; p < np; ++p) {
-                int ph;
-                if (step == 0) {
-                    ph = prm.prob[p].jac_cached ? PH_JACGS : PH_JAC;
-                } else {
-                    ph = ((volatile int *)prm.sched)[p];
-                }
-                s_phase[p] = ph;
-                s_offs[p] = o;
-                o += phase_items(prm.prob[p], ph);
-            }
-            s_offs[np] = o;
-            s_stop = (step > 0 && ((volatile int *)&sync->finished)[0]) ||
-                     ((volatile int *)&sync->err)[0];
-        }
-        for (int p = threadIdx.x; p < np; p += blockDim.x) {
-            const volatile PState *S = prm.st + p;
-            s_alpha[p] = S->alpha;
-            s_beta[p] = S->beta;
-            s_bmean[p] = S->bmean;
-            s_scale[p] = S->scale;
-            s_shift[p] = S->shift;
-            s_first[p] = S->first;
-            s_pending[p] = S->pending;
-            s_part[p][0] = s_part[p][1] = s_part[p][2] = 0.0;
-        }
-        __syncthreads();
-        if (s_stop) break;
-
-        // ---- work items
-        const long long total = s_offs[np];
-        double v[3] = {0.0, 0.0, 0.0};
-        double acc = 0.0;
-        int cur = -1;
-        for (long long it = blockIdx.x; it < total; it += gridDim.x) {
-            int p = 0;
-            while (p + 1 < np && s_offs[p + 1] <= it) ++p;
-            if (p != cur) {
-                if (cur >= 0) {
-                    v[0] += acc;
-                    acc = 0.0;
-                    block_accumulate(v, s_red, s_part[cur]);
-                }
-                cur = p;
-            }
-            const ProbDesc &P = prm.prob[p];
-            const int ph = s_phase[p];
-            const int64_t local = it - s_offs[p];
-            PState S;
-            S.alpha = s_alpha[p];
-            S.beta = s_beta[p];
-            S.bmean = s_bmean[p];
-            S.scale = s_scale[p];
-            S.shift = s_shift[p];
-            S.pending = s_pending[p];
-            if (ph == PH_AX0 || ph == PH_A || ph == PH_A32) {
-                ElemDispatch<MODE, NPs...>::run(P, ph, S.alpha, S.beta, s_first[p], local,
-                                                prm.inner_tc, smem, acc);
-            } else if (ph == PH_JAC || ph == PH_UPD || ph == PH_FINAL || ph == PH_SHIFT ||
-                       ph == PH_XUPD || ph == PH_XREST) {
-                local_item(P, S, ph, local, v);
-            } else {
-                uniq_item(P, S, ph, local, v);
-            }
-        }
-        if (cur >= 0) {
-            v[0] += acc;
-            block_accumulate(v, s_red, s_part[cur]);
-        }
-
-        // ---- publish partials, reducing barrier
-        double *part = prm.partials + (size_t)blockIdx.x * MAXP * 3;
-        for (int t = threadIdx.x; t < np * 3; t += blockDim.x) part[t] = s_part[t / 3][t % 3];
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            s_gen = ((volatile unsigned *)&sync->gen)[0];
-            const unsigned arrived = atomicAdd(&sync->count, 1u);
-            s_last = (arrived == gridDim.x - 1);
-        }
-        __syncthreads();
-        if (s_last) {
-            __threadfence();
-            // fixed-order reduction of every (problem, value) pair: one warp each
-            const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-            for (int pk = warp; pk < np * 3; pk += SEM_SOLVE_THREADS / 32) {
-                const int p = pk / 3, k = pk % 3;
-                double s = 0.0;
-                if (k < phase_nvals(s_phase[p]))
-                    for (int b = lane; b < (int)gridDim.x; b += 32)
-                        s += __ldcg(prm.partials + ((size_t)b * MAXP + p) * 3 + k);
-                s = warp_sum(s);
-                if (lane == 0) s_part[p][k] = s;
-            }
-            __syncthreads();
-            for (int p = threadIdx.x; p < np; p += blockDim.x) {
-                PState S = prm.st[p];
-                S.phase = s_phase[p];
-                advance<MAXP>(prm, prm.prob[p], S, s_part[p]);
-                prm.st[p] = S;
-                prm.sched[p] = S.phase;
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                int fin = 1;
-                for (int p = 0; p < np; ++p) fin &= (prm.sched[p] == PH_DONE);
-                sync->finished = fin;
-                sync->count = 0;
-                __threadfence();
-                atomicAdd(&sync->gen, 1u);
-            }
-        } else if (threadIdx.x == 0) {
-            const unsigned long long t0 = sem_globaltimer();
-            while (ld_acquire_u32(&sync->gen) == s_gen) {
-                if (((volatile int *)&sync->err)[0]) break;
-                if ((long long)(sem_globaltimer() - t0) > prm.timeout_ns) {
-                    atomicExch(&sync->err, SEM_ERR_TIMEOUT);
-                    break;
-                }
-                __nanosleep(128);
-            }
-            __threadfence();
-        }
-        __syncthreads();
+    switch (ph) {
+        case PH_AX0: case PH_A: case PH_A32: return KIND_ELEM;
+        case PH_JAC: case PH_XREST: case PH_FINAL: case PH_SHIFT: return KIND_LOCAL;
+        default: return KIND_UNIQ;
     }
 }
 
 constexpr size_t sem_max_sz(size_t a, size_t b) { return a > b ? a : b; }
 
-// Dynamic shared memory of the element phases of one problem order and mode.
-template <int NP, int MODE>
+// Dynamic shared memory of the element phases of one order and mode on TH threads.
+template <int NP, int MODE, int TH>
 constexpr size_t solve_smem_np()
 {
     return MODE == MODE_F64N ? ax_smem_bytes<NP, double>()
-           : MODE == MODE_F64 ? (solve_bfp<NP>() ? SEM_BFP_RED_BYTES + ax_bfp_smem_bytes_ne<NP, BfpCfg<NP>::NE>()
-                                 : df_folded<NP>() ? ax_dfeo_smem_bytes<NP>() : ax_df_smem_bytes<NP>())
-           : MODE == MODE_F32 ? sem_max_sz(ax_smem_bytes<NP, float>(), ax_df_lowreg_smem_bytes<NP>())
+           : MODE == MODE_F64 ? (line_mode<NP, MODE>() ? line64_smem_bytes<NP, TH>() : ax_df_smem_bytes<NP>())
+           : MODE == MODE_F32 ? sem_max_sz(elem32_smem_bytes<NP, TH>(), TH / SEM_SOLVE_THREADS * lowreg_smem_bytes<NP>())
                               : sem_max_sz(sem_max_sz(ax_tc_smem_bytes<NP>(), ax_tc_split_smem_bytes<NP>()),
-                                           sem_max_sz(ax_df_lowreg_smem_bytes<NP>(), ax_smem_bytes<NP, float>()));
+                                           sem_max_sz(lowreg_smem_bytes<NP>(), elem32_smem_bytes<NP, TH>()));
 }
 
-template <int MODE, int... NPs>
+template <int MODE, int TH, int... NPs>
 struct SmemMax;
-template <int MODE>
-struct SmemMax<MODE> {
+template <int MODE, int TH>
+struct SmemMax<MODE, TH> {
     static constexpr size_t v = 0;
 };
-template <int MODE, int NP0, int... NPs>
-struct SmemMax<MODE, NP0, NPs...> {
-    static constexpr size_t v = sem_max_sz(solve_smem_np<NP0, MODE>(), SmemMax<MODE, NPs...>::v);
+template <int MODE, int TH, int NP0, int... NPs>
+struct SmemMax<MODE, TH, NP0, NPs...> {
+    static constexpr size_t v = sem_max_sz(solve_smem_np<NP0, MODE, TH>(), SmemMax<MODE, TH, NPs...>::v);
 };
 
-// Host launcher (cooperative, grid sized for co-residency).
-template <int MAXP, int MODE, int... NPs>
-int launch_solve(const SolveParams<MAXP> &prm, int num_sms, long long max_items, cudaStream_t s)
+// Static shared memory of the kernel (states, sums, reduction words).
+template <int MAXP, int TH, bool PAIRS>
+constexpr size_t solve_static_smem()
 {
-    auto kern = k_solve<MAXP, MODE, NPs...>;
-    const size_t smem = SmemMax<MODE, NPs...>::v;
+    return MAXP * (sizeof(PState) + 3 * sizeof(double)) + 64 + TH / 8 +
+           (PAIRS && MAXP * (TH / 32) > TH ? MAXP * 3 * (TH / 32) : 3 * TH) * sizeof(double);
+}
+
+// Threads of a CTA: one CTA that fills its multiprocessor for the line phases
+// (512 threads of 128 registers in FP64, 768 of 80 in FP32) where the shared
+// memory allows it; 256 (two resident) for the others, whose element groups
+// are whole CTAs.
+template <int MAXP, int MODE, int... NPs>
+constexpr int solve_threads()
+{
+    constexpr int big = MODE == MODE_F32 ? 768 : 512;
+    return (line_mode<NPs, MODE>() && ...) &&
+                   SmemMax<MODE, big, NPs...>::v + solve_static_smem<MAXP, big, MODE == MODE_F32>() <= 227 * 1024
+               ? big
+               : SEM_SOLVE_THREADS;
+}
+
+template <int MODE, int TH, int... NPs>
+struct PhaseDispatch;
+
+template <int MODE, int TH, int NP0, int... NPs>
+struct PhaseDispatch<MODE, TH, NP0, NPs...> {
+    // This CTA's share of P's phase; returns the next problem's rot.
+    __device__ __forceinline__ static unsigned run(const ProbDesc &P, const PState &S, int kind, const Deal &deal,
+                                                   unsigned char *smem, double v[3], dfacc d[2])
+    {
+        if constexpr (sizeof...(NPs) > 0)
+            if (P.n != NP0) return PhaseDispatch<MODE, TH, NPs...>::run(P, S, kind, deal, smem, v, d);
+        if (kind == KIND_ELEM)
+            return phase_elem_np<NP0, MODE, TH>(P, S.phase, S.beta, S.first, deal, smem, v[0], d[0]);
+        // unique phases: warps take 32 chunks in turn
+        constexpr unsigned NW = TH / 32;
+        const unsigned units = uq_units<NP0>(P.mesh), portions = (units + 31) / 32;
+        for (unsigned g = deal.first(threadIdx.x / 32, 1, NW); g < portions; g += deal.ncta * NW) {
+            const unsigned t = g * 32 + (threadIdx.x & 31);
+            if (t < units) uniq_item<NP0, MODE>(P, S, S.phase, t, v, d);
+        }
+        return deal.after(portions, 1, NW, NW);
+    }
+    // Portions (groups of elements or four warps of chunks, the larger) of P.
+    static unsigned portions(const ProbDesc &P)
+    {
+        if constexpr (sizeof...(NPs) > 0)
+            if (P.n != NP0) return PhaseDispatch<MODE, TH, NPs...>::portions(P);
+        const unsigned ge = line_mode<NP0, MODE>() ? GrpCfg<NP0, TH>::GE : (unsigned)P.NE;
+        const unsigned a = ((unsigned)P.E + ge - 1) / ge, b = (uq_units<NP0>(P.mesh) + 127) / 128;
+        return a > b ? a : b;
+    }
+};
+
+template <int MAXP, int MODE, int TH, int... NPs>
+__global__ void __launch_bounds__(TH, TH > SEM_SOLVE_THREADS ? 1 : 2)
+    k_solve(const __grid_constant__ SolveParams<MAXP> prm)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ PState s_st[MAXP];
+    __shared__ double s_sum[MAXP][3];
+    // Sums of a problem's phase over the CTA: [value][thread], or, in an FP32
+    // launch of several problems, [problem][value][warp].
+    constexpr bool PAIRS = MODE == MODE_F32 || MODE == MODE_TC;
+    constexpr int NW = TH / 32;
+    constexpr int RED = PAIRS && MAXP * NW > TH ? MAXP * 3 * NW : 3 * TH;
+    __shared__ double s_red[RED];
+    __shared__ int s_fail;
+    // Kept in shared memory so that no register holds them through an element
+    // phase, which needs every register that it can get: the step, and each
+    // warp's copy of the next problem's start.
+    __shared__ unsigned s_step, s_rot[NW];
+    const int np = prm.nprob;
+    SyncState *sync = prm.sync;
+    const unsigned grid = gridDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int p = threadIdx.x; p < np; p += TH) {
+        PState S;
+        memset(&S, 0, sizeof(S));
+        const ProbDesc &P = prm.prob[p];
+        // (the sum of b that JACGS makes is only needed to remove its mean)
+        S.phase = !P.jac_cached ? PH_JAC : P.singular ? PH_JACGS : PH_AX0;
+        s_st[p] = S;
+    }
+    if (threadIdx.x == 0) s_step = 0;
+    __syncthreads();
+    auto partials = [&] { return prm.partials + (size_t)(s_step & 1) * MAXP * 3 * grid; };
+
+    for (;;) {
+        // ---- this CTA's share of every problem's phase; its sums are published
+        bool all_done = true;
+        int layout = -1;  // how the last element phase laid the shared memory out
+        if (MAXP > 1 && lane == 0) s_rot[warp] = 0;
+        for (int o = 0; o < (MAXP == 1 ? 1 : np); ++o) {
+            const int p = MAXP == 1 ? 0 : prm.order[o];
+            const PState &S = s_st[p];
+            if (S.phase == PH_DONE) continue;
+            all_done = false;
+            const ProbDesc &P = prm.prob[p];
+            const int kind = phase_kind(S.phase);
+            if (MAXP > 1 && kind == KIND_ELEM) {
+                const int want = P.n * 16 + P.tc * 2 + (S.phase == PH_AX0);
+                if (layout >= 0 && layout != want) __syncthreads();
+                layout = want;
+            }
+            double v[3] = {0.0, 0.0, 0.0};
+            dfacc d[2] = {{0.f, 0.f}, {0.f, 0.f}};
+            if (kind != KIND_LOCAL) {
+                if (MAXP > 1) __syncwarp();
+                const Deal deal = {blockIdx.x, grid, MAXP == 1 ? 0u : s_rot[warp]};
+                const unsigned rot = PhaseDispatch<MODE, TH, NPs...>::run(P, S, kind, deal, smem, v, d);
+                if (MAXP > 1) {
+                    __syncwarp();
+                    if (lane == 0) s_rot[warp] = rot;
+                }
+            } else if (S.phase != PH_JAC || !P.jac_shared) {
+                for (unsigned q = blockIdx.x * TH + threadIdx.x; q < (unsigned)P.nL; q += grid * TH)
+                    local_item(P, S, S.phase, q, v);
+            }
+            const int nv = phase_nvals(s_st[p].phase);
+            if (nv == 0) continue;
+            if (PAIRS && MAXP > 1 && np > 1) {
+                // no barrier between the problems of an FP32 launch: a warp sums
+                // its lanes' pairs and leaves the values for the end of the step
+                const bool pairs = phase_pairs(s_st[p].phase);
+#pragma unroll
+                for (int k = 0; k < 2; ++k)
+                    if (k < nv) {
+                        const double t = pairs ? dfacc_value(warp_sum_pair(d[k])) : warp_sum(v[k]);
+                        if (lane == 0) s_red[(p * 3 + k) * NW + warp] = t;
+                    }
+                continue;
+            }
+            // one warp per value sums the CTA's TH in a fixed order
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                if (k < nv)
+                    s_red[k * TH + threadIdx.x] =
+                        PAIRS && k < 2 && phase_pairs(s_st[p].phase) ? dfacc_value(d[k]) : v[k];
+            __syncthreads();
+            if ((int)warp < nv) {
+                double t[NW];
+#pragma unroll
+                for (int j = 0; j < NW; ++j) t[j] = s_red[warp * TH + lane + 32 * j];
+                const double s = warp_sum(tree_sum(t));
+                if (lane == 0) partials()[(size_t)(p * 3 + warp) * grid + blockIdx.x] = s;
+            }
+            if (np > 1) __syncthreads();  // (s_red is written again)
+        }
+        if (all_done) break;
+
+        if (PAIRS && MAXP > 1 && np > 1) {
+            __syncthreads();
+            for (int pk = warp; pk < np * 3; pk += NW) {
+                const int p = pk / 3, k = pk - 3 * p;
+                if (k < phase_nvals(s_st[p].phase)) {
+                    const double t = warp_sum((int)lane < NW ? s_red[pk * NW + lane] : 0.0);
+                    if (lane == 0) partials()[(size_t)pk * grid + blockIdx.x] = t;
+                }
+            }
+        }
+
+        // ---- grid barrier: the count reaches (steps so far + 1) * grid
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            s_fail = 0;
+            red_release_add_u32(&sync->count, 1u);
+            const unsigned goal = (s_step + 1u) * grid;
+            const unsigned long long t0 = sem_globaltimer();
+            for (unsigned spin = 0; (int)(ld_acquire_u32(&sync->count) - goal) < 0; ++spin) {
+                if ((spin & 15u) != 0u) continue;
+                if (((volatile int *)&sync->err)[0]) {
+                    s_fail = 1;
+                    break;
+                }
+                if ((long long)(sem_globaltimer() - t0) > prm.timeout_ns) {
+                    atomicExch(&sync->err, SEM_ERR_TIMEOUT);
+                    s_fail = 1;
+                    break;
+                }
+            }
+        }
+        __syncthreads();
+        if (s_fail) break;
+
+        // ---- every CTA sums the partials in the same fixed order, one warp a value
+        // (eight loads in flight a lane: one at a time their latencies added up to
+        // 3 us a phase)
+        for (int pk = warp; pk < np * 3; pk += NW) {
+            const int p = pk / 3, k = pk - 3 * p;
+            if (k < phase_nvals(s_st[p].phase)) {
+                const double *src = partials() + (size_t)pk * grid;
+                double s = 0.0;
+                for (unsigned b0 = 0; b0 < grid; b0 += 256) {
+                    double t[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const unsigned b = b0 + 32 * j + lane;
+                        t[j] = b < grid ? __ldcg(src + b) : 0.0;
+                    }
+                    s += tree_sum(t);
+                }
+                s = warp_sum(s);
+                if (lane == 0) s_sum[p][k] = s;
+            }
+        }
+        __syncthreads();
+        for (int p = threadIdx.x; p < np; p += TH)
+            if (s_st[p].phase != PH_DONE) advance<MAXP>(prm, prm.prob[p], s_st[p], s_sum[p]);
+        if (threadIdx.x == 0) s_step += 1;
+        __syncthreads();
+    }
+    // the final states, once (after a time-out: the states at the last whole step)
+    __syncthreads();
+    if (blockIdx.x == 0)
+        for (int p = threadIdx.x; p < np; p += TH) prm.st[p] = s_st[p];
+}
+
+// Host launcher (cooperative, grid sized for co-residency and no larger than
+// the element and unique phases can use).
+template <int MAXP, int MODE, int... NPs>
+int launch_solve(const SolveParams<MAXP> &prm, int num_sms, cudaStream_t s)
+{
+    constexpr int TH = solve_threads<MAXP, MODE, NPs...>();
+    auto kern = k_solve<MAXP, MODE, TH, NPs...>;
+    const size_t smem = SmemMax<MODE, TH, NPs...>::v;
     static std::atomic<unsigned> attr{0};
     SEM_CUDA(sem_smem_attr(kern, smem, attr));
     int per_sm = 0;
-    SEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SEM_SOLVE_THREADS, smem));
+    SEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TH, smem));
     if (per_sm < 1) return SEM_ERR_ARG;
+    long long most = 0;
+    for (int p = 0; p < prm.nprob; ++p) most += PhaseDispatch<MODE, TH, NPs...>::portions(prm.prob[p]);
     long long grid = (long long)per_sm * num_sms;
-    if (grid > max_items) grid = max_items;
+    const long long fit = prm.partials_cap / (2 * MAXP * 3);
+    if (grid > most) grid = most;
+    if (grid > fit) grid = fit;
     if (grid < 1) grid = 1;
     void *args[] = {(void *)&prm};
-    SEM_CUDA(cudaLaunchCooperativeKernel((const void *)kern, dim3((unsigned)grid),
-                                         dim3(SEM_SOLVE_THREADS), args, smem, s));
+    SEM_CUDA(cudaLaunchCooperativeKernel((const void *)kern, dim3((unsigned)grid), dim3(TH), args, smem, s));
     return SEM_OK;
 }
 

@@ -38,10 +38,8 @@ int sem_run_geometry(sem_ctx *c, double *xyz, bool with_jinv, cudaStream_t s);
 int sem_alloc_ws(sem_ctx *c, int slot);
 int sem_dssum_dev(sem_ctx *c, void *u, sem_dtype dt, cudaStream_t s);
 int sem_ax_dev(sem_ctx *c, const void *u, void *w, double h1, double h2, sem_dtype dt, cudaStream_t s);
-int sem_pcg_solve_dev(sem_ctx *c, int slot, const double *b, double *x, double h1, double h2,
-                      const sem_solve_opts &o, cudaStream_t s);
 int sem_pcg_solve_dev_batch(sem_ctx *c, int np, const double *const *b, double *const *x, double h1,
-                            double h2, const sem_solve_opts &o, cudaStream_t s, int slot0);
+                            double h2, const sem_solve_opts &o, cudaStream_t s, int slot0, bool ordered);
 const void *sem_solve_state_ptr(const sem_ctx *c, int p, int *iters_off, int *status_off);
 int sem_gmres_solve_dev(sem_hsmg *H, int precond, const double *b_in, double *x, const sem_solve_opts &o,
                         int m, sem_solve_info *info, cudaStream_t s, int x_zero);
@@ -943,7 +941,7 @@ static void proj_free(sem_tgv *T);
 // convergence status goes to the step's log, like the persistent solver's).
 static int pressure_solve(sem_tgv *T, const double *b, double *x, int x_zero, cudaStream_t s)
 {
-    if (!T->psolver) return sem_pcg_solve_dev(T->c, 4, b, x, 1.0, 0.0, T->po, s);
+    if (!T->psolver) return sem_pcg_solve_dev_batch(T->c, 1, &b, &x, 1.0, 0.0, T->po, s, 4, true);
     const int rc = sem_gmres_solve_dev(T->hsmg, 1, b, x, T->po, T->prestart, &T->pinfo, s, x_zero);
     if (rc == SEM_OK || rc == SEM_ERR_NOT_CONVERGED || rc == SEM_ERR_BREAKDOWN) return SEM_OK;
     return rc;
@@ -1037,7 +1035,7 @@ static int step_once(sem_tgv *T, int q, cudaStream_t s)
     const double *bb[3] = {T->rhs[0], T->rhs[1], T->rhs[2]};
     double *xx[3] = {T->unew[0], T->unew[1], T->unew[2]};
     // (workspace slots 5-7; slot 4 keeps the pressure's Jacobi inverse between steps)
-    rc = sem_pcg_solve_dev_batch(c, 3, bb, xx, T->nu, k.b0 / T->dt, T->vo, s, 5);
+    rc = sem_pcg_solve_dev_batch(c, 3, bb, xx, T->nu, k.b0 / T->dt, T->vo, s, 5, !T->psolver);
     if (rc) return rc;
     k_tgv_log_iters<<<1, 32, 0, s>>>(st0, stride, io, so, serr, 1, 3, T->dev, T->log, 0);
     SEM_CHECK_LAUNCH();

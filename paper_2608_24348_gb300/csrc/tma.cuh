@@ -93,3 +93,14 @@ __device__ __forceinline__ void l2_prefetch_span(const void *base, int64_t begin
     const uintptr_t e = ((uintptr_t)base + (uintptr_t)end) & ~(uintptr_t)15;
     if (e > b) bulk_prefetch_l2((const void *)b, (uint32_t)(e - b));
 }
+
+// Asynchronous copies of one value (8 or 4 bytes) into shared memory.
+__device__ __forceinline__ void cp_async8(double *dst, const double *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async4(float *dst, const float *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
