@@ -134,6 +134,9 @@ constexpr int dfeo_group_sync()
 
 int sem_launch_ax_bfp(const sem_ctx *c, int variant, const double *u, double *w, double h1,
                       double h2, cudaStream_t s);  // ax_bfp.cu
+int sem_launch_ax_dfl(const sem_ctx *c, const double *u, double *w, double h1, double h2,
+                      cudaStream_t s);  // ax_dfl.cu
+int sem_make_dfl_tabs(sem_ctx *c);
 
 template <int NP>
 static int launch_df(const sem_ctx *c, const double *u, double *w, double h1, double h2,
@@ -173,10 +176,22 @@ static int launch_df(const sem_ctx *c, const double *u, double *w, double h1, do
     return SEM_OK;
 }
 
+int sem_launch_ax_df_columns(const sem_ctx *c, const double *u, double *w, double h1, double h2,
+                             cudaStream_t s)
+{
+    SEM_DISPATCH_NP(c->n, return launch_df<NP>(c, u, w, h1, h2, s));
+    return SEM_ERR_ARG;
+}
+
 int sem_launch_ax_df(const sem_ctx *c, const double *u, double *w, double h1, double h2,
                      cudaStream_t s)
 {
-    SEM_DISPATCH_NP(c->n, return launch_df<NP>(c, u, w, h1, h2, s));
+    SEM_DISPATCH_NP(c->n, {
+        if constexpr (NP % 2 == 1 && NP <= 11)
+            return sem_launch_ax_dfl(c, u, w, h1, h2, s);
+        else
+            return launch_df<NP>(c, u, w, h1, h2, s);
+    });
     return SEM_ERR_ARG;
 }
 
@@ -202,6 +217,8 @@ int sem_make_geo_df(sem_ctx *c)
         ax_bfp_tables(c->n, c->hD, T);
         c->bfp_tabs = T;
     }
+    const int rc = sem_make_dfl_tabs(c);
+    if (rc) return rc;
     dfp hD[SEM_NPMAX * SEM_NPMAX];
     for (int t = 0; t < c->n * c->n; ++t) {
         const float h = (float)c->hD[t];

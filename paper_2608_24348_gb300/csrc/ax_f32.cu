@@ -7,8 +7,10 @@
 // computes group g the copy of its next group is in flight, so the kernel
 // keeps enough bytes moving without needing many resident warps.
 #include <stdint.h>
+#include <string.h>
 
 #include "ax_launch.cuh"
+#include "ax_line32.cuh"
 #include "tma.cuh"
 
 // Tile shape of the staged kernel: about TH threads per block (whole
@@ -132,7 +134,84 @@ static int launch_tma(const sem_ctx *c, const float *u, float *w, float h1, floa
     }
 }
 
-// Variants of the FP32 operator (see sem_tune_ax): 0 direct loads, 1 staged
+// The line operator (ax_line32.cuh): 256 threads, the next element group's u
+// copied into shared memory by asynchronous copies (every thread its own
+// column), groups synchronised by themselves.  Bound: FP32 issue and HBM alike
+// (36 bytes a node); 0.1055 ms at 32^3 elements, N = 7 (0.1209 by the staged form
+// below, 0.089 the bytes alone).
+template <int NP>
+struct L32Shape {
+    static constexpr int NP2 = NP * NP;
+    static constexpr int GT = NP <= 4 ? 32 : NP == 8 ? 64 : (NP == 5 || NP == 6 || NP == 10 || NP == 11) ? 128 : 256;
+    static constexpr int GE = GT / NP2, NG = 256 / GT, NE = NG * GE;
+    static constexpr size_t SMEM = sizeof(float) * ((size_t)NE * 3 * Line32Cfg<NP>::SLAB + NP * 256);
+};
+
+template <int NP>
+__global__ void __launch_bounds__(256, NP <= 10 ? 4 : 1)
+    k_ax_line32(const float *__restrict__ u, float *__restrict__ w, const float *__restrict__ geo,
+                const __grid_constant__ LineTab32 T, float h1, float h2, int64_t E)
+{
+    using S = L32Shape<NP>;
+    constexpr int NP2 = NP * NP, NP3 = NP2 * NP;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int grp = threadIdx.x / S::GT, lt = threadIdx.x - grp * S::GT;
+    const int ge = lt / NP2 < S::GE ? lt / NP2 : 0, tid = lt / NP2 < S::GE ? lt - ge * NP2 : -1;
+    float *slab = reinterpret_cast<float *>(smem) + (size_t)(grp * S::GE + ge) * 3 * Line32Cfg<NP>::SLAB;
+    float *su = reinterpret_cast<float *>(smem) + (size_t)S::NE * 3 * Line32Cfg<NP>::SLAB + threadIdx.x;
+    auto sync = [&] {
+        if constexpr (S::GT == 256)
+            __syncthreads();
+        else if constexpr (S::GT == 32)
+            __syncwarp();
+        else
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(S::GT) : "memory");
+    };
+    const int64_t groups = (E + S::GE - 1) / S::GE, stride = (int64_t)gridDim.x * S::NG;
+    auto fetch = [&](int64_t g) {
+        const int64_t e = g * S::GE + ge;
+        if (g < groups && tid >= 0 && e < E) {
+#pragma unroll
+            for (int k = 0; k < NP; ++k) cp_async4(su + k * 256, u + e * NP3 + k * NP2 + tid);
+        }
+    };
+    int64_t g = (int64_t)grp * gridDim.x + blockIdx.x;
+    fetch(g);
+    for (; g < groups; g += stride) {
+        const int64_t e0 = g * S::GE, e = e0 + ge;
+        const bool active = tid >= 0 && e < E;
+        if (lt == 0)
+            l2_prefetch_span(geo, e0 * 7 * NP3 * 4, (e0 + S::GE < E ? e0 + S::GE : E) * 7 * NP3 * 4);
+        float *we = w + (active ? e : 0) * NP3 + tid;
+        cp_async_wait_all();
+        auto load = [&](int k) { return su[k * 256]; };
+        auto store = [&](int k, float v, float) { we[k * NP2] = v; };
+        ax_line32_element<NP>(load, store, geo + (active ? e : 0) * 7 * NP3, h1, h2, T, slab, tid, active,
+                              [&] { fetch(g + stride); }, sync);
+    }
+}
+
+template <int NP>
+static int launch_line32(const sem_ctx *c, const float *u, float *w, float h1, float h2, cudaStream_t s)
+{
+    using S = L32Shape<NP>;
+    static std::atomic<unsigned> attr{0};
+    SEM_CUDA(sem_smem_attr(k_ax_line32<NP>, S::SMEM, attr));
+    int per_sm = 0;
+    SEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ax_line32<NP>, 256, S::SMEM));
+    if (per_sm < 1) return SEM_ERR_ARG;
+    const int64_t groups = sem_ceil_div(c->E, S::GE);
+    int64_t grid = (int64_t)per_sm * c->num_sms;
+    if (grid > groups) grid = groups;
+    LineTab32 T;
+    memset(&T, 0, sizeof(T));
+    for (int t = 0; t < NP * NP; ++t) T.d[t] = (float)c->hD[t];
+    k_ax_line32<NP><<<(unsigned)grid, 256, S::SMEM, s>>>(u, w, c->geo32, T, h1, h2, c->E);
+    SEM_CHECK_LAUNCH();
+    return SEM_OK;
+}
+
+// Variants of the FP32 operator (see sem_tune_ax): 0 whole lines, 1 staged
 // 256 threads x 2 stages, 2 staged 128 threads x 3 stages.
 int sem_launch_ax_f32_variant(const sem_ctx *c, int variant, const float *u, float *w, float h1,
                               float h2, cudaStream_t s)
@@ -152,8 +231,28 @@ int sem_launch_ax_f32_variant(const sem_ctx *c, int variant, const float *u, flo
             default: break;
         }
     }
-    const float *tab = c->tab32 + 2 * n;
-    const float *geo = c->geo32;
-    SEM_DISPATCH_NP(n, return launch_ax<NP, float>(c, u, w, geo, tab, h1, h2, s));
+    SEM_DISPATCH_NP(n, return launch_line32<NP>(c, u, w, h1, h2, s));
     return SEM_ERR_ARG;
+}
+
+// The operator with the three directions' products of a node summed in turn (the
+// order of ax_element), whatever variant is in force.  The multigrid V-cycle uses
+// it: its FP32 rounding passes through GMRES into the solution at the level of
+// the pressure tolerance, so a change of summation order there would change the
+// stepper's results by far more than FP64 rounding.
+int sem_launch_ax_f32_columns(const sem_ctx *c, const float *u, float *w, float h1, float h2, cudaStream_t s)
+{
+    const float *tab = c->tab32 + 2 * c->n;
+    switch (c->n) {
+        case 4: return launch_tma<4, 256, 2>(c, u, w, h1, h2, s);
+        case 6: return launch_tma<6, 256, 2>(c, u, w, h1, h2, s);
+        case 8: return launch_tma<8, 128, 3>(c, u, w, h1, h2, s);
+        case 10: return launch_tma<10, 128, 3>(c, u, w, h1, h2, s);
+        case 2: return launch_ax<2, float>(c, u, w, c->geo32, tab, h1, h2, s);
+        case 3: return launch_ax<3, float>(c, u, w, c->geo32, tab, h1, h2, s);
+        case 5: return launch_ax<5, float>(c, u, w, c->geo32, tab, h1, h2, s);
+        case 7: return launch_ax<7, float>(c, u, w, c->geo32, tab, h1, h2, s);
+        case 9: return launch_ax<9, float>(c, u, w, c->geo32, tab, h1, h2, s);
+        default: return SEM_ERR_ARG;
+    }
 }

@@ -34,7 +34,7 @@ void sem_note_cuda_error(cudaError_t e, const char *where);
 
 // One PCG workspace: the vectors of a solve (FP64 and FP32 sets).
 struct sem_ws {
-    double *r, *p, *w, *minv, *b;   // FP64 E-vectors (b: mean-free scratch copy is not kept)
+    double *r, *p, *w, *minv, *b;   // FP64 E-vectors (b: the sum of the corrections of a solve)
     float *r32, *p32, *w32, *d32, *minv32;
     // minv (and minv32) hold the Jacobi inverse of (jac_h1, jac_h2) when jac_ok (jac32_ok)
     double jac_h1, jac_h2;
@@ -60,6 +60,7 @@ struct sem_ctx {
     void *tabdf;       // float pairs of D
     void *tabdfeo;     // float pairs of the folded half tables (even N+1)
     void *bfp_tabs;    // host copy of the block-floating-point kernel's tables (even N+1)
+    void *dfl_tabs;    // host copy of the float-pair line kernel's tables (odd N+1 <= 11)
     double *vert;      // device vertex grid [(nelz+1)(nely+1)(nelx+1)][3]
     double *jinv64;    // [E][9][n^3] dr_a/dx_c at a*3+c (allocated by the stepper)
     float *jinv32;

@@ -34,6 +34,8 @@
 
 int sem_dssum_dev(sem_ctx *c, void *u, sem_dtype dt, cudaStream_t s);
 int sem_ax_dev(sem_ctx *c, const void *u, void *w, double h1, double h2, sem_dtype dt, cudaStream_t s);
+int sem_ax_dev_columns(sem_ctx *c, const double *u, double *w, double h1, double h2, cudaStream_t s);
+int sem_launch_ax_f32_columns(const sem_ctx *c, const float *u, float *w, float h1, float h2, cudaStream_t s);
 int sem_pcg_solve_dev(sem_ctx *c, int slot, const double *b, double *x, double h1, double h2,
                       const sem_solve_opts &o, cudaStream_t s);
 
@@ -690,7 +692,11 @@ static int hs_cycle(sem_hsmg *H, int l, T *r, T *z, cudaStream_t s)
     HsLevel &C = H->L[l + 1];
     T *w = (T *)L.w;
     if ((rc = hs_fdm<T>(H, L, r, z, s))) return rc;
-    if ((rc = sem_ax_dev(c, z, w, H->h1, H->h2, H->dt, s))) return rc;
+    if constexpr (sizeof(T) == 4)
+        rc = sem_launch_ax_f32_columns(c, z, w, (float)H->h1, (float)H->h2, s);
+    else
+        rc = sem_ax_dev_columns(c, z, w, H->h1, H->h2, s);
+    if (rc) return rc;
     if ((rc = sem_dssum_dev(c, w, H->dt, s))) return rc;
     k_hs_sub<T><<<hs_grid(n), 256, 0, s>>>(w, r, n);
     SEM_CHECK_LAUNCH();
@@ -789,7 +795,8 @@ static int hs_ensure(sem_hsmg *H, int m)
 static int hs_op(sem_hsmg *H, const double *x, double *y, bool tight, cudaStream_t s)
 {
     sem_ctx *c = H->L[0].c;
-    int rc = sem_ax_dev(c, x, y, H->h1, H->h2, tight ? SEM_F64_NATIVE : SEM_F64, s);
+    int rc = tight ? sem_ax_dev(c, x, y, H->h1, H->h2, SEM_F64_NATIVE, s)
+                   : sem_ax_dev_columns(c, x, y, H->h1, H->h2, s);
     if (rc) return rc;
     return sem_dssum_dev(c, y, SEM_F64, s);
 }

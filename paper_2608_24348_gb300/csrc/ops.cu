@@ -14,6 +14,8 @@ int sem_launch_ax_f64(const sem_ctx *c, const double *u, double *w, double h1, d
                       cudaStream_t s);  // ax_f64.cu
 int sem_launch_ax_f32_variant(const sem_ctx *c, int variant, const float *u, float *w, float h1,
                               float h2, cudaStream_t s);  // ax_f32.cu
+int sem_launch_ax_df_columns(const sem_ctx *c, const double *u, double *w, double h1, double h2,
+                             cudaStream_t s);
 int sem_launch_ax_df(const sem_ctx *c, const double *u, double *w, double h1, double h2,
                      cudaStream_t s);   // ax_df.cu
 
@@ -32,8 +34,11 @@ static int sem_nvariant(sem_dtype dt) { return dt == SEM_F64 ? 11 : dt == SEM_F3
 static int g_variant[SEM_NMAX + 1][5];  // 0 = not set -> built-in default
 static int g_variant_set[SEM_NMAX + 1][5];
 
-// Built-in defaults from measurements on GB300.  FP32: staged 128 x 3 for
-// N = 7 and 9, staged 256 x 2 for N = 3 and 5, direct loads otherwise.
+// Built-in defaults from measurements on GB300.  FP32: the bulk-copy staged form
+// for N = 3 (128 x 3: 0.0471 ms at 48^3 elements against 0.0505 by whole lines)
+// and N = 5 (256 x 2: 0.0860 against 0.1044 at 40^3); whole lines otherwise
+// (N = 7: 0.1055 against 0.1209 staged at 32^3; N = 9: 0.1376 against 0.1471 at
+// 24^3).
 // FP64-accurate: the block-floating-point kernel with u staged, one element
 // per block (0.27 ms against 0.43 ms for the float-pair folded kernel at 32^3,
 // N = 7), for odd N <= 11 (even N+1 <= 12); the float-pair kernels otherwise.
@@ -41,9 +46,7 @@ static int default_variant(int N, sem_dtype dt)
 {
     if (dt == SEM_F64) return (N % 2 == 1 && N <= 11) ? 8 : 0;
     if (dt != SEM_F32) return 0;
-    if (N == 7 || N == 9) return 2;
-    if (N == 3 || N == 5) return 1;
-    return 0;
+    return N == 3 ? 2 : N == 5 ? 1 : 0;
 }
 
 int sem_ax_variant(int N, sem_dtype dt)
@@ -74,6 +77,16 @@ GsDesc sem_gs_desc(const sem_ctx *c)
     d.px = c->periodic[0]; d.py = c->periodic[1]; d.pz = c->periodic[2];
     d.nG = c->nG;
     return d;
+}
+
+// The operator of flexible GMRES and of the projection space: at odd N+1 in the
+// summation order of a column a thread (ax_df.cuh), 212 us a launch against 157
+// by whole lines (4.7 M nodes, N = 8).  A loosely stopped GMRES follows the last
+// bits of its operator: by lines the pressure of a Taylor-Green step moved by
+// 3e-9 of itself, 1000 times what the rest of the step's arithmetic moves it.
+int sem_ax_dev_columns(sem_ctx *c, const double *u, double *w, double h1, double h2, cudaStream_t s)
+{
+    return c->E == 0 ? SEM_OK : sem_launch_ax_df_columns(c, u, w, h1, h2, s);
 }
 
 // Device-pointer form (used by the stepper as well).

@@ -37,7 +37,7 @@ GsDesc sem_gs_desc(const sem_ctx *c);
 int sem_run_geometry(sem_ctx *c, double *xyz, bool with_jinv, cudaStream_t s);
 int sem_alloc_ws(sem_ctx *c, int slot);
 int sem_dssum_dev(sem_ctx *c, void *u, sem_dtype dt, cudaStream_t s);
-int sem_ax_dev(sem_ctx *c, const void *u, void *w, double h1, double h2, sem_dtype dt, cudaStream_t s);
+int sem_ax_dev_columns(sem_ctx *c, const double *u, double *w, double h1, double h2, cudaStream_t s);
 int sem_pcg_solve_dev_batch(sem_ctx *c, int np, const double *const *b, double *const *x, double h1,
                             double h2, const sem_solve_opts &o, cudaStream_t s, int slot0, bool ordered);
 const void *sem_solve_state_ptr(const sem_ctx *c, int p, int *iters_off, int *status_off);
@@ -1407,7 +1407,7 @@ static int pressure_projected(sem_tgv *T, cudaStream_t s)
     k_proj_restart<<<1, 1, 0, s>>>(T->pint, T->proj_max);
     k_copy_if<<<g, 256, 0, s>>>(T->pdx, T->p, restart, n);
     SEM_CHECK_LAUNCH();
-    if ((rc = sem_ax_dev(c, T->pdx, T->padx, 1.0, 0.0, SEM_F64, s))) return rc;
+    if ((rc = sem_ax_dev_columns(c, T->pdx, T->padx, 1.0, 0.0, s))) return rc;
     if ((rc = sem_dssum_dev(c, T->padx, SEM_F64, s))) return rc;
     k_proj_dot<<<TGV_PBLK, 256, 0, s>>>(T->pdx, T->padx, T->pw, one, n, T->ppart);
     k_proj_dot_final<<<1, 1024, 0, s>>>(T->ppart, one, nrm);
