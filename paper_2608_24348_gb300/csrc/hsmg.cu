@@ -31,17 +31,21 @@
 #include <vector>
 
 #include "common.cuh"
+#include "uniq.cuh"
 
+GsDesc sem_gs_desc(const sem_ctx *c);  // ops.cu
 int sem_dssum_dev(sem_ctx *c, void *u, sem_dtype dt, cudaStream_t s);
 int sem_ax_dev(sem_ctx *c, const void *u, void *w, double h1, double h2, sem_dtype dt, cudaStream_t s);
 int sem_ax_dev_columns(sem_ctx *c, const double *u, double *w, double h1, double h2, cudaStream_t s);
-int sem_launch_ax_f32_columns(const sem_ctx *c, const float *u, float *w, float h1, float h2, cudaStream_t s);
+int sem_launch_ax_f32_columns(const sem_ctx *c, const float *u, float *w, float h1, float h2,
+                              cudaStream_t s);  // ax_f32.cu
 int sem_pcg_solve_dev(sem_ctx *c, int slot, const double *b, double *x, double h1, double h2,
                       const sem_solve_opts &o, cudaStream_t s);
 
 #define HS_MAXLEV 3
 #define HS_DOT_BLOCKS 1216  // 8 x 152 SMs; fixed so that the sums are deterministic
-#define HS_DOT_K 8          // inner products per pass over the data
+#define HS_DOT_K 8          // inner products a block forms in one pass over its nodes
+#define HS_DOT_MAX 72       // values of one call: up to 64 vectors, <w,w>, <w,1>, <w,w> after a pass
 
 // ---------------------------------------------------------------------------
 // Host: 1-D factors of the local solves
@@ -146,90 +150,153 @@ static double hs_edge_len(const sem_ctx *c, const double *vert, int ex, int ey, 
 // Device kernels
 // ---------------------------------------------------------------------------
 
-// Fast-diagonalisation local solves of every element, weighted by 1/mult:
+// Fast-diagonalisation local solves, weighted by 1/mult:
 // z_e = (1/mult) (S x S x S) diag(1/(h1 sum lam + h2)) (S x S x S)^T r_e.
-// fidx[e*3 + a] selects element e's factor set of direction a.
+// fidx[e*3 + a] selects element e's factor set of direction a.  TI: type of r
+// (the finest level's residual is FP64 whatever the V-cycle's precision).
+//
+// Bound: latency and shared-memory traffic (12 bytes a node in FP32, much of it
+// in L2).  Every 1-D product takes a whole line into registers and multiplies
+// it by the factor matrix read as broadcast vectors; the two z products, with
+// the diagonal between them, stay in registers.  A node at a time, both
+// operands of every product read from shared memory: 35.0 us at 16^3 elements,
+// N = 7, FP32, now 20.0; 12.0 and 5.5 at N = 3.
 template <int NP, typename T>
-__global__ void k_hs_fdm(const T *__restrict__ r, T *__restrict__ z, const T *__restrict__ Sf,
-                         const T *__restrict__ lamf, const int *__restrict__ fidx,
-                         const T *__restrict__ imult, T h1, T h2, int64_t E)
+struct FdmCfg {
+    static constexpr int N2 = NP * NP, N3 = N2 * NP;
+    static constexpr int NE = 256 / N2, THREADS = NE * N2;
+    static constexpr bool V4 = sizeof(T) == 4 && NP % 4 == 0;
+    // row and plane strides of a slab (as in ax_line32.cuh)
+    static constexpr int LS = V4 ? (NP % 8 == 0 ? NP + 4 : NP) : (NP | 1);
+    static constexpr int KS = NP * LS + (V4 ? (NP % 8 == 0 ? 8 : 4) : 0);
+    static constexpr int SLAB = NP * KS, FAC = 3 * N2 + (3 * NP + 3) / 4 * 4;
+};
+
+// y_i = sum_l S[l][i] x_l (TR) or sum_l S[i][l] x_l, in order of l.
+template <int NP, bool TR, typename T>
+__device__ __forceinline__ void fdm_mul(const T *S, const T (&x)[NP], T (&y)[NP])
 {
-    constexpr int N2 = NP * NP, N3 = N2 * NP;
-    __shared__ T sS[3][N2], sl[3][NP], su[N3], st[N3];
-    for (int64_t e = blockIdx.x; e < E; e += gridDim.x) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < 3 * N2; t += blockDim.x) {
-            const int a = t / N2, q = t - a * N2;
-            sS[a][q] = Sf[(size_t)fidx[e * 3 + a] * N2 + q];
-        }
-        for (int t = threadIdx.x; t < 3 * NP; t += blockDim.x) {
-            const int a = t / NP, q = t - a * NP;
-            sl[a][q] = lamf[(size_t)fidx[e * 3 + a] * NP + q];
-        }
-        const int64_t off = e * N3;
-        for (int t = threadIdx.x; t < N3; t += blockDim.x) su[t] = r[off + t];
-        __syncthreads();
-        // forward: (S^T u)_i = sum_l S[l][i] u_l along x, then y, then z
-        for (int t = threadIdx.x; t < N3; t += blockDim.x) {
-            const int i = t % NP, jk = t - i;
-            T s = 0;
 #pragma unroll
-            for (int l = 0; l < NP; ++l) s = fma(sS[0][l * NP + i], su[jk + l], s);
-            st[t] = s;
+    for (int i = 0; i < NP; ++i) y[i] = T(0);
+    if constexpr (sizeof(T) == 4 && NP % 4 == 0) {
+#pragma unroll
+        for (int a = 0; a < NP; ++a)
+#pragma unroll
+            for (int b = 0; b < NP; b += 4) {
+                const float4 s = *reinterpret_cast<const float4 *>(S + a * NP + b);
+                const T sv[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (TR) y[b + q] = fma(sv[q], x[a], y[b + q]);
+                    else y[a] = fma(sv[q], x[b + q], y[a]);
+                }
+            }
+    } else {
+#pragma unroll
+        for (int a = 0; a < NP; ++a)
+#pragma unroll
+            for (int b = 0; b < NP; ++b) {
+                if (TR) y[b] = fma(S[a * NP + b], x[a], y[b]);
+                else y[a] = fma(S[a * NP + b], x[b], y[a]);
+            }
+    }
+}
+
+template <int NP, typename T, typename TI>
+__global__ void __launch_bounds__(FdmCfg<NP, T>::THREADS)
+    k_hs_fdm(const TI *__restrict__ r, T *__restrict__ z, const T *__restrict__ Sf, const T *__restrict__ lamf,
+             const int *__restrict__ fidx, const T *__restrict__ imult, T h1, T h2, int64_t E)
+{
+    using C = FdmCfg<NP, T>;
+    constexpr int N2 = C::N2, N3 = C::N3, LS = C::LS, KS = C::KS;
+    __shared__ __align__(16) T s_slab[C::NE][C::SLAB];
+    __shared__ __align__(16) T s_fac[C::NE][C::FAC];
+    const int ge = threadIdx.x / N2, tid = threadIdx.x - ge * N2;
+    const int i = tid % NP, j = tid / NP;
+    T *su = s_slab[ge], *sS = s_fac[ge], *sl = sS + 3 * N2;
+    for (int64_t e0 = (int64_t)blockIdx.x * C::NE; e0 < E; e0 += (int64_t)gridDim.x * C::NE) {
+        const int64_t e = e0 + ge;
+        const bool active = e < E;
+        const int64_t off = (active ? e : 0) * N3;
+        __syncthreads();
+        if (active) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const int f = fidx[e * 3 + a];
+                sS[a * N2 + tid] = Sf[(size_t)f * N2 + tid];
+                if (tid < NP) sl[a * NP + tid] = lamf[(size_t)f * NP + tid];
+            }
+#pragma unroll
+            for (int k = 0; k < NP; ++k) su[k * KS + j * LS + i] = (T)r[off + k * N2 + tid];
         }
         __syncthreads();
-        for (int t = threadIdx.x; t < N3; t += blockDim.x) {
-            const int i = t % NP, j = (t / NP) % NP, k = t / N2;
-            T s = 0;
+        T x[NP], y[NP];
+        const int row = j * KS + i * LS, sln = j * KS + i;  // the lines (j' = i, k' = j) along x, (i' = i, k' = j) along y
+        if (active) {  // forward: S^T along x, then y, then z
 #pragma unroll
-            for (int l = 0; l < NP; ++l) s = fma(sS[1][l * NP + j], st[(k * NP + l) * NP + i], s);
-            su[t] = s;
+            for (int l = 0; l < NP; ++l) x[l] = su[row + l];
+            fdm_mul<NP, true>(sS, x, y);
+#pragma unroll
+            for (int l = 0; l < NP; ++l) su[row + l] = y[l];
         }
         __syncthreads();
-        for (int t = threadIdx.x; t < N3; t += blockDim.x) {
-            const int i = t % NP, j = (t / NP) % NP, k = t / N2;
-            T s = 0;
+        if (active) {
 #pragma unroll
-            for (int l = 0; l < NP; ++l) s = fma(sS[2][l * NP + k], su[(l * NP + j) * NP + i], s);
-            const T den = h1 * (sl[0][i] + sl[1][j] + sl[2][k]) + h2;
-            st[t] = den != T(0) ? s / den : T(0);
+            for (int l = 0; l < NP; ++l) x[l] = su[sln + l * LS];
+            fdm_mul<NP, true>(sS + N2, x, y);
+#pragma unroll
+            for (int l = 0; l < NP; ++l) su[sln + l * LS] = y[l];
         }
         __syncthreads();
-        // backward: (S u)_i = sum_l S[i][l] u_l along z, then y, then x
-        for (int t = threadIdx.x; t < N3; t += blockDim.x) {
-            const int i = t % NP, j = (t / NP) % NP, k = t / N2;
-            T s = 0;
+        if (active) {  // along z, the diagonal, and back along z
 #pragma unroll
-            for (int l = 0; l < NP; ++l) s = fma(sS[2][k * NP + l], st[(l * NP + j) * NP + i], s);
-            su[t] = s;
+            for (int l = 0; l < NP; ++l) x[l] = su[l * KS + j * LS + i];
+            fdm_mul<NP, true>(sS + 2 * N2, x, y);
+#pragma unroll
+            for (int k = 0; k < NP; ++k) {
+                const T den = h1 * (sl[i] + sl[NP + j] + sl[2 * NP + k]) + h2;
+                x[k] = den != T(0) ? y[k] / den : T(0);
+            }
+            fdm_mul<NP, false>(sS + 2 * N2, x, y);
+#pragma unroll
+            for (int l = 0; l < NP; ++l) su[l * KS + j * LS + i] = y[l];
         }
         __syncthreads();
-        for (int t = threadIdx.x; t < N3; t += blockDim.x) {
-            const int i = t % NP, j = (t / NP) % NP, k = t / N2;
-            T s = 0;
+        if (active) {  // backward: S along y, then x
 #pragma unroll
-            for (int l = 0; l < NP; ++l) s = fma(sS[1][j * NP + l], su[(k * NP + l) * NP + i], s);
-            st[t] = s;
+            for (int l = 0; l < NP; ++l) x[l] = su[sln + l * LS];
+            fdm_mul<NP, false>(sS + N2, x, y);
+#pragma unroll
+            for (int l = 0; l < NP; ++l) su[sln + l * LS] = y[l];
         }
         __syncthreads();
-        for (int t = threadIdx.x; t < N3; t += blockDim.x) {
-            const int i = t % NP, jk = t - i;
-            T s = 0;
+        if (active) {
 #pragma unroll
-            for (int l = 0; l < NP; ++l) s = fma(sS[0][i * NP + l], st[jk + l], s);
-            z[off + t] = s * imult[off + t];
+            for (int l = 0; l < NP; ++l) x[l] = su[row + l];
+            fdm_mul<NP, false>(sS, x, y);
+#pragma unroll
+            for (int l = 0; l < NP; ++l) su[row + l] = y[l];
         }
+        __syncthreads();
+        if (active)
+#pragma unroll
+            for (int k = 0; k < NP; ++k) {
+                const int64_t q = off + k * N2 + tid;
+                z[q] = su[k * KS + j * LS + i] * imult[q];
+            }
     }
 }
 
 // Grid transfer between levels of nf and nc points per direction (nc < nf <= 10).
-// prolong (dir 0): out_f = (J x J x J) in_c  (add != 0: out_f += ...);
-// restrict (dir 1): out_c = (J^T x J^T x J^T)(in_f / mult_f).
+// prolong (dir 0): out_f = base_f + (J x J x J) in_c;
+// restrict (dir 1): out_c = (J^T x J^T x J^T)((base_f - in_f) / mult_f).
 // J[f*nc + c] = l_c(xi_f), the coarse Lagrange basis at the fine GLL points.
+// The V-cycle's residual r - A z and its changes of precision (TI, TB, TO: types
+// of in, base and out; the arithmetic is T's) ride in these passes.
 #define HS_TMAX 10
-template <typename T>
-__global__ void k_hs_transfer(const T *__restrict__ in, T *__restrict__ out, const T *__restrict__ J,
-                              const T *__restrict__ imult_f, int nf, int nc, int dir, int add, int64_t E)
+template <typename T, typename TI, typename TB, typename TO>
+__global__ void k_hs_transfer(const TI *__restrict__ in, const TB *base, TO *out, const T *__restrict__ J,
+                              const T *__restrict__ imult_f, int nf, int nc, int dir, int64_t E)
 {
     __shared__ T sJ[HS_TMAX * HS_TMAX];
     __shared__ T sa[HS_TMAX * HS_TMAX * HS_TMAX], sb[HS_TMAX * HS_TMAX * HS_TMAX];
@@ -239,7 +306,7 @@ __global__ void k_hs_transfer(const T *__restrict__ in, T *__restrict__ out, con
     for (int64_t e = blockIdx.x; e < E; e += gridDim.x) {
         __syncthreads();
         for (int t = threadIdx.x; t < ni3; t += blockDim.x)
-            sa[t] = dir ? in[e * ni3 + t] * imult_f[e * ni3 + t] : in[e * ni3 + t];
+            sa[t] = dir ? ((T)base[e * ni3 + t] - (T)in[e * ni3 + t]) * imult_f[e * ni3 + t] : (T)in[e * ni3 + t];
         __syncthreads();
         // weight of input point a for output point o along one direction
         auto wgt = [&](int o, int a) -> T { return dir ? sJ[a * nc + o] : sJ[o * nc + a]; };
@@ -264,7 +331,7 @@ __global__ void k_hs_transfer(const T *__restrict__ in, T *__restrict__ out, con
             const int ji = t % (no * no), k = t / (no * no);
             T s = 0;
             for (int c = 0; c < ni; ++c) s = fma(wgt(k, c), sa[c * no * no + ji], s);
-            out[e * no3 + t] = add ? out[e * no3 + t] + s : s;
+            out[e * no3 + t] = (TO)(dir ? s : (T)base[e * no3 + t] + s);
         }
     }
 }
@@ -276,11 +343,23 @@ __global__ void k_hs_sub(T *__restrict__ w, const T *__restrict__ r, int64_t n) 
         w[t] = r[t] - w[t];
 }
 
-template <typename A, typename B>
-__global__ void k_hs_conv(const A *__restrict__ a, B *__restrict__ b, int64_t n)
+// The coarse problem: b = r in FP64 (r32 != 0: rounded to FP32 values, the
+// V-cycle's precision), a zero guess.
+template <typename A>
+__global__ void k_hs_coarse_in(const A *__restrict__ r, double *__restrict__ b, double *__restrict__ x, int r32,
+                               int64_t n)
+{
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+        b[t] = r32 ? (double)(float)r[t] : (double)r[t];
+        x[t] = 0.0;
+    }
+}
+
+// b = a rounded to FP32 values
+__global__ void k_hs_round(const double *__restrict__ a, double *__restrict__ b, int64_t n)
 {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
-        b[t] = (B)a[t];
+        b[t] = (double)(float)a[t];
 }
 
 __global__ void k_hs_fill(double *a, double v, int64_t n)
@@ -289,50 +368,164 @@ __global__ void k_hs_fill(double *a, double v, int64_t n)
         a[t] = v;
 }
 
-// Partial inner products <w, v_i> = sum_local w v_i / mult for up to
-// HS_DOT_K vectors v_i = V + i*ld (V == nullptr: the constant 1), one row of
-// HS_DOT_BLOCKS partials per vector, summed by k_hs_dot_final in a fixed order.
-__global__ void k_hs_dots(const double *__restrict__ w, const double *__restrict__ V, int64_t ld, int k,
-                          const double *__restrict__ imult, double *__restrict__ part, int64_t n)
+// Inner products over the unique nodes, <w, v_i> for i < k (v_i = V + i*ld),
+// then <w, w> (ww != 0) and <w, 1> (one != 0): part[v][block], then the values
+// in out[v].  Block (x, y) takes HS_DOT_K of the vectors over the x-th share of
+// the nodes; the last block of a y to finish sums its vectors' partials in a
+// fixed order (deterministic) and clears the counter.
+//
+// Bound: HBM (0.77 of each vector: only the first copy of a node is read) and
+// the FP64 pipe (one FMA a unique node and vector).  Over all local nodes with
+// the weight 1/mult, eight vectors a launch and a second launch for the final
+// sums, about seven launches of 53 us a GMRES iteration (16^3 elements, N = 7, up
+// to 30 vectors); now two of 52 us.
+template <int NP>
+__global__ void __launch_bounds__(256) k_hs_dots(const double *__restrict__ w, const double *__restrict__ V,
+                                                 int64_t ld, int k, int ww, int one, UqMesh M,
+                                                 double *__restrict__ part, unsigned *__restrict__ counter,
+                                                 double *__restrict__ out)
 {
+    constexpr int CH = UqCfg<NP>::CH;
+    const int v0 = blockIdx.y * HS_DOT_K, nv = k + ww + one;
     double acc[HS_DOT_K];
 #pragma unroll
     for (int i = 0; i < HS_DOT_K; ++i) acc[i] = 0.0;
-    const int64_t G = (int64_t)gridDim.x * blockDim.x;
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    // four grid strides per pass, every load of a pass issued before its use
-    for (; t + 3 * G < n; t += 4 * G) {
-        double a[4];
+    const unsigned units = uq_units<NP>(M);
+    for (unsigned t = blockIdx.x * 256u + threadIdx.x; t < units; t += gridDim.x * 256u) {
+        const UqChunk U = uq_chunk<NP>(M, t);
+        double a[CH];
+        uq_ldv(w + U.f, a);
+        if (U.own < CH) a[CH - 1] = 0.0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) a[q] = w[t + q * G] * imult[t + q * G];
+        for (int i = 0; i < HS_DOT_K; ++i) {
+            const int v = v0 + i;
+            if (v >= nv) break;
+            double x[CH];
+            if (v < k) {
+                uq_ldv(V + v * ld + U.f, x);
+            } else {
 #pragma unroll
-        for (int i = 0; i < HS_DOT_K; ++i)
-            if (i < k) {
-                double v[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) v[q] = V ? V[i * ld + t + q * G] : 1.0;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) acc[i] = fma(a[q], v[q], acc[i]);
+                for (int q = 0; q < CH; ++q) x[q] = (ww && v == k) ? a[q] : 1.0;
             }
-    }
-    for (; t < n; t += G) {
-        const double a = w[t] * imult[t];
 #pragma unroll
-        for (int i = 0; i < HS_DOT_K; ++i)
-            if (i < k) acc[i] = fma(a, V ? V[i * ld + t] : 1.0, acc[i]);
+            for (int q = 0; q < CH; ++q) acc[i] = fma(a[q], x[q], acc[i]);
+        }
     }
-    __shared__ double red[HS_DOT_K][32];
+    // one warp per value sums the block's 256 (an eighth of the FP64 additions of a
+    // shuffle tree in every warp)
+    __shared__ double red[HS_DOT_K][256];
+    __shared__ bool last;
+    static_assert(HS_DOT_K == 8, "one value per warp of the block");
 #pragma unroll
-    for (int i = 0; i < HS_DOT_K; ++i) {
-        double v = acc[i];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if ((threadIdx.x & 31) == 0) red[i][threadIdx.x >> 5] = v;
+    for (int i = 0; i < HS_DOT_K; ++i) red[i][threadIdx.x] = acc[i];
+    __syncthreads();
+    const int nk = nv - v0 < HS_DOT_K ? nv - v0 : HS_DOT_K;
+    const int wv = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (wv < nk) {
+        double t[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) t[q] = red[wv][lane + 32 * q];
+        double s = ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) {
+            part[(size_t)(v0 + wv) * gridDim.x + blockIdx.x] = s;
+            __threadfence();
+        }
     }
     __syncthreads();
-    if (threadIdx.x < k) {
+    if (threadIdx.x == 0) last = atomicAdd(&counter[blockIdx.y], 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (wv < nk) {
+        const double *p = part + (size_t)(v0 + wv) * gridDim.x;
         double s = 0.0;
-        for (int wp = 0; wp < (int)(blockDim.x >> 5); ++wp) s += red[threadIdx.x][wp];
-        part[threadIdx.x * gridDim.x + blockIdx.x] = s;
+        for (unsigned b0 = 0; b0 < gridDim.x; b0 += 256) {  // eight loads in flight a lane
+            double t[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const unsigned b = b0 + 32 * q + lane;
+                t[q] = b < gridDim.x ? __ldcg(p + b) : 0.0;
+            }
+            s += ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+        }
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) out[v0 + wv] = s;
+    }
+    if (threadIdx.x == 0) counter[blockIdx.y] = 0u;
+}
+
+// w -= sum_{i<k} c_i v_i at every copy of every node (c: k coefficients on the
+// device), and <w, w> of the result into out[0]: a pass of Gram-Schmidt whose
+// coefficients never leave the device.  Formed at the first copies and stored to
+// all.
+template <int NP>
+__global__ void __launch_bounds__(256) k_hs_ortho(double *__restrict__ w, const double *__restrict__ V, int64_t ld,
+                                                  int k, const double *__restrict__ c, UqMesh M,
+                                                  double *__restrict__ part, unsigned *__restrict__ counter,
+                                                  double *__restrict__ out)
+{
+    constexpr int CH = UqCfg<NP>::CH;
+    __shared__ double sc[64];
+    __shared__ double red[8];
+    __shared__ bool last;
+    if ((int)threadIdx.x < k) sc[threadIdx.x] = -c[threadIdx.x];
+    __syncthreads();
+    double ww = 0.0;
+    const unsigned units = uq_units<NP>(M);
+    for (unsigned t = blockIdx.x * 256u + threadIdx.x; t < units; t += gridDim.x * 256u) {
+        const UqChunk U = uq_chunk<NP>(M, t);
+        double a[CH];
+        uq_ldv(w + U.f, a);
+        int i = 0;
+        for (; i + 4 <= k; i += 4) {
+            double x[4][CH];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) uq_ldv(V + (i + q) * ld + U.f, x[q]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int m = 0; m < CH; ++m) a[m] = fma(sc[i + q], x[q][m], a[m]);
+        }
+        for (; i < k; ++i) {
+            double x[CH];
+            uq_ldv(V + i * ld + U.f, x);
+#pragma unroll
+            for (int m = 0; m < CH; ++m) a[m] = fma(sc[i], x[m], a[m]);
+        }
+#pragma unroll
+        for (int m = 0; m < CH; ++m)
+            if (m < U.own) ww = fma(a[m], a[m], ww);
+        uq_scatter(w, U, a);
+    }
+    for (int o = 16; o > 0; o >>= 1) ww += __shfl_xor_sync(0xffffffffu, ww, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ww;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double s = 0.0;
+#pragma unroll
+        for (int wp = 0; wp < 8; ++wp) s += red[wp];
+        part[blockIdx.x] = s;
+        __threadfence();
+        last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    double s = 0.0;
+    for (unsigned b0 = 0; b0 < gridDim.x; b0 += 256) {
+        double t[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const unsigned b = b0 + 32 * q + threadIdx.x;
+            t[q] = b < gridDim.x ? __ldcg(part + b) : 0.0;
+        }
+        s += ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) {
+        out[0] = s;
+        *counter = 0u;
     }
 }
 
@@ -429,7 +622,8 @@ struct sem_hsmg {
     double *c64[2];   // coarse right-hand side and solution (FP64)
     // GMRES storage (grown on demand)
     int m_cap;
-    double *V, *Z, *r, *w, *imult64, *part, *dots;
+    double *V, *Z, *r, *w, *part, *dots;
+    unsigned *counter; // blocks done, per group of inner products
     double *hdots;    // pinned host mirror of dots
     sem_solve_info last;
 };
@@ -453,8 +647,8 @@ extern "C" void sem_hsmg_destroy(sem_hsmg *H)
         if (L.own) sem_destroy(L.c);
     }
     cudaFree(H->c64[0]); cudaFree(H->c64[1]);
-    cudaFree(H->V); cudaFree(H->Z); cudaFree(H->r); cudaFree(H->w); cudaFree(H->imult64);
-    cudaFree(H->part); cudaFree(H->dots);
+    cudaFree(H->V); cudaFree(H->Z); cudaFree(H->r); cudaFree(H->w);
+    cudaFree(H->part); cudaFree(H->dots); cudaFree(H->counter);
     if (H->hdots) cudaFreeHost(H->hdots);
     free(H);
 }
@@ -609,17 +803,15 @@ extern "C" int sem_hsmg_create(sem_ctx *c, int nlev, const int *orders, double h
             if (rc) { cudaFree(tmp); sem_hsmg_destroy(H); return rc; }
         }
     }
-    // FP64 1/mult of the finest level (GMRES inner products)
-    HS_CU(cudaMalloc(&H->imult64, sizeof(double) * c->nL));
-    rc = hs_imult(c, H->imult64, SEM_F64, tmp, 0);
     cudaFree(tmp);
-    if (rc) { sem_hsmg_destroy(H); return rc; }
     const int64_t ncl = H->L[nlev - 1].c->nL;
     HS_CU(cudaMalloc(&H->c64[0], sizeof(double) * ncl));
     HS_CU(cudaMalloc(&H->c64[1], sizeof(double) * ncl));
-    HS_CU(cudaMalloc(&H->part, sizeof(double) * HS_DOT_BLOCKS * HS_DOT_K));
-    HS_CU(cudaMalloc(&H->dots, sizeof(double) * 64));
-    HS_CU(cudaMallocHost(&H->hdots, sizeof(double) * 64));
+    HS_CU(cudaMalloc(&H->part, sizeof(double) * HS_DOT_BLOCKS * HS_DOT_MAX));
+    HS_CU(cudaMalloc(&H->dots, sizeof(double) * HS_DOT_MAX));
+    HS_CU(cudaMalloc(&H->counter, sizeof(unsigned) * (HS_DOT_MAX / HS_DOT_K + 1)));
+    HS_CU(cudaMemset(H->counter, 0, sizeof(unsigned) * (HS_DOT_MAX / HS_DOT_K + 1)));
+    HS_CU(cudaMallocHost(&H->hdots, sizeof(double) * HS_DOT_MAX));
     HS_CU(cudaDeviceSynchronize());
 #undef HS_TRY
 #undef HS_CU
@@ -631,19 +823,17 @@ extern "C" int sem_hsmg_create(sem_ctx *c, int nlev, const int *orders, double h
 // V-cycle
 // ---------------------------------------------------------------------------
 
-template <typename T>
-static int hs_fdm(sem_hsmg *H, HsLevel &L, const T *r, T *z, cudaStream_t s)
+template <typename T, typename TI>
+static int hs_fdm(sem_hsmg *H, HsLevel &L, const TI *r, T *z, cudaStream_t s)
 {
     sem_ctx *c = L.c;
-    const int n3 = c->n * c->n * c->n;
-    const int threads = n3 >= 256 ? 256 : ((n3 + 31) / 32) * 32;
-    const int64_t grid64 = c->E < (int64_t)c->num_sms * 16 ? c->E : (int64_t)c->num_sms * 16;
-    const unsigned grid = (unsigned)(grid64 > 0 ? grid64 : 1);
-#define HS_FDM_CASE(NPV)                                                                          \
-    case NPV:                                                                                     \
-        k_hs_fdm<NPV, T><<<grid, threads, 0, s>>>(r, z, (const T *)L.S, (const T *)L.lam, L.fidx, \
-                                                   (const T *)L.imult, (T)H->h1, (T)H->h2, c->E); \
-        break;
+#define HS_FDM_CASE(NPV)                                                                                          \
+    case NPV: {                                                                                                   \
+        using C = FdmCfg<NPV, T>;                                                                                 \
+        const int64_t groups = sem_ceil_div(c->E, C::NE), most = (int64_t)c->num_sms * 8;                         \
+        k_hs_fdm<NPV, T, TI><<<(unsigned)(groups < most ? groups : most), C::THREADS, 0, s>>>(                    \
+            r, z, (const T *)L.S, (const T *)L.lam, L.fidx, (const T *)L.imult, (T)H->h1, (T)H->h2, c->E);        \
+    } break;
     switch (c->n) {
         HS_FDM_CASE(2) HS_FDM_CASE(3) HS_FDM_CASE(4) HS_FDM_CASE(5) HS_FDM_CASE(6)
         HS_FDM_CASE(7) HS_FDM_CASE(8) HS_FDM_CASE(9) HS_FDM_CASE(10)
@@ -654,71 +844,79 @@ static int hs_fdm(sem_hsmg *H, HsLevel &L, const T *r, T *z, cudaStream_t s)
     return sem_dssum_dev(c, z, H->dt, s);
 }
 
-template <typename T>
-static int hs_transfer(sem_hsmg *H, int l, const T *in, T *out, int dir, int add, cudaStream_t s)
+// dir 1: out (level l + 1) = the restriction of base - in (level l), summed;
+// dir 0: out (level l) = base + the prolongation of in (level l + 1).
+template <typename T, typename TI, typename TB, typename TO>
+static int hs_transfer(sem_hsmg *H, int l, const TI *in, const TB *base, TO *out, int dir, cudaStream_t s)
 {
     HsLevel &L = H->L[l];
     const sem_ctx *cf = L.c, *cc = H->L[l + 1].c;
     const unsigned grid = (unsigned)(cf->E < (int64_t)cf->num_sms * 16 ? cf->E : (int64_t)cf->num_sms * 16);
-    k_hs_transfer<T><<<grid > 0 ? grid : 1, 128, 0, s>>>(in, out, (const T *)L.J, (const T *)L.imult, cf->n,
-                                                         cc->n, dir, add, cf->E);
+    k_hs_transfer<T><<<grid > 0 ? grid : 1, 128, 0, s>>>(in, base, out, (const T *)L.J, (const T *)L.imult, cf->n,
+                                                         cc->n, dir, cf->E);
     SEM_CHECK_LAUNCH();
     if (dir) return sem_dssum_dev(H->L[l + 1].c, out, H->dt, s);
     return SEM_OK;
 }
 
-// z = M_l^{-1} r on level l (r, z: level vectors in the V-cycle precision).
-template <typename T>
-static int hs_cycle(sem_hsmg *H, int l, T *r, T *z, cudaStream_t s)
+// The coarsest level: Jacobi-PCG in FP64 from a zero guess; the solution is left
+// in H->c64[1].
+template <typename TR>
+static int hs_coarse(sem_hsmg *H, const TR *r, cudaStream_t s)
 {
-    HsLevel &L = H->L[l];
-    sem_ctx *c = L.c;
+    sem_ctx *c = H->L[H->nlev - 1].c;
     const int64_t n = c->nL;
+    k_hs_coarse_in<TR><<<hs_grid(n), 256, 0, s>>>(r, H->c64[0], H->c64[1], H->dt == SEM_F32, n);
+    SEM_CHECK_LAUNCH();
+    sem_solve_opts o;
+    sem_solve_opts_default(&o);
+    o.tol = H->ctol;
+    o.abs_tol = 0;
+    o.maxit = H->cmaxit;
+    return sem_pcg_solve_dev(c, 0, H->c64[0], H->c64[1], H->h1, H->h2, o, s);
+}
+
+// z = M_l^{-1} r on level l < nlev - 1 (r: TR, z: TZ, the level's own vectors in
+// the V-cycle precision T).
+template <typename T, typename TR, typename TZ>
+static int hs_cycle(sem_hsmg *H, int l, const TR *r, TZ *z, cudaStream_t s)
+{
+    HsLevel &L = H->L[l], &C = H->L[l + 1];
+    sem_ctx *c = L.c;
+    T *w = (T *)L.w, *zl = (T *)L.z;
     int rc;
-    if (l == H->nlev - 1) {  // coarsest: Jacobi-PCG in FP64 from a zero guess
-        k_hs_conv<T, double><<<hs_grid(n), 256, 0, s>>>(r, H->c64[0], n);
-        SEM_CHECK_LAUNCH();
-        SEM_CUDA(cudaMemsetAsync(H->c64[1], 0, sizeof(double) * n, s));
-        sem_solve_opts o;
-        sem_solve_opts_default(&o);
-        o.tol = H->ctol;
-        o.abs_tol = 0;
-        o.maxit = H->cmaxit;
-        if ((rc = sem_pcg_solve_dev(c, 0, H->c64[0], H->c64[1], H->h1, H->h2, o, s))) return rc;
-        k_hs_conv<double, T><<<hs_grid(n), 256, 0, s>>>(H->c64[1], z, n);
-        SEM_CHECK_LAUNCH();
-        return SEM_OK;
-    }
-    HsLevel &C = H->L[l + 1];
-    T *w = (T *)L.w;
-    if ((rc = hs_fdm<T>(H, L, r, z, s))) return rc;
+    if ((rc = hs_fdm<T>(H, L, r, zl, s))) return rc;
     if constexpr (sizeof(T) == 4)
-        rc = sem_launch_ax_f32_columns(c, z, w, (float)H->h1, (float)H->h2, s);
+        rc = sem_launch_ax_f32_columns(c, zl, w, (float)H->h1, (float)H->h2, s);
     else
-        rc = sem_ax_dev_columns(c, z, w, H->h1, H->h2, s);
+        rc = sem_ax_dev_columns(c, zl, w, H->h1, H->h2, s);
     if (rc) return rc;
     if ((rc = sem_dssum_dev(c, w, H->dt, s))) return rc;
-    k_hs_sub<T><<<hs_grid(n), 256, 0, s>>>(w, r, n);
-    SEM_CHECK_LAUNCH();
-    if ((rc = hs_transfer<T>(H, l, w, (T *)C.r, 1, 0, s))) return rc;
-    if ((rc = hs_cycle<T>(H, l + 1, (T *)C.r, (T *)C.z, s))) return rc;
-    return hs_transfer<T>(H, l, (const T *)C.z, z, 0, 1, s);
+    if ((rc = hs_transfer<T>(H, l, w, r, (T *)C.r, 1, s))) return rc;
+    if (l + 1 == H->nlev - 1) {
+        if ((rc = hs_coarse(H, (const T *)C.r, s))) return rc;
+        return hs_transfer<T>(H, l, (const double *)H->c64[1], zl, z, 0, s);
+    }
+    if ((rc = hs_cycle<T>(H, l + 1, (const T *)C.r, (T *)C.z, s))) return rc;
+    return hs_transfer<T>(H, l, (const T *)C.z, zl, z, 0, s);
 }
 
 // z = M^{-1} r for FP64 E-vectors of the finest level.
 static int hs_apply_dev(sem_hsmg *H, const double *r, double *z, cudaStream_t s)
 {
-    const int64_t n = H->L[0].c->nL;
-    if (H->dt == SEM_F32) {
-        k_hs_conv<double, float><<<hs_grid(n), 256, 0, s>>>(r, (float *)H->L[0].r, n);
-        SEM_CHECK_LAUNCH();
-        int rc = hs_cycle<float>(H, 0, (float *)H->L[0].r, (float *)H->L[0].z, s);
+    if (H->nlev == 1) {
+        const int64_t n = H->L[0].c->nL;
+        const int rc = hs_coarse(H, r, s);
         if (rc) return rc;
-        k_hs_conv<float, double><<<hs_grid(n), 256, 0, s>>>((const float *)H->L[0].z, z, n);
-        SEM_CHECK_LAUNCH();
+        if (H->dt == SEM_F32) {  // (the V-cycle's precision is that of its result)
+            k_hs_round<<<hs_grid(n), 256, 0, s>>>(H->c64[1], z, n);
+            SEM_CHECK_LAUNCH();
+        } else {
+            SEM_CUDA(cudaMemcpyAsync(z, H->c64[1], sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+        }
         return SEM_OK;
     }
-    return hs_cycle<double>(H, 0, (double *)r, z, s);
+    return H->dt == SEM_F32 ? hs_cycle<float>(H, 0, r, z, s) : hs_cycle<double>(H, 0, r, z, s);
 }
 
 extern "C" int sem_hsmg_apply(sem_hsmg *H, const double *r, double *z, void *stream)
@@ -731,17 +929,24 @@ extern "C" int sem_hsmg_apply(sem_hsmg *H, const double *r, double *z, void *str
 // Flexible GMRES
 // ---------------------------------------------------------------------------
 
-// dots[i] = <w, v_i>, i < k (V == nullptr: <w, 1>), into H->hdots (synchronises s).
-// (enqueue only: the values land in H->dots + at)
-static int hs_dots_enq(sem_hsmg *H, const double *w, const double *V, int64_t ld, int k, int at, cudaStream_t s)
+// Inner products of w (see k_hs_dots) into H->dots; enqueue only.
+static int hs_dots_enq(sem_hsmg *H, const double *w, const double *V, int64_t ld, int k, int ww, int one,
+                       cudaStream_t s)
 {
-    const int64_t n = H->L[0].c->nL;
-    for (int i0 = 0; i0 < k; i0 += HS_DOT_K) {
-        const int kk = k - i0 < HS_DOT_K ? k - i0 : HS_DOT_K;
-        k_hs_dots<<<HS_DOT_BLOCKS, 256, 0, s>>>(w, V ? V + i0 * ld : nullptr, ld, kk, H->imult64, H->part, n);
-        k_hs_dot_final<<<kk, 256, 0, s>>>(H->part, HS_DOT_BLOCKS, H->dots + at + i0);
-        SEM_CHECK_LAUNCH();
+    const sem_ctx *c = H->L[0].c;
+    const UqMesh M = uq_mesh(sem_gs_desc(c));
+    const int nv = k + ww + one;
+    if (nv < 1 || nv > HS_DOT_MAX) return SEM_ERR_ARG;
+    const dim3 grid(c->num_sms * 2, (nv + HS_DOT_K - 1) / HS_DOT_K);
+    if ((int)grid.x > HS_DOT_BLOCKS) return SEM_ERR_ARG;
+#define HS_CASE(NPV) \
+    case NPV: k_hs_dots<NPV><<<grid, 256, 0, s>>>(w, V, ld, k, ww, one, M, H->part, H->counter, H->dots); break;
+    switch (c->n) {
+        HS_CASE(2) HS_CASE(3) HS_CASE(4) HS_CASE(5) HS_CASE(6) HS_CASE(7) HS_CASE(8) HS_CASE(9) HS_CASE(10)
+        default: return SEM_ERR_ARG;
     }
+#undef HS_CASE
+    SEM_CHECK_LAUNCH();
     return SEM_OK;
 }
 
@@ -752,10 +957,33 @@ static int hs_dots_read(sem_hsmg *H, int k, cudaStream_t s)
     return SEM_OK;
 }
 
-static int hs_dots(sem_hsmg *H, const double *w, const double *V, int64_t ld, int k, cudaStream_t s)
+// <w, w> (or <w, 1>) into H->hdots[0]; synchronises s.
+static int hs_dot(sem_hsmg *H, const double *w, bool one, cudaStream_t s)
 {
-    int rc = hs_dots_enq(H, w, V, ld, k, 0, s);
-    return rc ? rc : hs_dots_read(H, k, s);
+    const int rc = hs_dots_enq(H, w, nullptr, 0, 0, !one, one, s);
+    return rc ? rc : hs_dots_read(H, 1, s);
+}
+
+// One pass of classical Gram-Schmidt of w against v_0 .. v_{k-1}: H->hdots[i] =
+// <w, v_i>, [k] = <w, w> before it, [k + 1] = <w, w> after it; synchronises s.
+static int hs_gs_pass(sem_hsmg *H, double *w, const double *V, int64_t ld, int k, cudaStream_t s)
+{
+    const sem_ctx *c = H->L[0].c;
+    const UqMesh M = uq_mesh(sem_gs_desc(c));
+    const int rc = hs_dots_enq(H, w, V, ld, k, 1, 0, s);
+    if (rc) return rc;
+#define HS_CASE(NPV)                                                                                            \
+    case NPV:                                                                                                   \
+        k_hs_ortho<NPV><<<c->num_sms * 4, 256, 0, s>>>(w, V, ld, k, H->dots, M, H->part, H->counter,            \
+                                                       H->dots + k + 1);                                        \
+        break;
+    switch (c->n) {
+        HS_CASE(2) HS_CASE(3) HS_CASE(4) HS_CASE(5) HS_CASE(6) HS_CASE(7) HS_CASE(8) HS_CASE(9) HS_CASE(10)
+        default: return SEM_ERR_ARG;
+    }
+#undef HS_CASE
+    SEM_CHECK_LAUNCH();
+    return hs_dots_read(H, k + 2, s);
 }
 
 // y += sum_i c[i] v_i
@@ -819,12 +1047,12 @@ int sem_gmres_solve_dev(sem_hsmg *H, int precond, const double *b_in, double *x,
     SEM_CUDA(cudaMemcpyAsync(r, b_in, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     double bmean = 0.0;
     if (singular) {
-        if ((rc = hs_dots(H, r, nullptr, 0, 1, s))) return rc;
+        if ((rc = hs_dot(H, r, true, s))) return rc;
         bmean = H->hdots[0] / (double)c->nG;
         k_hs_add_scalar<<<hs_grid(n), 256, 0, s>>>(r, -bmean, n);
         SEM_CHECK_LAUNCH();
     }
-    if ((rc = hs_dots(H, r, r, n, 1, s))) return rc;
+    if ((rc = hs_dot(H, r, false, s))) return rc;
     const double bnorm = sqrt(H->hdots[0]);
     const double target = o.abs_tol ? o.tol : o.tol * bnorm;
     // The true residual decides convergence.  Below 1e-8 ||b|| it is taken
@@ -845,7 +1073,7 @@ int sem_gmres_solve_dev(sem_hsmg *H, int precond, const double *b_in, double *x,
         k_hs_sub<double><<<hs_grid(n), 256, 0, s>>>(w, r, n);  // w = r - w
         SEM_CHECK_LAUNCH();
         SEM_CUDA(cudaMemcpyAsync(r, w, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-        if ((rc2 = hs_dots(H, r, r, n, 1, s))) return rc2;
+        if ((rc2 = hs_dot(H, r, false, s))) return rc2;
         *beta = sqrt(H->hdots[0]);
         return SEM_OK;
     };
@@ -879,22 +1107,16 @@ int sem_gmres_solve_dev(sem_hsmg *H, int precond, const double *b_in, double *x,
             std::fill(h.begin(), h.end(), 0.0);
             double hn = 0.0;
             for (int pass = 0; pass < 2; ++pass) {
-                if ((rc = hs_dots_enq(H, w, V, n, j + 1, 0, s))) return rc;
-                if ((rc = hs_dots_enq(H, w, w, n, 1, j + 1, s))) return rc;
-                if ((rc = hs_dots_read(H, j + 2, s))) return rc;
+                if ((rc = hs_gs_pass(H, w, V, n, j + 1, s))) return rc;
                 const double ww = H->hdots[j + 1];
-                std::vector<double> neg(j + 1);
                 double proj = 0.0;
                 for (int i = 0; i <= j; ++i) {
                     h[i] += H->hdots[i];
-                    neg[i] = -H->hdots[i];
                     proj += H->hdots[i] * H->hdots[i];
                 }
-                if ((rc = hs_maxpy(H, w, V, n, j + 1, neg.data(), s))) return rc;
+                hn = sqrt(H->hdots[j + 2]);
                 if (ww - proj > 0.5 * ww) break;
             }
-            if ((rc = hs_dots(H, w, w, n, 1, s))) return rc;
-            hn = sqrt(H->hdots[0]);
             for (int i = 0; i <= j; ++i) Hm[(size_t)i * m + j] = h[i];
             for (int i = 0; i < j; ++i) {  // earlier rotations on column j
                 const double a = Hm[(size_t)i * m + j], b2 = Hm[(size_t)(i + 1) * m + j];
