@@ -159,7 +159,7 @@ SEM_API int sem_ax(sem_ctx *ctx, const void *u, void *w, double h1, double h2, s
  * fastest for this process and returns it in *best; ms (NULL, or
  * SEM_TUNE_MAX entries) receives the average time of each candidate (-1
  * where a candidate does not apply).  Synchronous.  Candidates:
- *  - SEM_F32: 0 = direct loads, 1 = bulk-copy staged, 256 threads x 2 stages,
+ *  - SEM_F32: 0 = whole lines, 1 = bulk-copy staged, 256 threads x 2 stages,
  *    2 = staged, 128 threads x 3 stages;
  *  - SEM_F64 with even N+1 <= 12: the float-pair folded kernel with
  *    0 = 256/(N+1)^2 elements per block and block-wide barriers, 1 = one
@@ -387,7 +387,7 @@ typedef struct {
  * PCG; with op = SEM_F32 the default pressure solve is an FP32 inner PCG inside
  * FP64 refinement).  The solves' inner field selects their precision.
  * The stepper keeps a reference to ctx (which must outlive it) and solves on
- * the context's workspace slots 4-7; it allocates about 32 FP64 E-vectors plus
+ * the context's workspace slots 4-7; it allocates about 34 FP64 E-vectors plus
  * J^-1 and float-pair tables on the device (SEM_ERR_NOMEM if they do not fit).
  * SEM_ERR_ARG: NULL ctx or out, nu or dt not positive, an unsupported op, a
  * context that is not periodic in all three directions, or N > 9.  The state

@@ -9,7 +9,7 @@
 //                                                                (k_tgv_g, unique nodes)
 //   4. A p     = dssum( sum_a D_a^T ( B sum_c (dr_a/dx_c) g_c ) )  (k_tgv_divg + PCG)
 //   5. (nu A + b0/dt B) u_c = dssum( F_c + B (sum_j b_j u_c/dt - dp/dx_c) )
-//                                                   (k_tgv_vrhs + 3-problem batched PCG)
+//                                                   (k_tgv_vel + 3-problem batched PCG)
 //   6. shift histories; KE and enstrophy into a device log      (k_tgv_diag_*)
 // Precision policy (Sec. 2, Fig. 2): the rule in force at a step selects the
 // convection precision (FP64, FP32, or FP16/BF16 operands with FP32
@@ -20,8 +20,8 @@
 // convective term is computed in FP32; the solves use the precision of the
 // options passed (the default pressure options then select an FP32 inner PCG
 // inside FP64 refinement; the velocity Helmholtz solves, a few iterations per
-// step, stay FP64 unless their options ask otherwise).  Steady-state steps (q = 3) are captured once into
-// a CUDA graph and replayed.  Orders N <= 9.
+// step, stay FP64 unless their options ask otherwise).  Steady-state steps (q = 3) are captured
+// into CUDA graphs (one per arrangement of the history buffers) and replayed.  Orders N <= 9.
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -29,14 +29,19 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "ax_df.cuh"
+#include "ax_dfl.cuh"
 #include "common.cuh"
 #include "df64.cuh"
 #include "gs.cuh"
+#include "tma.cuh"
+#include "uniq.cuh"
 
 GsDesc sem_gs_desc(const sem_ctx *c);
 int sem_run_geometry(sem_ctx *c, double *xyz, bool with_jinv, cudaStream_t s);
 int sem_alloc_ws(sem_ctx *c, int slot);
 int sem_dssum_dev(sem_ctx *c, void *u, sem_dtype dt, cudaStream_t s);
+int sem_dssum_dev_n(sem_ctx *c, int n, void *const *u, sem_dtype dt, cudaStream_t s);
 int sem_ax_dev_columns(sem_ctx *c, const double *u, double *w, double h1, double h2, cudaStream_t s);
 int sem_pcg_solve_dev_batch(sem_ctx *c, int np, const double *const *b, double *const *x, double h1,
                             double h2, const sem_solve_opts &o, cudaStream_t s, int slot0, bool ordered);
@@ -59,6 +64,11 @@ struct TgvDev {       // device-side counters
     long long count;  // entries written so far
     double t;
     double cfl;       // CFL number of the latest step
+};
+
+// Derivative matrix as a kernel parameter (constant-bank operands), row-major NP x NP.
+struct VelD {
+    double d[10 * 10];
 };
 
 struct sem_tgv {
@@ -99,9 +109,12 @@ struct sem_tgv {
     TgvLogEntry *log;  // device ring
     TgvLogEntry *hlog; // pinned host copy
     TgvDev *dev;
-    cudaGraphExec_t graph;
-    cudaStream_t graph_stream;
-    int graph_state;   // 0 not tried, 1 ready, -1 unavailable
+    int turn;          // arrangement of the history buffers (0..2; each step exchanges them)
+    double *bsum, *binv;  // dssum(B), 1 / dssum(B) (one allocation)
+    DflTabs dtabs;     // folded derivative tables of the diagnostics
+    VelD veld;         // derivative matrix of the velocity pass
+    cudaGraphExec_t graph[3];  // the captured step, one per arrangement
+    int graph_state[3];        // 0 not tried, 1 ready, -1 unavailable
     int graph_warm;    // a steady step ran directly since the last (re)capture was needed
     double *block;     // one allocation for all fields
 };
@@ -403,32 +416,45 @@ __global__ void __launch_bounds__(256) k_convect(ConvArgs a)
 // ---------------------------------------------------------------------------
 
 struct Coef {
-    double a[3], b[3], b0, dt;
+    double a[3], b[3], b0, dt, rdt;  // (rdt = 1 / dt)
 };
+
+// CH stored values from position q (FP32 when s32).
+template <int CH>
+__device__ __forceinline__ void ld_fsv(const void *p, size_t q, int s32, double (&v)[CH])
+{
+    if (s32) {
+        float f[CH];
+        uq_ldv((const float *)p + q, f);
+#pragma unroll
+        for (int i = 0; i < CH; ++i) v[i] = (double)f[i];
+    } else {
+        uq_ldv((const double *)p + q, v);
+    }
+}
+
+// k[0] x + k[1] y + k[2] z over the levels of a history; the order is written out
+// because the step's results follow its last bit (see div_r).
+__device__ __forceinline__ double sum3(const double (&k)[3], double x, double y, double z)
+{
+    return fma(k[2], z, fma(k[0], x, k[1] * y));
+}
+
+// a / b from r = 1 / b rounded: one residual step restores the quotient's last
+// bit (Markstein, IBM J. Res. Dev. 34, 1990), in three operations.  The steps
+// must not differ from a divided form by even that bit: the loosely stopped
+// solves downstream amplify a last-bit change of the velocity by 1e6 and more.
+__device__ __forceinline__ double div_r(double a, double b, double r)
+{
+    const double q = a * r;
+    return fma(fma(-q, b, a), r, q);
+}
 
 struct FArgs {
     const void *C[3][3];  // [level][comp], stored fields
     double *F[3];
     int s32;
 };
-
-// Initial guess of the velocity solves: u_c^* = sum_j a_j u_c^{n+1-j} (the EXT
-// weights of the step), from the stored histories into the FP64 iterate.
-struct XArgs {
-    const void *u[3][3];  // [level][comp], stored fields
-    double *x[3];
-    int s32;
-};
-
-__global__ void k_tgv_ext(XArgs a, Coef k, int64_t nL)
-{
-    int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q >= nL) return;
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-        a.x[c][q] = k.a[0] * ld_fs(a.u[0][c], q, a.s32) + k.a[1] * ld_fs(a.u[1][c], q, a.s32) +
-                    k.a[2] * ld_fs(a.u[2][c], q, a.s32);
-}
 
 __global__ void k_tgv_F(FArgs a, Coef k, int64_t nL)
 {
@@ -444,33 +470,41 @@ struct GArgs {
     const double *F[3];
     const void *u[3][3];  // [level][comp], stored fields
     double *g[3];
-    const double *geo64;
-    GsDesc gs;
+    const double *bsum, *binv;  // dssum(B) and its reciprocal
+    UqMesh mesh;
     Coef k;
     int s32;
 };
 
-// g_c = dssum(F_c) / dssum(B) + sum_j b_j u^{n+1-j}_c / dt at every copy.
-__global__ void k_tgv_g(GArgs a)
+// g_c = dssum(F_c) / dssum(B) + sum_j b_j u^{n+1-j}_c / dt at every copy, a
+// thread per chunk of unique nodes (uniq.cuh).
+//
+// Bound: the FP64 pipe (about 40 operations a unique node; 20 words).  A node at
+// a time, with dssum(B) gathered again and six divisions: 1.58 ms at 32^3,
+// N = 7, now 1.08.  Forming F
+// in the same pass was slower (2.75 ms against 0.66 for F alone and this).
+template <int NP>
+__global__ void __launch_bounds__(256) k_tgv_g(GArgs a)
 {
-    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (g >= a.gs.nG) return;
-    int64_t idx[8];
-    const int m = gs_copies(a.gs, g, idx);
-    const int n3 = a.gs.n * a.gs.n * a.gs.n;
-    double bs = 0.0;
-    for (int t = 0; t < m; ++t) {
-        const int64_t e = idx[t] / n3;
-        bs += a.geo64[(e * 7 + 6) * n3 + (idx[t] - e * n3)];
-    }
-    const int64_t f = idx[0];
+    constexpr int CH = UqCfg<NP>::CH;
+    const unsigned t = blockIdx.x * 256u + threadIdx.x;
+    if (t >= uq_units<NP>(a.mesh)) return;
+    const UqChunk U = uq_chunk<NP>(a.mesh, t);
+    double rb[CH], bs[CH];
+    uq_ldv(a.binv + U.f, rb);
+    uq_ldv(a.bsum + U.f, bs);
+#pragma unroll 1
     for (int c = 0; c < 3; ++c) {
-        double s = 0.0;
-        for (int t = 0; t < m; ++t) s += a.F[c][idx[t]];
-        const double hist = a.k.b[0] * ld_fs(a.u[0][c], f, a.s32) + a.k.b[1] * ld_fs(a.u[1][c], f, a.s32) +
-                            a.k.b[2] * ld_fs(a.u[2][c], f, a.s32);
-        const double v = s / bs + hist / a.k.dt;
-        for (int t = 0; t < m; ++t) a.g[c][idx[t]] = v;
+        double s[CH], h0[CH], h1[CH], h2[CH];
+        uq_gather(a.F[c], U, s, [&] {
+            ld_fsv(a.u[0][c], U.f, a.s32, h0);
+            ld_fsv(a.u[1][c], U.f, a.s32, h1);
+            ld_fsv(a.u[2][c], U.f, a.s32, h2);
+        });
+#pragma unroll
+        for (int i = 0; i < CH; ++i)
+            s[i] = div_r(s[i], bs[i], rb[i]) + div_r(sum3(a.k.b, h0[i], h1[i], h2[i]), a.k.dt, a.k.rdt);
+        uq_scatter(a.g[c], U, s);
     }
 }
 
@@ -515,113 +549,185 @@ __global__ void k_tgv_divg(const double *g0, const double *g1, const double *g2,
 struct VArgs {
     const double *F[3];
     const void *u[3][3];  // stored fields
+    double *x[3];         // initial guesses (may be the oldest velocities' buffers)
     int s32;
-    const double *p;
-    const double *jinv, *geo64, *D;
+    const double *p, *geo64;
+    const double *jinv;
     double *rhs[3];
     Coef k;
     int64_t E;
 };
 
-// rhs_c = F_c + B ( sum_j b_j u_c / dt - dp/dx_c )   (local, one block per element)
+// rhs_c = F_c + B ( sum_j b_j u_c / dt - dp/dx_c )   (local, one block per
+// element), and the initial guess of the velocity solves
+// x_c = sum_j a_j u_c^{n+1-j} (the EXT weights of the step) from the same
+// histories.  The pressure gradient by whole lines, a line a thread: each value
+// of p is read once a direction and the matrix entries are constant-bank
+// operands, in the order of one dot product a node.
+//
+// Bound: the FP64 pipe (66 operations a node) and HBM (29 words a node) alike.
+// One node a thread, every product with two shared reads and a division a
+// component, and the guess in a pass of its own: 2.1 + 0.56 ms at 32^3, N = 7,
+// now 2.08.
 template <int NP>
-__global__ void k_tgv_vrhs(VArgs a)
+struct VelCfg {
+    static constexpr int N2 = NP * NP, N3 = N2 * NP, LSX = NP | 1, SL = N2 * LSX;
+    static constexpr int TH = NP <= 4 ? 64 : NP <= 6 ? 128 : NP <= 8 ? 192 : 256;
+};
+
+template <int NP>
+__global__ void __launch_bounds__(VelCfg<NP>::TH) k_tgv_vel(VArgs a, const __grid_constant__ VelD D)
 {
-    constexpr int N3 = NP * NP * NP;
-    __shared__ double sp[N3];
-    __shared__ double sD[NP * NP];
-    for (int t = threadIdx.x; t < NP * NP; t += blockDim.x) sD[t] = a.D[t];
+    using C = VelCfg<NP>;
+    constexpr int N2 = C::N2, N3 = C::N3, LSX = C::LSX, SL = C::SL, TH = C::TH;
+    __shared__ double sp[SL], sg[3 * SL];
     for (int64_t e = blockIdx.x; e < a.E; e += gridDim.x) {
         __syncthreads();
         const int64_t off = e * N3;
-        for (int pn = threadIdx.x; pn < N3; pn += blockDim.x) sp[pn] = a.p[off + pn];
+        if (threadIdx.x == 0) l2_prefetch_span(a.jinv, e * 9 * N3 * 8, (e + 1) * 9 * N3 * 8);
+        for (int pn = threadIdx.x; pn < N3; pn += TH) {
+            const int row = pn / NP;
+            sp[row * LSX + (pn - row * NP)] = a.p[off + pn];
+        }
         __syncthreads();
-        for (int pn = threadIdx.x; pn < N3; pn += blockDim.x) {
-            const int i = pn % NP, j = (pn / NP) % NP, k = pn / (NP * NP);
-            double gr = 0, gs = 0, gt = 0;
+        for (int t = threadIdx.x; t < 3 * N2; t += TH) {
+            const int dir = t / N2, ln = t - dir * N2, p = ln / NP, q = ln - p * NP;
+            const int st = dir == 0 ? 1 : dir == 1 ? LSX : NP * LSX;
+            const int o = dir == 0 ? ln * LSX : dir == 1 ? p * NP * LSX + q : p * LSX + q;
+            double x[NP];
 #pragma unroll
-            for (int l = 0; l < NP; ++l) {
-                gr += sD[i * NP + l] * sp[(k * NP + j) * NP + l];
-                gs += sD[j * NP + l] * sp[(k * NP + l) * NP + i];
-                gt += sD[k * NP + l] * sp[(l * NP + j) * NP + i];
+            for (int l = 0; l < NP; ++l) x[l] = sp[o + l * st];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                double y = 0.0;
+#pragma unroll
+                for (int l = 0; l < NP; ++l) y += D.d[i * NP + l] * x[l];
+                sg[dir * SL + o + i * st] = y;
             }
+        }
+        __syncthreads();
+        for (int pn = threadIdx.x; pn < N3; pn += TH) {
+            const int row = pn / NP, o = row * LSX + (pn - row * NP);
             const double *ji = a.jinv + e * 9 * N3 + pn;
+            double J[9];
+#pragma unroll
+            for (int m = 0; m < 9; ++m) J[m] = ji[m * N3];
             const double bm = a.geo64[(e * 7 + 6) * N3 + pn];
+            const double gr = sg[o], gs = sg[SL + o], gt = sg[2 * SL + o];
             const int64_t q = off + pn;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const double dpdx = ji[(0 * 3 + c) * N3] * gr + ji[(1 * 3 + c) * N3] * gs +
-                                    ji[(2 * 3 + c) * N3] * gt;
-                const double hist = a.k.b[0] * ld_fs(a.u[0][c], q, a.s32) + a.k.b[1] * ld_fs(a.u[1][c], q, a.s32) +
-                                    a.k.b[2] * ld_fs(a.u[2][c], q, a.s32);
-                a.rhs[c][q] = a.F[c][q] + bm * (hist / a.k.dt - dpdx);
+                const double dpdx = J[c] * gr + J[3 + c] * gs + J[6 + c] * gt;
+                const double u0 = ld_fs(a.u[0][c], q, a.s32), u1 = ld_fs(a.u[1][c], q, a.s32),
+                             u2 = ld_fs(a.u[2][c], q, a.s32);
+                const double hist = sum3(a.k.b, u0, u1, u2);
+                a.rhs[c][q] = a.F[c][q] + bm * (div_r(hist, a.k.dt, a.k.rdt) - dpdx);
+                // (orders of the guess's products: those of the pass it had to itself)
+                a.x[c][q] = c == 2 ? fma(a.k.a[2], u2, fma(a.k.a[1], u1, a.k.a[0] * u0)) : sum3(a.k.a, u0, u1, u2);
             }
         }
     }
 }
 
-// Per-element sum of B|u|^2 and B|curl u|^2.
-// T as in k_tgv_divg: the gradients, the vorticity and both integrals per
-// element in T; the block sums in FP64.
-// With them, the element's largest sum_a |U_a| / dxi_a over its nodes (U_a =
-// sum_c (dr_a/dx_c) u_c, dxi_a the GLL gap at the node's index along a; the
-// CFL number per unit step, Sec. 3), in FP64 from the T-accurate U_a.
+// Per-element sums of B|u|^2 and B|curl u|^2 (part[0][e], part[1][e]) and the
+// element's largest sum_a |U_a| / dxi_a over its nodes (part[2][e]; U_a = sum_c
+// (dr_a/dx_c) u_c, dxi_a the GLL gap at the node's index along a; the CFL number
+// per unit step, Sec. 3).  Gradients, vorticity and both integrands in float
+// pairs (jinv, geo, D as pairs), the sums over an element in FP64.
+//
+// Bound: FP32 issue and HBM (13 words a node).  The nine derivatives run by whole
+// folded lines (ax_dfl.cuh), and only the six products that the vorticity needs
+// are formed; a node at a time, with all nine: 1.73 ms at 32^3, N = 7, now 1.07.
 struct GapInv {
-    double v[SEM_NPMAX];
+    dfp v[SEM_NPMAX];
 };
 
-template <int NP, typename T>
-__global__ void k_tgv_diag_part(const void *u0, const void *u1, const void *u2, int s32,
-                                const T *jinv, const T *geo, const T *D, GapInv ig, double *part, int64_t E)
+template <int NP>
+struct DiagCfg {
+    static constexpr int N2 = NP * NP, N3 = N2 * NP, LSX = NP | 1;
+    static constexpr int TH = NP <= 4 ? 64 : NP <= 6 ? 128 : NP <= 8 ? 192 : 256;
+    static constexpr size_t SMEM = sizeof(dfp) * 12 * (size_t)(N2 * LSX);
+};
+
+template <int NP>
+__global__ void __launch_bounds__(DiagCfg<NP>::TH)
+    k_tgv_diag_part(const void *u0, const void *u1, const void *u2, int s32, const dfp *__restrict__ jinv,
+                    const dfp *__restrict__ geo, const __grid_constant__ DflTabs T, const __grid_constant__ GapInv ig, double *part,
+                    int64_t E)
 {
-    constexpr int N3 = NP * NP * NP;
-    __shared__ T su[3 * N3];
-    __shared__ T sD[NP * NP];
-    __shared__ double sred[3 * 32];
-    for (int t = threadIdx.x; t < NP * NP; t += blockDim.x) sD[t] = D[t];
-    const void *uu[3] = {u0, u1, u2};
+    using C = DiagCfg<NP>;
+    constexpr int N2 = C::N2, N3 = C::N3, LSX = C::LSX, TH = C::TH, SL = N2 * LSX;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    dfp *su = reinterpret_cast<dfp *>(smem_raw), *sg = su + 3 * SL;  // u_c; derivative (c, direction)
+    __shared__ double sred[3 * (TH / 32)];
     for (int64_t e = blockIdx.x; e < E; e += gridDim.x) {
         __syncthreads();
         const int64_t off = e * N3;
-        for (int t = threadIdx.x; t < 3 * N3; t += blockDim.x) su[t] = T(ld_fs(uu[t / N3], off + t % N3, s32));
-        __syncthreads();
-        T tke = 0, ten = 0;
-        double cmax = 0.0;
-        for (int pn = threadIdx.x; pn < N3; pn += blockDim.x) {
-            const int i = pn % NP, j = (pn / NP) % NP, k = pn / (NP * NP);
-            const T *ji = jinv + e * 9 * N3 + pn;
-            {
-                const int ia[3] = {i, j, k};
-                double cn = 0.0;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const T U = fma(ji[(a * 3 + 0) * N3], su[pn],
-                                    fma(ji[(a * 3 + 1) * N3], su[N3 + pn], ji[(a * 3 + 2) * N3] * su[2 * N3 + pn]));
-                    cn += fabs((double)U) * ig.v[ia[a]];
-                }
-                cmax = fmax(cmax, cn);
-            }
-            T du[3][3];  // du[c][d] = du_c / dx_d
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const T *uc = su + c * N3;
-                T gr = 0, gs = 0, gt = 0;
-#pragma unroll
-                for (int l = 0; l < NP; ++l) {
-                    gr = fma(sD[i * NP + l], uc[(k * NP + j) * NP + l], gr);
-                    gs = fma(sD[j * NP + l], uc[(k * NP + l) * NP + i], gs);
-                    gt = fma(sD[k * NP + l], uc[(l * NP + j) * NP + i], gt);
-                }
-#pragma unroll
-                for (int d = 0; d < 3; ++d)
-                    du[c][d] = fma(ji[(0 * 3 + d) * N3], gr, fma(ji[(1 * 3 + d) * N3], gs, ji[(2 * 3 + d) * N3] * gt));
-            }
-            const T wx = du[2][1] - du[1][2], wy = du[0][2] - du[2][0], wz = du[1][0] - du[0][1];
-            const T bm = geo[(e * 7 + 6) * N3 + pn];
-            tke = fma(bm, fma(su[pn], su[pn], fma(su[N3 + pn], su[N3 + pn], su[2 * N3 + pn] * su[2 * N3 + pn])), tke);
-            ten = fma(bm, fma(wx, wx, fma(wy, wy, wz * wz)), ten);
+        if (threadIdx.x == 0) l2_prefetch_span(jinv, e * 9 * N3 * 8, (e + 1) * 9 * N3 * 8);
+        for (int pn = threadIdx.x; pn < N3; pn += TH) {
+            const int row = pn / NP, o = row * LSX + (pn - row * NP);
+            const df64 a(ld_fs(u0, off + pn, s32)), b(ld_fs(u1, off + pn, s32)), c(ld_fs(u2, off + pn, s32));
+            su[o] = {a.hi, a.lo};
+            su[SL + o] = {b.hi, b.lo};
+            su[2 * SL + o] = {c.hi, c.lo};
         }
-        double ke = (double)tke, en = (double)ten;
+        __syncthreads();
+        for (int t = threadIdx.x; t < 9 * N2; t += TH) {
+            const int cd = t / N2, ln = t - cd * N2, c = cd / 3, dir = cd - 3 * c, p = ln / NP, q = ln - p * NP;
+            const int st = dir == 0 ? 1 : dir == 1 ? LSX : NP * LSX;
+            const int o = dir == 0 ? ln * LSX : dir == 1 ? p * NP * LSX + q : p * LSX + q;
+            dfp x[NP], y[NP];
+#pragma unroll
+            for (int l = 0; l < NP; ++l) x[l] = su[c * SL + o + l * st];
+            dfl_line<NP, 0>(x, y, T);
+#pragma unroll
+            for (int l = 0; l < NP; ++l) sg[cd * SL + o + l * st] = y[l];
+        }
+        __syncthreads();
+        dfacc tke = {0.f, 0.f}, ten = {0.f, 0.f};
+        double cmax = 0.0;
+        for (int pn = threadIdx.x; pn < N3; pn += TH) {
+            const int row = pn / NP, i = pn - row * NP, j = row % NP, k = row / NP, o = row * LSX + i;
+            const dfp *ji = jinv + e * 9 * N3 + pn;
+            dfp J[9];
+#pragma unroll
+            for (int m = 0; m < 9; ++m) J[m] = ji[m * N3];
+            const dfp bm = geo[(e * 7 + 6) * N3 + pn];
+            const dfp uu[3] = {su[o], su[SL + o], su[2 * SL + o]};
+            const int ia[3] = {i, j, k};
+            dfacc cn = {0.f, 0.f};
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                dfacc U = df_mul(J[a * 3], uu[0]);
+                df_mad(U, J[a * 3 + 1], uu[1]);
+                df_mad(U, J[a * 3 + 2], uu[2]);
+                const float s = __fadd_rn(U.s, U.e), r = __fsub_rn(U.e, __fsub_rn(s, U.s));
+                df_mad(cn, ig.v[ia[a]], s < 0.f ? dfp{-s, -r} : dfp{s, r});
+            }
+            cmax = fmax(cmax, df_widen(cn.s) + df_widen(cn.e));
+            // component du_c/dx_d - du_d/dx_c
+            auto curl = [&](int c, int d) {
+                dfacc w = {0.f, 0.f};
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    const dfp g = sg[(3 * c + r) * SL + o], h = sg[(3 * d + r) * SL + o];
+                    df_mad(w, J[r * 3 + d], g);
+                    df_mad(w, J[r * 3 + c], {-h.hi, -h.lo});
+                }
+                const float s = __fadd_rn(w.s, w.e);
+                return dfp{s, __fsub_rn(w.e, __fsub_rn(s, w.s))};
+            };
+            const dfp wx = curl(2, 1), wy = curl(0, 2), wz = curl(1, 0);
+            dfacc q = df_mul(uu[0], uu[0]);
+            df_mad(q, uu[1], uu[1]);
+            df_mad(q, uu[2], uu[2]);
+            df_mad(tke, bm, df_raw(q));
+            q = df_mul(wx, wx);
+            df_mad(q, wy, wy);
+            df_mad(q, wz, wz);
+            df_mad(ten, bm, df_raw(q));
+        }
+        double ke = (double)tke.s + (double)tke.e, en = (double)ten.s + (double)ten.e;
         for (int o = 16; o > 0; o >>= 1) {
             ke += __shfl_xor_sync(0xffffffffu, ke, o);
             en += __shfl_xor_sync(0xffffffffu, en, o);
@@ -635,33 +741,39 @@ __global__ void k_tgv_diag_part(const void *u0, const void *u1, const void *u2, 
         __syncthreads();
         if (threadIdx.x == 0) {
             double a = 0, b = 0, m = 0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+            for (int w = 0; w < TH / 32; ++w) {
                 a += sred[3 * w];
                 b += sred[3 * w + 1];
                 m = fmax(m, sred[3 * w + 2]);
             }
-            part[3 * e] = a;
-            part[3 * e + 1] = b;
-            part[3 * e + 2] = m;
+            part[e] = a;
+            part[E + e] = b;
+            part[2 * E + e] = m;
         }
     }
 }
 
 // Fixed-order sum of the element partials into the log (and the largest CFL
-// rate times dt); advances time and count.
-__global__ void k_tgv_diag_final(const double *part, int64_t E, double V, double dt, TgvDev *dv,
-                                 TgvLogEntry *log, int advance)
+// rate times dt); advances time and count.  One block: each thread keeps four
+// strided sums, so that their loads overlap.
+__global__ void __launch_bounds__(1024) k_tgv_diag_final(const double *part, int64_t E, double V, double dt,
+                                                         TgvDev *dv, TgvLogEntry *log, int advance)
 {
-    __shared__ double s[3][256];
-    double a = 0.0, b = 0.0, m = 0.0;
-    for (int64_t e = threadIdx.x; e < E; e += blockDim.x) {
-        a += part[3 * e];
-        b += part[3 * e + 1];
-        m = fmax(m, part[3 * e + 2]);
-    }
-    s[0][threadIdx.x] = a;
-    s[1][threadIdx.x] = b;
-    s[2][threadIdx.x] = m;
+    __shared__ double s[3][1024];
+    double a[4] = {0.0, 0.0, 0.0, 0.0}, b[4] = {0.0, 0.0, 0.0, 0.0}, m[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int64_t e0 = threadIdx.x; e0 < E; e0 += 4 * 1024)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t e = e0 + q * 1024;
+            if (e < E) {
+                a[q] += part[e];
+                b[q] += part[E + e];
+                m[q] = fmax(m[q], part[2 * E + e]);
+            }
+        }
+    s[0][threadIdx.x] = (a[0] + a[1]) + (a[2] + a[3]);
+    s[1][threadIdx.x] = (b[0] + b[1]) + (b[2] + b[3]);
+    s[2][threadIdx.x] = fmax(fmax(m[0], m[1]), fmax(m[2], m[3]));
     __syncthreads();
     for (int o = blockDim.x / 2; o > 0; o >>= 1) {
         if (threadIdx.x < o) {
@@ -724,6 +836,27 @@ __global__ void k_tgv_log_host(TgvDev *dv, TgvLogEntry *log, int slot, int iters
     if (status != 0 && L.status == 0) L.status = status;
 }
 
+__global__ void k_recip(const double *a, double *r, int64_t n)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        r[i] = 1.0 / a[i];
+}
+
+// The mass B (component 6 of the element-blocked geometry) as an E-vector.
+__global__ void k_take_B(const double *__restrict__ geo, double *__restrict__ out, int n3, int64_t n)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = i / n3;
+        out[i] = geo[(e * 7 + 6) * n3 + (i - e * n3)];
+    }
+}
+
+static unsigned vec_grid(int64_t n)
+{
+    const int64_t b = sem_ceil_div(n, 256);
+    return (unsigned)(b < 2048 ? b : 2048);
+}
+
 // FP64 values as float pairs (hi = round(v), lo = round(v - hi)).
 __global__ void k_split_df64(const double *__restrict__ a, df64 *__restrict__ out, int64_t n)
 {
@@ -760,6 +893,16 @@ static unsigned conv_grid(int64_t n)
 {
     const int64_t b = sem_ceil_div(n, 256);
     return (unsigned)(b < 65535 * 8 ? b : 65535 * 8);
+}
+
+// Drops the captured steps; they are captured again when steady steps resume.
+static void graph_drop(sem_tgv *T)
+{
+    for (int r = 0; r < 3; ++r)
+        if (T->graph_state[r] == 1) {
+            cudaGraphExecDestroy(T->graph[r]);
+            T->graph_state[r] = 0;
+        }
 }
 
 // Convective term of history level `level` (stored velocity -> stored C).
@@ -881,6 +1024,7 @@ static Coef coef(int q, double h0, double h1, double h2)
     Coef k;
     memset(&k, 0, sizeof(k));
     k.dt = h0;
+    k.rdt = 1.0 / h0;
     const bool equal = h1 == h0 && (q < 3 || h2 == h0);
     if (q == 1) { k.b0 = 1.0; k.b[0] = 1.0; k.a[0] = 1.0; }
     else if (q == 2 && equal) { k.b0 = 1.5; k.b[0] = 2.0; k.b[1] = -0.5; k.a[0] = 2.0; k.a[1] = -1.0; }
@@ -913,7 +1057,9 @@ static GapInv gap_inv(const sem_ctx *c)
     for (int i = 0; i <= N; ++i) {
         const double l = i > 0 ? c->hxi[i] - c->hxi[i - 1] : 1e300;
         const double r = i < N ? c->hxi[i + 1] - c->hxi[i] : 1e300;
-        g.v[i] = 1.0 / (l < r ? l : r);
+        const double v = 1.0 / (l < r ? l : r);
+        const float h = (float)v;
+        g.v[i] = {h, (float)(v - (double)h)};
     }
     return g;
 }
@@ -923,12 +1069,16 @@ static int diag(sem_tgv *T, int advance, cudaStream_t s)
     sem_ctx *c = T->c;
     const int blocks = (int)(c->E < 65535 * 16 ? c->E : 65535 * 16);
     // FP64-accurate on the FP32 pipes (J^-1, B and D as float pairs)
-    TGV_DISPATCH(c->n, k_tgv_diag_part<NP, df64><<<blocks, 256, 0, s>>>(
-                           fu(T, 0, 0), fu(T, 0, 1), fu(T, 0, 2), (int)stored32(T), T->jinvdf,
-                           (const df64 *)c->geodf, (const df64 *)c->tabdf, gap_inv(c), T->part, c->E));
+    TGV_DISPATCH(c->n, {
+        static std::atomic<unsigned> attr{0};
+        SEM_CUDA(sem_smem_attr(k_tgv_diag_part<NP>, DiagCfg<NP>::SMEM, attr));
+        k_tgv_diag_part<NP><<<blocks, DiagCfg<NP>::TH, DiagCfg<NP>::SMEM, s>>>(
+            fu(T, 0, 0), fu(T, 0, 1), fu(T, 0, 2), (int)stored32(T), (const dfp *)T->jinvdf, (const dfp *)c->geodf,
+            T->dtabs, gap_inv(c), T->part, c->E);
+    });
     SEM_CHECK_LAUNCH();
     const double V = c->volume;
-    k_tgv_diag_final<<<1, 256, 0, s>>>(T->part, c->E, V, T->dt, T->dev, T->log, advance);
+    k_tgv_diag_final<<<1, 1024, 0, s>>>(T->part, c->E, V, T->dt, T->dev, T->log, advance);
     SEM_CHECK_LAUNCH();
     return SEM_OK;
 }
@@ -947,12 +1097,36 @@ static int pressure_solve(sem_tgv *T, const double *b, double *x, int x_zero, cu
     return rc;
 }
 
-// One step of order q on stream s (capturable).
+// Level l takes the buffers of level l - 1; the oldest level's, which hold the
+// new velocity (and are free for the next convective term), become level 0.
+static void shift_histories(sem_tgv *T)
+{
+    auto turn = [](auto &h) {
+        for (int cc = 0; cc < 3; ++cc) {
+            auto *last = h[2][cc];
+            h[2][cc] = h[1][cc];
+            h[1][cc] = h[0][cc];
+            h[0][cc] = last;
+        }
+    };
+    turn(T->u);
+    turn(T->C);
+    turn(T->u32);
+    turn(T->C32);
+    T->turn = (T->turn + 1) % 3;
+}
+
+static void unshift_histories(sem_tgv *T)
+{
+    shift_histories(T);
+    shift_histories(T);
+}
+
+// One step of order q on stream s (capturable); shifts the histories.
 static int step_once(sem_tgv *T, int q, cudaStream_t s)
 {
     sem_ctx *c = T->c;
     const int64_t nL = c->nL;
-    const size_t bytes = sizeof(double) * nL;
     const Coef k = coef(q, T->dt, T->hist_dt[0], T->hist_dt[1]);
     int rc;
     const int s32 = stored32(T);
@@ -976,10 +1150,11 @@ static int step_once(sem_tgv *T, int q, cudaStream_t s)
         for (int l = 0; l < 3; ++l) ga.u[l][cc] = fu(T, l, cc);
     }
     ga.s32 = s32;
-    ga.geo64 = c->geo64;
-    ga.gs = sem_gs_desc(c);
+    ga.bsum = T->bsum;
+    ga.binv = T->binv;
+    ga.mesh = uq_mesh(sem_gs_desc(c));
     ga.k = k;
-    k_tgv_g<<<(unsigned)sem_ceil_div(c->nG, 256), 256, 0, s>>>(ga);
+    TGV_DISPATCH(c->n, k_tgv_g<NP><<<(uq_units<NP>(ga.mesh) + 255) / 256, 256, 0, s>>>(ga));
     SEM_CHECK_LAUNCH();
     // 4. pressure: weak divergence, dssum, Poisson solve from p^n
     const int blocks = (int)(c->E < 65535 * 16 ? c->E : 65535 * 16);
@@ -1003,56 +1178,44 @@ static int step_once(sem_tgv *T, int q, cudaStream_t s)
     else
         k_tgv_log_iters<<<1, 32, 0, s>>>(st0, stride, io, so, serr, 0, 1, T->dev, T->log, 1);
     SEM_CHECK_LAUNCH();
-    // 5. velocity right-hand sides and the three Helmholtz solves (from the extrapolated velocity)
+    // 5. velocity right-hand sides and the three Helmholtz solves, which start
+    // from the extrapolated velocity.  FP64 histories: the oldest level, which
+    // the step drops, becomes the iterate in place; FP32 histories: a buffer of
+    // its own, rounded into the oldest level afterwards.
     VArgs va;
+    double *xx[3];
+    const double *bb[3] = {T->rhs[0], T->rhs[1], T->rhs[2]};
     for (int cc = 0; cc < 3; ++cc) {
+        xx[cc] = s32 ? T->unew[cc] : T->u[2][cc];
         va.F[cc] = T->F[cc];
         va.rhs[cc] = T->rhs[cc];
+        va.x[cc] = xx[cc];
         for (int l = 0; l < 3; ++l) va.u[l][cc] = fu(T, l, cc);
     }
     va.s32 = s32;
     va.p = T->p;
     va.jinv = c->jinv64;
     va.geo64 = c->geo64;
-    va.D = c->tab64 + 2 * c->n;
     va.k = k;
     va.E = c->E;
-    TGV_DISPATCH(c->n, k_tgv_vrhs<NP><<<blocks, 256, 0, s>>>(va));
+    TGV_DISPATCH(c->n, k_tgv_vel<NP><<<blocks, VelCfg<NP>::TH, 0, s>>>(va, T->veld));
     SEM_CHECK_LAUNCH();
-    for (int cc = 0; cc < 3; ++cc) {
-        rc = sem_dssum_dev(c, T->rhs[cc], SEM_F64, s);
-        if (rc) return rc;
-    }
-    // the solves start from the extrapolated velocity (EXT weights of the step)
-    XArgs xa;
-    for (int cc = 0; cc < 3; ++cc) {
-        xa.x[cc] = T->unew[cc];
-        for (int l = 0; l < 3; ++l) xa.u[l][cc] = fu(T, l, cc);
-    }
-    xa.s32 = s32;
-    k_tgv_ext<<<(unsigned)sem_ceil_div(nL, 256), 256, 0, s>>>(xa, k, nL);
-    SEM_CHECK_LAUNCH();
-    const double *bb[3] = {T->rhs[0], T->rhs[1], T->rhs[2]};
-    double *xx[3] = {T->unew[0], T->unew[1], T->unew[2]};
+    void *const rh[3] = {T->rhs[0], T->rhs[1], T->rhs[2]};
+    rc = sem_dssum_dev_n(c, 3, rh, SEM_F64, s);
+    if (rc) return rc;
     // (workspace slots 5-7; slot 4 keeps the pressure's Jacobi inverse between steps)
     rc = sem_pcg_solve_dev_batch(c, 3, bb, xx, T->nu, k.b0 / T->dt, T->vo, s, 5, !T->psolver);
     if (rc) return rc;
     k_tgv_log_iters<<<1, 32, 0, s>>>(st0, stride, io, so, serr, 1, 3, T->dev, T->log, 0);
     SEM_CHECK_LAUNCH();
-    // 6. shift histories (copies keep every buffer address fixed for graph replay)
-    const size_t sbytes = (s32 ? sizeof(float) : sizeof(double)) * nL;
-    for (int cc = 0; cc < 3; ++cc) {
-        SEM_CUDA(cudaMemcpyAsync(fu(T, 2, cc), fu(T, 1, cc), sbytes, cudaMemcpyDeviceToDevice, s));
-        SEM_CUDA(cudaMemcpyAsync(fu(T, 1, cc), fu(T, 0, cc), sbytes, cudaMemcpyDeviceToDevice, s));
-        if (s32) {  // the new velocity, rounded to FP32 where it is stored
-            k_conv_f64_f32<<<conv_grid(nL), 256, 0, s>>>(T->unew[cc], T->u32[0][cc], nL);
+    // 6. the histories shift by exchanging buffers (advance replays one captured
+    // graph per arrangement)
+    if (s32)
+        for (int cc = 0; cc < 3; ++cc) {  // the new velocity, rounded to FP32 where it is stored
+            k_conv_f64_f32<<<conv_grid(nL), 256, 0, s>>>(T->unew[cc], T->u32[2][cc], nL);
             SEM_CHECK_LAUNCH();
-        } else {
-            SEM_CUDA(cudaMemcpyAsync(T->u[0][cc], T->unew[cc], bytes, cudaMemcpyDeviceToDevice, s));
         }
-        SEM_CUDA(cudaMemcpyAsync(fC(T, 2, cc), fC(T, 1, cc), sbytes, cudaMemcpyDeviceToDevice, s));
-        SEM_CUDA(cudaMemcpyAsync(fC(T, 1, cc), fC(T, 0, cc), sbytes, cudaMemcpyDeviceToDevice, s));
-    }
+    shift_histories(T);
     return diag(T, 1, s);
 }
 
@@ -1060,11 +1223,12 @@ extern "C" void sem_tgv_destroy(sem_tgv *T)
 {
     if (!T) return;
     cudaDeviceSynchronize();
-    if (T->graph_state == 1) cudaGraphExecDestroy(T->graph);
+    graph_drop(T);
     proj_free(T);
     if (T->block) cudaFree(T->block);
     if (T->block32) cudaFree(T->block32);
     if (T->part) cudaFree(T->part);
+    if (T->bsum) cudaFree(T->bsum);
     if (T->tab64) cudaFree(T->tab64);
     if (T->tab32) cudaFree(T->tab32);
     if (T->tabdf) cudaFree(T->tabdf);
@@ -1129,6 +1293,16 @@ extern "C" int sem_tgv_init(sem_ctx *c, double nu, double dt, sem_dtype op, cons
     T->bp = b; b += nL;
     for (int k = 0; k < 3; ++k) { T->rhs[k] = b; b += nL; }
     TGV_TRY(cudaMalloc(&T->part, sizeof(double) * 3 * c->E));
+    TGV_TRY(cudaMalloc(&T->bsum, sizeof(double) * 2 * nL));
+    T->binv = T->bsum + nL;
+    k_take_B<<<vec_grid(nL), 256>>>(c->geo64, T->bsum, n * n * n, nL);
+    TGV_TRY(cudaGetLastError());
+    {
+        const int rc = sem_dssum_dev(c, T->bsum, SEM_F64, 0);
+        if (rc) { sem_tgv_destroy(T); return rc; }
+    }
+    k_recip<<<vec_grid(nL), 256>>>(T->bsum, T->binv, nL);
+    TGV_TRY(cudaGetLastError());
     // dealiasing tables
     double eta[64], wq[64], J[64 * SEM_NPMAX], h64[2 * 64 + 64 * SEM_NPMAX];
     float h32[2 * 64 + 64 * SEM_NPMAX];
@@ -1151,6 +1325,8 @@ extern "C" int sem_tgv_init(sem_ctx *c, double nu, double dt, sem_dtype op, cons
         TGV_TRY(cudaMalloc(&T->tabdf, sizeof(df64) * ntab));
         TGV_TRY(cudaMemcpy(T->tabdf, hdf, sizeof(df64) * ntab, cudaMemcpyHostToDevice));
     }
+    ax_dfl_tables(n, c->hD, &T->dtabs);
+    memcpy(T->veld.d, c->hD, sizeof(double) * n * n);
     TGV_TRY(cudaMalloc(&T->log, sizeof(TgvLogEntry) * TGV_LOG));
     TGV_TRY(cudaMemset(T->log, 0, sizeof(TgvLogEntry) * TGV_LOG));
     TGV_TRY(cudaMallocHost(&T->hlog, sizeof(TgvLogEntry) * TGV_LOG));
@@ -1344,22 +1520,10 @@ __global__ void k_proj_inc(int *pint, const double *nrm)
     if (nrm[1] > 1e-20 * nrm[0] && nrm[1] > 0.0) pint[0] += 1;
 }
 
-__global__ void k_recip_inplace(double *a, int64_t n)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        a[i] = 1.0 / a[i];
-}
-
 __global__ void k_fill(double *a, double v, int64_t n)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         a[i] = v;
-}
-
-static unsigned vec_grid(int64_t n)
-{
-    const int64_t b = sem_ceil_div(n, 256);
-    return (unsigned)(b < 2048 ? b : 2048);
 }
 
 // c[0..L) = <X_k, v> (assembled), L from *Ld.
@@ -1431,11 +1595,8 @@ extern "C" int sem_tgv_set_projection(sem_tgv *T, int max_vectors)
     if (!T || max_vectors < 0 || max_vectors > TGV_PMAX) return SEM_ERR_ARG;
     SEM_CUDA(cudaDeviceSynchronize());
     proj_free(T);
-    if (T->graph_state == 1) {
-        cudaGraphExecDestroy(T->graph);
-        T->graph_state = 0;
-        T->graph_warm = 0;
-    }
+    graph_drop(T);
+    T->graph_warm = 0;
     if (max_vectors == 0) return SEM_OK;
     sem_ctx *c = T->c;
     const int64_t n = c->nL;
@@ -1460,7 +1621,7 @@ extern "C" int sem_tgv_set_projection(sem_tgv *T, int max_vectors)
     SEM_CHECK_LAUNCH();
     int rc = sem_dssum_dev(c, T->pw, SEM_F64, 0);
     if (rc) return rc;
-    k_recip_inplace<<<vec_grid(n), 256>>>(T->pw, n);
+    k_recip<<<vec_grid(n), 256>>>(T->pw, T->pw, n);
     SEM_CHECK_LAUNCH();
     SEM_CUDA(cudaDeviceSynchronize());
     T->proj_max = max_vectors;
@@ -1530,10 +1691,7 @@ static int apply_policy(sem_tgv *T, int step, cudaStream_t s)
         T->po.inner = T->rules[r].pres;
         T->storage = T->rules[r].storage;
     }
-    if (T->graph_state == 1) {
-        cudaGraphExecDestroy(T->graph);
-        T->graph_state = 0;
-    }
+    graph_drop(T);
     T->graph_warm = 0;
     T->cur_rule = r;
     if (was32 != stored32(T)) return move_storage(T, stored32(T), s);
@@ -1552,29 +1710,31 @@ static int advance(sem_tgv *T, int nsteps, cudaStream_t s)
                             T->hist_dt[1] == T->dt;
         int rc = apply_policy(T, T->step + 1, s);
         if (rc) return rc;
-        if (steady && s != 0 && T->graph_state == 0 && !T->graph_warm) {
+        const int r = T->turn;
+        if (steady && s != 0 && T->graph_state[r] == 0 && !T->graph_warm) {
             // one steady step runs directly first, so the Jacobi inverses of its
-            // solves are cached when the next one is captured (the graph then
-            // keeps reusing them)
+            // solves are cached when the next ones are captured (the graphs then
+            // keep reusing them)
             T->graph_warm = 1;
-        } else if (steady && s != 0 && T->graph_state == 0) {
-            // capture one steady-state step; fall back to direct launches if capture fails
+        } else if (steady && s != 0 && T->graph_state[r] == 0) {
+            // capture one steady-state step of this arrangement of the history
+            // buffers; fall back to direct launches if capture fails
             cudaGraph_t g = nullptr;
-            T->graph_state = -1;
+            T->graph_state[r] = -1;
             if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
                 rc = step_once(T, 3, s);
+                if (T->turn != r) unshift_histories(T);  // (nothing has run yet)
                 cudaError_t ce = cudaStreamEndCapture(s, &g);
                 if (rc == SEM_OK && ce == cudaSuccess && g &&
-                    cudaGraphInstantiate(&T->graph, g, 0) == cudaSuccess) {
-                    T->graph_state = 1;
-                    T->graph_stream = s;
-                }
+                    cudaGraphInstantiate(&T->graph[r], g, 0) == cudaSuccess)
+                    T->graph_state[r] = 1;
                 if (g) cudaGraphDestroy(g);
             }
             cudaGetLastError();
         }
-        if (steady && T->graph_state == 1) {
-            SEM_CUDA(cudaGraphLaunch(T->graph, s));
+        if (steady && T->graph_state[r] == 1) {
+            SEM_CUDA(cudaGraphLaunch(T->graph[r], s));
+            shift_histories(T);
         } else {
             rc = step_once(T, q, s);
             if (rc) return rc;
@@ -1606,10 +1766,7 @@ extern "C" int sem_tgv_set_pressure_solver(sem_tgv *T, int kind, int restart, se
 {
     if (!T || kind < 0 || kind > 1) return SEM_ERR_ARG;
     if (kind == 1 && (restart < 1 || restart > 64 || (vcycle != SEM_F32 && vcycle != SEM_F64))) return SEM_ERR_ARG;
-    if (T->graph_state == 1) {
-        cudaGraphExecDestroy(T->graph);
-        T->graph_state = 0;
-    }
+    graph_drop(T);
     T->graph_warm = 0;
     SEM_CUDA(cudaDeviceSynchronize());
     sem_hsmg_destroy(T->hsmg);
@@ -1633,11 +1790,10 @@ extern "C" int sem_tgv_set_dt(sem_tgv *T, double dt, double cfl_target, double d
     if (dt > 0) T->dt = dt;
     T->cfl_target = cfl_target;
     T->dt_max = dt_max;
-    if (T->graph_state == 1 && (dt > 0 || cfl_target > 0)) {  // the graph holds the old step's coefficients
-        cudaGraphExecDestroy(T->graph);
-        T->graph_state = 0;
+    if (dt > 0 || cfl_target > 0) {  // the graphs hold the old step's coefficients
+        graph_drop(T);
+        T->graph_warm = 0;
     }
-    if (dt > 0 || cfl_target > 0) T->graph_warm = 0;
     return SEM_OK;
 }
 
