@@ -62,13 +62,3 @@ __device__ __forceinline__ int gs_copies(const GsDesc &d, int64_t g, int64_t idx
     return m;
 }
 
-// Multiplicity of local node (i, j, k) of element (ex, ey, ez).
-__device__ __forceinline__ int gs_mult_local(const GsDesc &d, int ex, int ey, int ez, int i, int j,
-                                             int k)
-{
-    int m = 1;
-    if ((i == 0 && (d.px || ex > 0)) || (i == d.N && (d.px || ex < d.nelx - 1))) m *= 2;
-    if ((j == 0 && (d.py || ey > 0)) || (j == d.N && (d.py || ey < d.nely - 1))) m *= 2;
-    if ((k == 0 && (d.pz || ez > 0)) || (k == d.N && (d.pz || ez < d.nelz - 1))) m *= 2;
-    return m;
-}
