@@ -37,9 +37,16 @@ static const ordered_fn k_ordered[3] = {sem_solve_ordered_c, sem_solve_ordered_a
 static const ordered_tab_fn k_ordered_tab[3] = {sem_solve_ordered_tables_c, sem_solve_ordered_tables_a,
                                                 sem_solve_ordered_tables_b};
 
+// The ordered solver's constant memory (even N + 1 <= 10), as sem_solve_upload_tables;
+// at stepper setup, since only its steps use it.
+int sem_solve_upload_ordered(const sem_ctx *c)
+{
+    return c->n % 2 == 0 && c->n <= 10 ? k_ordered_tab[c->n % 3](c->n, c->hD) : SEM_OK;
+}
+
 // Fills the constant memory of the solver kernels that serve the context's
-// order (the per-order unit, for N + 1 in {6, 8, 10} the mixed-order unit and
-// for even N + 1 <= 10 the ordered solver's) with the tables made from its derivative matrix, on the current device.
+// order (the per-order unit and, for N + 1 in {6, 8, 10}, the mixed-order
+// unit) with the tables made from its derivative matrix, on the current device.
 int sem_solve_upload_tables(const sem_ctx *c)
 {
     typedef int (*tab_fn)(const double *);
@@ -52,7 +59,6 @@ int sem_solve_upload_tables(const sem_ctx *c)
     if (c->n < 2 || c->n > 16) return SEM_ERR_ARG;
     int rc = f[c->n](c->hD);
     if (rc == SEM_OK && (c->n == 6 || c->n == 8 || c->n == 10)) rc = sem_solve_tables_multi(c->n, c->hD);
-    if (rc == SEM_OK && c->n % 2 == 0 && c->n <= 10) rc = k_ordered_tab[c->n % 3](c->n, c->hD);
     return rc;
 }
 

@@ -40,6 +40,7 @@
 GsDesc sem_gs_desc(const sem_ctx *c);
 int sem_run_geometry(sem_ctx *c, double *xyz, bool with_jinv, cudaStream_t s);
 int sem_alloc_ws(sem_ctx *c, int slot);
+int sem_solve_upload_ordered(const sem_ctx *c);
 int sem_dssum_dev(sem_ctx *c, void *u, sem_dtype dt, cudaStream_t s);
 int sem_dssum_dev_n(sem_ctx *c, int n, void *const *u, sem_dtype dt, cudaStream_t s);
 int sem_ax_dev_columns(sem_ctx *c, const double *u, double *w, double h1, double h2, cudaStream_t s);
@@ -1326,6 +1327,10 @@ extern "C" int sem_tgv_init(sem_ctx *c, double nu, double dt, sem_dtype op, cons
         TGV_TRY(cudaMemcpy(T->tabdf, hdf, sizeof(df64) * ntab, cudaMemcpyHostToDevice));
     }
     ax_dfl_tables(n, c->hD, &T->dtabs);
+    {
+        const int rc = sem_solve_upload_ordered(c);
+        if (rc) { sem_tgv_destroy(T); return rc; }
+    }
     memcpy(T->veld.d, c->hD, sizeof(double) * n * n);
     TGV_TRY(cudaMalloc(&T->log, sizeof(TgvLogEntry) * TGV_LOG));
     TGV_TRY(cudaMemset(T->log, 0, sizeof(TgvLogEntry) * TGV_LOG));
