@@ -7,8 +7,8 @@
 // operator's quantisation, one changed bit in 1e-4 of the velocities moves the
 // pressure of the next step by 1e-10 of itself, and a small velocity component
 // by 2e-9 to 8e-9 (N = 7, 24^3 and 32^3 elements; 8e-8 at N = 8).  The solver of
-// solver.cuh takes half the time (5.4 ms a launch against 11 at 32^3, N = 7) but
-// sums in another order; runs that are to repeat to 1e-9 therefore keep this one.
+// solver.cuh is faster (5.4 ms a launch against 6.8 at 32^3, N = 7; half the
+// time at 16^3) but sums in another order; runs that are to repeat to 1e-9 therefore keep this one.
 // Solves whose tolerance ends the iteration on the solution itself, and steps
 // with GMRES, whose iterates agree to 1e-10 either way, use solver.cuh.
 //
