@@ -219,8 +219,9 @@ struct TcSplitCfg {
     static constexpr int NP2 = NP * NP, NP3 = NP2 * NP;
     static constexpr int MT = (NP2 + 15) / 16;
     static constexpr int NE = 8;  // one element per warp, 256-thread blocks
-    // gradient slabs (3 NP^3 floats), output accumulator (NP^3 floats), three 16-bit parts
-    static constexpr size_t PER_ELEM = (size_t)NP3 * 4 * 4 + (size_t)NP3 * 2 * 3;
+    // gradient slabs (3 NP^3 floats), output accumulator (NP^3 floats), three 16-bit parts,
+    // rounded up so that the next warp's floats are aligned (odd NP: 22 NP^3 is not a multiple of 4)
+    static constexpr size_t PER_ELEM = ((size_t)NP3 * 4 * 4 + (size_t)NP3 * 2 * 3 + 15) / 16 * 16;
     static constexpr bool OK = NP <= 8;
 };
 
