@@ -36,7 +36,8 @@ void sem_note_cuda_error(cudaError_t e, const char *where);
 struct sem_ws {
     double *r, *p, *w, *minv, *b;   // FP64 E-vectors (b: the sum of the corrections of a solve)
     float *r32, *p32, *w32, *d32, *minv32;
-    // minv (and minv32) hold the Jacobi inverse of (jac_h1, jac_h2) when jac_ok (jac32_ok)
+    // a launch was enqueued that leaves the Jacobi inverse of (jac_h1, jac_h2) in minv when
+    // jac_ok (in minv32 too when jac32_ok); whether it got that far: sem_ctx::jac_dev
     double jac_h1, jac_h2;
     int jac_ok, jac32_ok;
 };
@@ -66,6 +67,8 @@ struct sem_ctx {
     float *jinv32;
     // solver workspaces (slot 0 allocated at setup)
     int nws;              // (unused)
+    unsigned *jac_dev;    // device word of each workspace: bit 0 minv, bit 1 minv32 hold a whole inverse
+                          // (behind err_dev, in its allocation)
     sem_ws ws[8];         // 0-3: solves through the API; 4-7: the Taylor-Green stepper's own
                           // (allocated on first use; a slot is allocated when its r is set)
     // device-side solve state + pinned host mirror of the last solve's info

@@ -124,13 +124,15 @@ static bool share_jacobi(const ProbDesc &q, ProbDesc &d, const sem_ctx *cq, cons
     d.minv = q.minv;
     d.minv32 = q.minv32;
     d.jac_cached = q.jac_cached;
-    d.jac_shared = !q.jac_cached;
+    d.jac_dev = q.jac_dev;
+    d.jac_shared = 1;
     return true;
 }
 
 // Fills d for a solve on workspace ws; the Jacobi inverse is recomputed unless
 // ws still holds the one of (h1, h2) (and its FP32 copy when mixed), and ws
-// records what the launch leaves in minv / minv32.  first .. first + nfirst:
+// records what the launch leaves in minv / minv32 (the launch that finds them
+// incomplete, because the one that was to make them timed out, makes them).  first .. first + nfirst:
 // the launch's earlier problems and their contexts, one of which may share its
 // Jacobi inverse.
 static void fill_desc(const sem_ctx *c, sem_ws &ws, const double *b, double *x, double h1,
@@ -172,6 +174,7 @@ static void fill_desc(const sem_ctx *c, sem_ws &ws, const double *b, double *x, 
         d.d32 = ws.d32;
         d.minv32 = ws.minv32;
     }
+    d.jac_dev = c->jac_dev + (&ws - c->ws);
     for (int q = 0; q < nfirst; ++q)
         if (share_jacobi(first[q], d, fctx[q], c)) return;
     d.jac_cached = ws.jac_ok && ws.jac_h1 == h1 && ws.jac_h2 == h2 && (!mixed || ws.jac32_ok);
@@ -429,6 +432,10 @@ extern "C" int sem_pcg_solve_batched(int nprob, sem_ctx *const *ctxs, const doub
     // other order mixes: one launch per problem, in order
     int worst = SEM_OK;
     for (int p = 0; p < nprob; ++p) {
+        if (d[p].jac_shared) {  // made by an earlier launch, or again by this one
+            d[p].jac_shared = 0;
+            d[p].jac_cached = 1;
+        }
         rc = enqueue(owner, o, &d[p], 1, s);
         if (rc) {
             for (int q = 0; q < nprob; ++q) jac_forget(ctxs[q], rc);

@@ -403,8 +403,9 @@ extern "C" int sem_setup(int N, int nelx, int nely, int nelz, const double exten
     SETUP_TRY(cudaMemset(c->solve_dev, 0, sem_solve_state_bytes()));
     SETUP_TRY(cudaMallocHost(&c->solve_host, sem_solve_state_bytes()));
     SETUP_TRY(cudaMalloc(&c->partials, sem_partials_bytes(c->num_sms)));
-    SETUP_TRY(cudaMalloc(&c->err_dev, sizeof(int)));
-    SETUP_TRY(cudaMemset(c->err_dev, 0, sizeof(int)));
+    SETUP_TRY(cudaMalloc(&c->err_dev, 9 * sizeof(int)));
+    SETUP_TRY(cudaMemset(c->err_dev, 0, 9 * sizeof(int)));
+    c->jac_dev = (unsigned *)c->err_dev + 1;
     memset(c->solve_host, 0, sem_solve_state_bytes());
     SETUP_TRY(cudaDeviceSynchronize());
 #undef SETUP_TRY

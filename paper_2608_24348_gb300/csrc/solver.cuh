@@ -87,9 +87,10 @@ struct ProbDesc {
     int n, NE, NE32, singular;  // NE: elements per group (CUDA cores); NE32: inner operator
     int tc;                     // inner path of a MODE_TC launch: 0 FP32 CUDA cores, 1 BF16, 2 FP16,
                                 // 3 FP16 x2, 4 BF16 x3 tensor cores
-    int jac_cached;             // minv (and minv32 if mixed) already hold this problem's Jacobi inverse
+    int jac_cached;             // an earlier launch was to leave this problem's Jacobi inverse in minv
+                                // (and minv32 if mixed); *jac_dev says whether it did
     int vec;                    // b and x are aligned for vector accesses
-    int jac_shared;             // an earlier problem of the launch makes the Jacobi inverse in minv
+    int jac_shared;             // an earlier problem of the launch makes (or keeps) the inverse in minv
     int64_t E, nL, nG;
     UqMesh mesh;
     FastDiv dn3;
@@ -104,11 +105,13 @@ struct ProbDesc {
     double *x;
     double *r, *p, *w, *minv;
     double *y;          // the sum of the corrections; null: x is updated in every iteration instead
+    unsigned *jac_dev;  // bit 0: minv, bit 1: minv32 hold a whole inverse (null: never kept)
     float *r32, *p32, *w32, *d32, *minv32;
 };
 
 struct PState {
     int phase, iters, outer, inner_iters, status, first;
+    int jac;  // the Jacobi inverse was there when the launch began
     double rz, alpha, beta, bnorm, rnorm, target, bmean, scale, prev_rnorm, inner_target, shift;
 };
 
@@ -157,6 +160,15 @@ __device__ __forceinline__ void red_release_add_u32(unsigned *p, unsigned v)
 __device__ __forceinline__ bool phase_pairs(int ph)
 {
     return ph == PH_A32 || ph == PH_C32 || ph == PH_INIT32;
+}
+
+// Bits of *P.jac_dev that a solve of P needs and a whole JACGS phase leaves.  A
+// launch that times out before that leaves zero: the next one makes the inverse.
+__device__ __forceinline__ unsigned jac_bits(const ProbDesc &P) { return P.minv32 ? 3u : 1u; }
+
+__device__ __forceinline__ bool jac_kept(const ProbDesc &P)
+{
+    return P.jac_cached && (*(const volatile unsigned *)P.jac_dev & jac_bits(P)) == jac_bits(P);
 }
 
 __host__ __device__ __forceinline__ int phase_nvals(int ph)
@@ -816,7 +828,7 @@ __device__ __forceinline__ void uniq_item(const ProbDesc &P, const PState &S, in
 #pragma unroll
             for (int i = 0; i < CH; ++i)
                 if (i < U.own) v[0] += __ldcg(P.b + U.f + i);
-        if (P.jac_cached || P.jac_shared) return;  // only the sum of b
+        if (S.jac || P.jac_shared) return;  // only the sum of b
         double s[CH];
         uq_gather(P.minv, U, s, [] {});
 #pragma unroll
@@ -1117,9 +1129,12 @@ __global__ void __launch_bounds__(TH, TH > SEM_SOLVE_THREADS ? 1 : 2)
         PState S;
         memset(&S, 0, sizeof(S));
         const ProbDesc &P = prm.prob[p];
+        S.jac = jac_kept(P);
         // (the sum of b that JACGS makes is only needed to remove its mean)
-        S.phase = !P.jac_cached ? PH_JAC : P.singular ? PH_JACGS : PH_AX0;
+        S.phase = !S.jac ? PH_JAC : P.singular ? PH_JACGS : PH_AX0;
         s_st[p] = S;
+        // (CTAs that read the word after this find it incomplete as well)
+        if (blockIdx.x == 0 && !S.jac && !P.jac_shared && P.jac_dev) *P.jac_dev = 0u;
     }
     if (threadIdx.x == 0) s_step = 0;
     __syncthreads();
@@ -1245,7 +1260,13 @@ __global__ void __launch_bounds__(TH, TH > SEM_SOLVE_THREADS ? 1 : 2)
         }
         __syncthreads();
         for (int p = threadIdx.x; p < np; p += TH)
-            if (s_st[p].phase != PH_DONE) advance<MAXP>(prm, prm.prob[p], s_st[p], s_sum[p]);
+            if (s_st[p].phase != PH_DONE) {
+                const ProbDesc &P = prm.prob[p];
+                // (every CTA has read the word before its first barrier)
+                if (blockIdx.x == 0 && s_st[p].phase == PH_JACGS && !s_st[p].jac && !P.jac_shared && P.jac_dev)
+                    *P.jac_dev = jac_bits(P);
+                advance<MAXP>(prm, P, s_st[p], s_sum[p]);
+            }
         if (threadIdx.x == 0) s_step += 1;
         __syncthreads();
     }

@@ -240,7 +240,7 @@ __device__ __forceinline__ void uniq_item(const ProbDesc &P, const PState &S, in
     }
     switch (ph) {
         case PH_JACGS: {
-            if (P.jac_cached) {  // the Jacobi inverse is kept from an earlier solve: only sum b
+            if (S.jac) {  // the Jacobi inverse is kept from an earlier solve: only sum b
 #pragma unroll
                 for (int r = 0; r < RU; ++r)
                     if (ok[r]) v[0] += __ldcg(P.b + R[r].off[0] + xo[0]);
@@ -412,7 +412,7 @@ __global__ void __launch_bounds__(SEM_SOLVE_THREADS, 2)
     __shared__ int s_phase[MAXP];
     __shared__ long long s_offs[MAXP + 1];
     __shared__ double s_alpha[MAXP], s_beta[MAXP], s_bmean[MAXP], s_shift[MAXP];
-    __shared__ int s_first[MAXP];
+    __shared__ int s_first[MAXP], s_jac[MAXP];
     __shared__ int s_last, s_stop;
     __shared__ unsigned s_gen;
     const int np = prm.nprob;
@@ -427,7 +427,11 @@ __global__ void __launch_bounds__(SEM_SOLVE_THREADS, 2)
             for (int p = 0; p < np; ++p) {
                 int ph;
                 if (step == 0) {
-                    ph = prm.prob[p].jac_cached ? PH_JACGS : PH_JAC;
+                    const ProbDesc &P = prm.prob[p];
+                    s_jac[p] = jac_kept(P);
+                    ph = s_jac[p] ? PH_JACGS : PH_JAC;
+                    // (CTAs that read the word after this find it incomplete as well)
+                    if (blockIdx.x == 0 && !s_jac[p]) *P.jac_dev = 0u;
                 } else {
                     ph = ((volatile PState *)prm.st)[p].phase;
                 }
@@ -475,6 +479,7 @@ __global__ void __launch_bounds__(SEM_SOLVE_THREADS, 2)
             S.beta = s_beta[p];
             S.bmean = s_bmean[p];
             S.shift = s_shift[p];
+            S.jac = s_jac[p];
             if (ph == PH_AX0) {
                 elem_item<NP, 0>(P, 0.0, 0.0, 1, local, smem, acc);
             } else if (ph == PH_A) {
@@ -518,6 +523,8 @@ __global__ void __launch_bounds__(SEM_SOLVE_THREADS, 2)
             for (int p = threadIdx.x; p < np; p += blockDim.x) {
                 PState S = prm.st[p];
                 S.phase = s_phase[p];
+                // (every CTA has read the word before it arrived here)
+                if (S.phase == PH_JACGS && !s_jac[p]) *prm.prob[p].jac_dev = jac_bits(prm.prob[p]);
                 advance(prm, prm.prob[p], S, s_part[p]);
                 prm.st[p] = S;
             }
