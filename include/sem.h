@@ -206,7 +206,8 @@ SEM_API int sem_jacobi(sem_ctx *ctx, double h1, double h2, double *minv, void *s
  * maxit bounds the PCG iterations (total inner iterations for refinement),
  * max_outer the refinement steps.  wait_timeout_s bounds every device-side
  * wait of the persistent solver (<= 0 selects 10 s); when one runs out the
- * solve ends with SEM_ERR_TIMEOUT and the context stays usable. */
+ * solve ends with SEM_ERR_TIMEOUT, x holds an iterate that may be an earlier one
+ * than iters and final_rnorm speak of, and the context stays usable. */
 typedef struct {
     double tol;
     int abs_tol;

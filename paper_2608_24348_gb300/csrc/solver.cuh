@@ -112,6 +112,7 @@ struct ProbDesc {
 struct PState {
     int phase, iters, outer, inner_iters, status, first;
     int jac;  // the Jacobi inverse was there when the launch began
+    // rnorm: its square while an FP64 solve is between two C phases
     double rz, alpha, beta, bnorm, rnorm, target, bmean, scale, prev_rnorm, inner_target, shift;
 };
 
@@ -1273,7 +1274,12 @@ __global__ void __launch_bounds__(TH, TH > SEM_SOLVE_THREADS ? 1 : 2)
     // the final states, once (after a time-out: the states at the last whole step)
     __syncthreads();
     if (blockIdx.x == 0)
-        for (int p = threadIdx.x; p < np; p += TH) prm.st[p] = s_st[p];
+        for (int p = threadIdx.x; p < np; p += TH) {
+            // (a solve that timed out between two C phases still keeps the norm's square)
+            if ((s_st[p].phase == PH_A || s_st[p].phase == PH_C) && s_st[p].iters > 0)
+                s_st[p].rnorm = sqrt(s_st[p].rnorm);
+            prm.st[p] = s_st[p];
+        }
 }
 
 // Host launcher (cooperative, grid sized for co-residency and no larger than

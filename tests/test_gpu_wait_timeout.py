@@ -36,6 +36,35 @@ def test_later_solve_makes_its_own_preconditioner(sem, inner, info, N):
     assert torch.equal(out[0][1], out[1][1])
 
 
+@pytest.mark.parametrize("inner", ["f64", "f64_native"])
+def test_residual_norm_of_an_interrupted_solve(sem, inner):
+    """The limit is halved between one that stops the solve at once and one that
+    does not stop it, until a solve stops on its way; the norm it reports is that of
+    a solve of as many iterations."""
+    torch, dev = torch_dev()
+    ctx, m, _ = pair(sem, 7, (9, 8, 7), 0.1, with_oracle=False)
+    bg, _ = fourier_rhs(ctx, m)
+    x = torch.zeros_like(bg)
+    lo, hi, info = 1e-9, 1e-3, None
+    for _ in range(60):
+        limit = (lo * hi) ** 0.5
+        x.zero_()
+        d = ctx.pcg_solve(bg, x, 1.0, 0.0, tol=1e-10, inner=inner, wait_timeout_s=limit)
+        if d["status"] != sem.ERR_TIMEOUT:
+            hi = limit
+        elif d["iters"] == 0:
+            lo = limit
+        else:
+            info = d
+            break
+    if info is None:
+        pytest.skip("no limit stopped the solve on its way")
+    x.zero_()
+    ref = ctx.pcg_solve(bg, x, 1.0, 0.0, tol=1e-10, inner=inner, maxit=info["iters"])
+    assert ref["iters"] == info["iters"]
+    assert abs(info["rnorm"] - ref["rnorm"]) <= 1e-9 * ref["rnorm"], (info, ref)
+
+
 @pytest.mark.parametrize("inner", ["f64", "f32"])
 @pytest.mark.parametrize("orders", [(7, 5), (7, 4)])  # one launch; a launch for each problem
 def test_later_batch_makes_its_own_preconditioners(sem, inner, orders):
