@@ -116,6 +116,15 @@ static int inner_tc_of(sem_dtype inner, int n)
     }
 }
 
+// Whether a solve with these options takes the context's order (the tensor-core
+// inner operators end at N + 1 = 10, their split-operand forms at 8).
+bool sem_pcg_accepts(const sem_ctx *c, const sem_solve_opts &o)
+{
+    const bool split = o.inner == SEM_F16X2_TC || o.inner == SEM_BF16X3_TC;
+    const bool tc = split || o.inner == SEM_BF16_TC || o.inner == SEM_F16_TC;
+    return !tc || c->n <= (split ? 8 : 10);
+}
+
 // Problem p on the same context and coefficients as an earlier problem q of the
 // launch takes q's Jacobi inverse instead of making (and keeping) its own.
 static bool share_jacobi(const ProbDesc &q, ProbDesc &d, const sem_ctx *cq, const sem_ctx *c)
@@ -296,10 +305,7 @@ int sem_pcg_solve_dev(sem_ctx *c, int slot, const double *b, double *x, double h
                       const sem_solve_opts &o, cudaStream_t s)
 {
     const bool mixed = o.inner != SEM_F64 && o.inner != SEM_F64_NATIVE;
-    const bool tc = o.inner == SEM_BF16_TC || o.inner == SEM_F16_TC || o.inner == SEM_F16X2_TC ||
-                    o.inner == SEM_BF16X3_TC;  // a tensor-core path was asked for
-    const int tc_nmax = (o.inner == SEM_F16X2_TC || o.inner == SEM_BF16X3_TC) ? 8 : 10;
-    if (tc && c->n > tc_nmax) return SEM_ERR_ARG;
+    if (!sem_pcg_accepts(c, o)) return SEM_ERR_ARG;
     ProbDesc d;
     fill_desc(c, c->ws[slot], b, x, h1, h2, mixed, inner_tc_of(o.inner, c->n), d);
     return jac_forget(c, enqueue(c, o, &d, 1, s));
@@ -314,10 +320,7 @@ int sem_pcg_solve_dev_batch(sem_ctx *c, int np, const double *const *b, double *
     for (int p = 0; p < np; ++p)
         if (!c->ws[slot0 + p].r) return SEM_ERR_ARG;
     const bool mixed = o.inner != SEM_F64 && o.inner != SEM_F64_NATIVE;
-    const bool tc = o.inner == SEM_BF16_TC || o.inner == SEM_F16_TC || o.inner == SEM_F16X2_TC ||
-                    o.inner == SEM_BF16X3_TC;  // a tensor-core path was asked for
-    const int tc_nmax = (o.inner == SEM_F16X2_TC || o.inner == SEM_BF16X3_TC) ? 8 : 10;
-    if (tc && c->n > tc_nmax) return SEM_ERR_ARG;
+    if (!sem_pcg_accepts(c, o)) return SEM_ERR_ARG;
     ordered = ordered && o.inner == SEM_F64 && !tight_f64(o) && c->n <= 10;
     ProbDesc d[8];
     sem_ctx *const cs[8] = {c, c, c, c, c, c, c, c};
@@ -385,9 +388,6 @@ extern "C" int sem_pcg_solve_batched(int nprob, sem_ctx *const *ctxs, const doub
     int rc = validate_opts(o);
     if (rc) return rc;
     const bool mixed = o.inner != SEM_F64 && o.inner != SEM_F64_NATIVE;
-    const bool tc = o.inner == SEM_BF16_TC || o.inner == SEM_F16_TC || o.inner == SEM_F16X2_TC ||
-                    o.inner == SEM_BF16X3_TC;  // a tensor-core path was asked for
-    const int tc_nmax = (o.inner == SEM_F16X2_TC || o.inner == SEM_BF16X3_TC) ? 8 : 10;
     cudaStream_t s = (cudaStream_t)stream;
     std::vector<ProbDesc> d(nprob);
     std::vector<int> slot(nprob, 0);
@@ -395,7 +395,7 @@ extern "C" int sem_pcg_solve_batched(int nprob, sem_ctx *const *ctxs, const doub
         sem_ctx *c = ctxs[p];
         if (!c || !b[p] || !x[p]) return SEM_ERR_ARG;
         if (!(h1[p] >= 0) || !(h2[p] >= 0) || (h1[p] == 0 && h2[p] == 0)) return SEM_ERR_ARG;
-        if (tc && c->n > tc_nmax) return SEM_ERR_ARG;
+        if (!sem_pcg_accepts(c, o)) return SEM_ERR_ARG;
         if (!sem_is_device_ptr(b[p]) || !sem_is_device_ptr(x[p])) return SEM_ERR_ARG;
         for (int q = 0; q < p; ++q) slot[p] += (ctxs[q] == c);
         if (slot[p] >= 4) return SEM_ERR_ARG;

@@ -44,6 +44,7 @@ int sem_solve_upload_ordered(const sem_ctx *c);
 int sem_dssum_dev(sem_ctx *c, void *u, sem_dtype dt, cudaStream_t s);
 int sem_dssum_dev_n(sem_ctx *c, int n, void *const *u, sem_dtype dt, cudaStream_t s);
 int sem_ax_dev_columns(sem_ctx *c, const double *u, double *w, double h1, double h2, cudaStream_t s);
+bool sem_pcg_accepts(const sem_ctx *c, const sem_solve_opts &o);
 int sem_pcg_solve_dev_batch(sem_ctx *c, int np, const double *const *b, double *const *x, double h1,
                             double h2, const sem_solve_opts &o, cudaStream_t s, int slot0, bool ordered);
 const void *sem_solve_state_ptr(const sem_ctx *c, int p, int *iters_off, int *status_off);
@@ -1715,6 +1716,9 @@ static int advance(sem_tgv *T, int nsteps, cudaStream_t s)
                             T->hist_dt[1] == T->dt;
         int rc = apply_policy(T, T->step + 1, s);
         if (rc) return rc;
+        // refused before anything is written: the velocity solves' guess takes the
+        // place of the oldest velocities
+        if (!sem_pcg_accepts(T->c, T->vo) || (!T->psolver && !sem_pcg_accepts(T->c, T->po))) return SEM_ERR_ARG;
         const int r = T->turn;
         if (steady && s != 0 && T->graph_state[r] == 0 && !T->graph_warm) {
             // one steady step runs directly first, so the Jacobi inverses of its

@@ -1,0 +1,59 @@
+"""The stepper's history levels where their buffers turn, are written in place or
+are taken by a graph of the caller's: what a step leaves in them has to be what
+the same steps alone leave, bit for bit."""
+import pytest
+
+from helpers import gpu_coords, pair, torch_dev
+from paper_2608_24348_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _stepper(sem, N=5, nel=(3, 4, 3), **kw):
+    """A stepper in the middle of a run: three different velocity levels."""
+    torch, dev = torch_dev()
+    ctx, _, _ = pair(sem, N, nel, 0.05, with_oracle=False)
+    T = sem.TGV(ctx, 0.02, 4e-3, **kw)
+    x, y, z = gpu_coords(ctx)
+    u, v, w, p = (t + 0 * x for t in inputs.tgv_initial(x, y, z, lib=torch))
+    w = w + 0.2 * torch.sin(x + 2 * y)
+    for level in (2, 1, 0):
+        s = 1.0 + 0.01 * level
+        T.set(s * u, s * v, s * w, p.contiguous() if level == 0 else None, level=level, step=3)
+    return ctx, T
+
+
+def _state(T, ctx):
+    torch, dev = torch_dev()
+    f = [torch.empty(ctx.nL, dtype=torch.float64, device=dev) for _ in range(4)]
+    T.get(*f)
+    return f
+
+
+def _same(a, b):
+    torch, _ = torch_dev()
+    return all(torch.equal(p, q) for p, q in zip(a, b))
+
+
+@pytest.mark.parametrize("which", ["vel", "pres"])
+def test_a_refused_step_leaves_the_state(sem, which):
+    """The split-operand inner operators end at N = 7: a step with them at N = 8 is
+    refused; after a policy that asks for FP64 solves the run goes on as if it had
+    not been tried."""
+    opts = {which: sem.opts(tol=1e-8, inner="f16x2_tc")}
+    other = "pres" if which == "vel" else "vel"
+    opts[other] = sem.opts(tol=1e-8)
+    out = []
+    for tried in (False, True):
+        ctx, T = _stepper(sem, 8, (3, 2, 3), **opts)
+        if tried:
+            before = _state(T, ctx)
+            with pytest.raises(sem.SemError):
+                T.step(1)
+            assert _same(before, _state(T, ctx))
+        T.set_policy([{}])
+        d = T.step(3)
+        assert all(r["status"] == 0 for r in d), d
+        out.append(_state(T, ctx))
+        T.close()
+    assert _same(*out)
