@@ -492,9 +492,14 @@ SEM_API int sem_tgv_set(sem_tgv *tgv, int level, const double *u, const double *
  * ran, with the last iterate of that solve); without diag the call is
  * stream-ordered and returns SEM_OK or a launch error (a CFL-controlled run
  * synchronises once per step).  With a fixed step, from the third step of one
- * size on each step is one CUDA graph replay (captured on the second such step
- * after setup or any policy, projection or step-size change; direct launches
- * if the capture fails) when stream is not NULL.
+ * size on each step is one CUDA graph replay when stream is not NULL: a step has
+ * three graphs, one for each arrangement of the history buffers, captured on the
+ * second to fourth such step after setup or any policy, projection or step-size
+ * change (direct launches if a capture fails).  A caller may capture a call
+ * without diag, with a fixed step and the PCG pressure solver, into a graph of
+ * its own: the step then moves its histories by copies, and each replay of that
+ * graph is the next step (the step count and time that the stepper keeps on the
+ * host do not follow replays).
  * SEM_ERR_ARG: NULL tgv or nsteps < 0. */
 SEM_API int sem_tgv_step(sem_tgv *tgv, int nsteps, sem_tgv_diag *diag, void *stream);
 

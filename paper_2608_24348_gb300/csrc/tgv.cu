@@ -1124,8 +1124,9 @@ static void unshift_histories(sem_tgv *T)
     shift_histories(T);
 }
 
-// One step of order q on stream s (capturable); shifts the histories.
-static int step_once(sem_tgv *T, int q, cudaStream_t s)
+// One step of order q on stream s (capturable); shifts the histories, by exchanging
+// their buffers or (hold) by copies between them.
+static int step_once(sem_tgv *T, int q, cudaStream_t s, bool hold = false)
 {
     sem_ctx *c = T->c;
     const int64_t nL = c->nL;
@@ -1182,13 +1183,13 @@ static int step_once(sem_tgv *T, int q, cudaStream_t s)
     SEM_CHECK_LAUNCH();
     // 5. velocity right-hand sides and the three Helmholtz solves, which start
     // from the extrapolated velocity.  FP64 histories: the oldest level, which
-    // the step drops, becomes the iterate in place; FP32 histories: a buffer of
-    // its own, rounded into the oldest level afterwards.
+    // the step drops, becomes the iterate in place; FP32 histories, or buffers
+    // that are to keep their levels: a buffer of its own, copied afterwards.
     VArgs va;
     double *xx[3];
     const double *bb[3] = {T->rhs[0], T->rhs[1], T->rhs[2]};
     for (int cc = 0; cc < 3; ++cc) {
-        xx[cc] = s32 ? T->unew[cc] : T->u[2][cc];
+        xx[cc] = s32 || hold ? T->unew[cc] : T->u[2][cc];
         va.F[cc] = T->F[cc];
         va.rhs[cc] = T->rhs[cc];
         va.x[cc] = xx[cc];
@@ -1212,6 +1213,22 @@ static int step_once(sem_tgv *T, int q, cudaStream_t s)
     SEM_CHECK_LAUNCH();
     // 6. the histories shift by exchanging buffers (advance replays one captured
     // graph per arrangement)
+    if (hold) {
+        const size_t bytes = (s32 ? sizeof(float) : sizeof(double)) * nL;
+        for (int cc = 0; cc < 3; ++cc) {
+            for (int l = 2; l > 0; --l) {
+                SEM_CUDA(cudaMemcpyAsync(fu(T, l, cc), fu(T, l - 1, cc), bytes, cudaMemcpyDeviceToDevice, s));
+                SEM_CUDA(cudaMemcpyAsync(fC(T, l, cc), fC(T, l - 1, cc), bytes, cudaMemcpyDeviceToDevice, s));
+            }
+            if (s32) {
+                k_conv_f64_f32<<<conv_grid(nL), 256, 0, s>>>(T->unew[cc], T->u32[0][cc], nL);
+                SEM_CHECK_LAUNCH();
+            } else {
+                SEM_CUDA(cudaMemcpyAsync(T->u[0][cc], T->unew[cc], bytes, cudaMemcpyDeviceToDevice, s));
+            }
+        }
+        return diag(T, 1, s);
+    }
     if (s32)
         for (int cc = 0; cc < 3; ++cc) {  // the new velocity, rounded to FP32 where it is stored
             k_conv_f64_f32<<<conv_grid(nL), 256, 0, s>>>(T->unew[cc], T->u32[2][cc], nL);
@@ -1704,15 +1721,29 @@ static int apply_policy(sem_tgv *T, int step, cudaStream_t s)
     return SEM_OK;
 }
 
-// Advance nsteps steps on stream s (no synchronisation).
+// Whether the caller is capturing stream s into a graph.
+static bool stream_capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (s == 0 || cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+// Advance nsteps steps on stream s (no synchronisation).  While the caller
+// captures s the buffers keep their levels: each replay of its graph is then the
+// next step (an exchange on the host would happen once, at the capture).
 static int advance(sem_tgv *T, int nsteps, cudaStream_t s)
 {
+    const bool hold = stream_capturing(s);
     for (int it = 0; it < nsteps; ++it) {
         const int q = T->step + 1 < 3 ? T->step + 1 : 3;
         const bool adaptive = T->cfl_target > 0;
         // graph replay only for third-order steps of one fixed size (and a
         // pressure solver that does not read back to the host)
-        const bool steady = q == 3 && !adaptive && !T->psolver && T->hist_dt[0] == T->dt &&
+        const bool steady = q == 3 && !hold && !adaptive && !T->psolver && T->hist_dt[0] == T->dt &&
                             T->hist_dt[1] == T->dt;
         int rc = apply_policy(T, T->step + 1, s);
         if (rc) return rc;
@@ -1745,7 +1776,7 @@ static int advance(sem_tgv *T, int nsteps, cudaStream_t s)
             SEM_CUDA(cudaGraphLaunch(T->graph[r], s));
             shift_histories(T);
         } else {
-            rc = step_once(T, q, s);
+            rc = step_once(T, q, s, hold);
             if (rc) return rc;
         }
         T->step += 1;

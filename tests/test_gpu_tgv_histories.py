@@ -57,3 +57,56 @@ def test_a_refused_step_leaves_the_state(sem, which):
         out.append(_state(T, ctx))
         T.close()
     assert _same(*out)
+
+
+@pytest.mark.parametrize("storage", ["f64", "f32"])
+@pytest.mark.parametrize("direct", [4, 5])
+def test_replays_of_a_step_captured_by_the_caller(sem, storage, direct):
+    """One captured step replayed five times is five steps, from either arrangement
+    of the history buffers, and the stepper goes on from there."""
+    torch, dev = torch_dev()
+    out = []
+    for captured in (False, True):
+        ctx, T = _stepper(sem, vel=sem.opts(tol=1e-8), pres=sem.opts(tol=1e-8))
+        T.set_policy([{"storage": storage}])
+        st = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        T.step(direct, diag=False, stream=st)
+        if captured:
+            st.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=st):
+                T.step(1, diag=False, stream=st)
+            for _ in range(5):
+                g.replay()
+            torch.cuda.synchronize()
+        else:
+            T.step(5, diag=False, stream=st)
+        T.step(2, diag=False, stream=st)
+        torch.cuda.synchronize()
+        out.append(_state(T, ctx))
+        T.close()
+    assert _same(*out)
+
+
+@pytest.mark.parametrize("storage", ["f64", "f32"])
+@pytest.mark.parametrize("direct", [1, 2, 3])
+def test_levels_set_between_steps(sem, storage, direct):
+    """The levels that sem_tgv_set writes are those the next steps read, from every
+    arrangement of the history buffers."""
+    torch, dev = torch_dev()
+    out = []
+    for before in (0, direct):
+        ctx, T = _stepper(sem, vel=sem.opts(tol=1e-8), pres=sem.opts(tol=1e-8))
+        T.set_policy([{"storage": storage}])
+        T.step(3)  # (the storage is the policy's from the first step on)
+        T.step(before)
+        x, y, z = gpu_coords(ctx)
+        u, v, w, p = (t + 0 * x for t in inputs.tgv_initial(x, y, z, lib=torch))
+        for level in (2, 1, 0):
+            s = 0.9 + 0.02 * level
+            T.set(s * u, s * v, w.contiguous(), p.contiguous() if level == 0 else None, level=level, step=3)
+        T.step(3)
+        out.append(_state(T, ctx))
+        T.close()
+    assert _same(*out)
