@@ -388,7 +388,7 @@ typedef struct {
  * PCG; with op = SEM_F32 the default pressure solve is an FP32 inner PCG inside
  * FP64 refinement).  The solves' inner field selects their precision.
  * The stepper keeps a reference to ctx (which must outlive it) and solves on
- * the context's workspace slots 4-7; it allocates about 34 FP64 E-vectors plus
+ * the context's workspace slots 4-7; it allocates about 31 FP64 E-vectors plus
  * J^-1 and float-pair tables on the device (SEM_ERR_NOMEM if they do not fit).
  * SEM_ERR_ARG: NULL ctx or out, nu or dt not positive, an unsupported op, a
  * context that is not periodic in all three directions, or N > 9.  The state

@@ -1297,18 +1297,18 @@ extern "C" int sem_tgv_init(sem_ctx *c, double nu, double dt, sem_dtype op, cons
             return e_ == cudaErrorMemoryAllocation ? SEM_ERR_NOMEM : SEM_ERR_CUDA;           \
         }                                                                                    \
     } while (0)
-    // fields: u 9, C 9, p 1, unew 3, F 3, g 3, bp 1, rhs 3 = 32 E-vectors
-    TGV_TRY(cudaMalloc(&T->block, sizeof(double) * 32 * nL));
-    TGV_TRY(cudaMemset(T->block, 0, sizeof(double) * 32 * nL));
+    // fields: u 9, C 9, p 1, F 3, g 3, bp 1, rhs 3 = 29 E-vectors; unew lies in g,
+    // which nothing reads once the pressure's right-hand side is made
+    TGV_TRY(cudaMalloc(&T->block, sizeof(double) * 29 * nL));
+    TGV_TRY(cudaMemset(T->block, 0, sizeof(double) * 29 * nL));
     double *b = T->block;
     for (int l = 0; l < 3; ++l)
         for (int k = 0; k < 3; ++k) { T->u[l][k] = b; b += nL; }
     for (int l = 0; l < 3; ++l)
         for (int k = 0; k < 3; ++k) { T->C[l][k] = b; b += nL; }
     T->p = b; b += nL;
-    for (int k = 0; k < 3; ++k) { T->unew[k] = b; b += nL; }
     for (int k = 0; k < 3; ++k) { T->F[k] = b; b += nL; }
-    for (int k = 0; k < 3; ++k) { T->g[k] = b; b += nL; }
+    for (int k = 0; k < 3; ++k) { T->unew[k] = T->g[k] = b; b += nL; }
     T->bp = b; b += nL;
     for (int k = 0; k < 3; ++k) { T->rhs[k] = b; b += nL; }
     TGV_TRY(cudaMalloc(&T->part, sizeof(double) * 3 * c->E));

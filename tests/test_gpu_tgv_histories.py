@@ -110,3 +110,19 @@ def test_levels_set_between_steps(sem, storage, direct):
         out.append(_state(T, ctx))
         T.close()
     assert _same(*out)
+
+
+def test_a_stepper_takes_no_more_memory_than_its_fields(sem):
+    """32 FP64 E-vectors of fields and workspace are enough for a step (29 of the
+    stepper and two of the mass); with J^-1 (9 + 4.5 on the context, 9 as pairs) and
+    four solver workspaces (7.5 each).  An E-vector here is 16 MiB."""
+    torch, dev = torch_dev()
+    ctx, _, _ = pair(sem, 7, (16, 16, 16), 0.0, with_oracle=False)
+    vec = 8 * ctx.nL
+    assert vec == 16 << 20
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    T = sem.TGV(ctx, 0.02, 1e-3)
+    used = before - torch.cuda.mem_get_info()[0]
+    T.close()
+    assert used <= (32 + 22.5 + 30) * vec + (8 << 20), used / vec
