@@ -779,13 +779,14 @@ extern "C" int sem_hsmg_create(sem_ctx *c, int nlev, const int *orders, double h
     for (int l = 0; l < nlev; ++l) {
         HsLevel &L = H->L[l];
         const int64_t n = L.c->nL;
-        HS_CU(cudaMalloc(&L.r, ts * n));
-        HS_CU(cudaMalloc(&L.z, ts * n));
-        HS_CU(cudaMalloc(&L.w, ts * n));
-        HS_CU(cudaMalloc(&L.imult, ts * n));
-        rc = hs_imult(L.c, L.imult, dt, tmp, 0);
-        if (rc) { cudaFree(tmp); sem_hsmg_destroy(H); return rc; }
+        // (the finest level's residual is the caller's; the coarsest level is a solve)
+        if (l > 0) HS_CU(cudaMalloc(&L.r, ts * n));
         if (l < nlev - 1) {
+            HS_CU(cudaMalloc(&L.z, ts * n));
+            HS_CU(cudaMalloc(&L.w, ts * n));
+            HS_CU(cudaMalloc(&L.imult, ts * n));
+            rc = hs_imult(L.c, L.imult, dt, tmp, 0);
+            if (rc) { cudaFree(tmp); sem_hsmg_destroy(H); return rc; }
             rc = hs_factors(H, L, vert);
             if (rc) { cudaFree(tmp); sem_hsmg_destroy(H); return rc; }
             // interpolation from level l+1's GLL points to level l's

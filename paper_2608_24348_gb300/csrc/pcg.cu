@@ -200,7 +200,6 @@ static void fill_common(SolveParams<MAXP> &p, sem_ctx *owner, const sem_solve_op
 {
     p.nprob = nprob;
     p.mixed = o.inner != SEM_F64 && o.inner != SEM_F64_NATIVE;
-    p.inner_tc = o.inner == SEM_F32_TUNED ? 0 : inner_tc_of(o.inner, 2);
     p.abs_tol = o.abs_tol;
     p.maxit = o.maxit;
     p.max_outer = o.max_outer;

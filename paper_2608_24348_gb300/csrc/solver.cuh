@@ -123,7 +123,7 @@ struct SyncState {
 
 template <int MAXP>
 struct SolveParams {
-    int nprob, mixed, inner_tc, abs_tol, maxit, max_outer;
+    int nprob, mixed, abs_tol, maxit, max_outer;
     double tol, inner_tol;
     long long timeout_ns;
     SyncState *sync;
