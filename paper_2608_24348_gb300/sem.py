@@ -171,8 +171,12 @@ def stream_ptr(stream=None):
         return stream.cuda_stream
     import torch
     # the handle alone: a small sem_ax is bound by this host path, and making a
-    # torch.cuda.Stream object for it took 2.5 of its 8.1 us
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    # torch.cuda.Stream object for it took 2.5 of its 8.1 us (a torch without the
+    # internal function: the public way)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 def opts(tol=1e-10, abs_tol=False, maxit=20000, inner="f64", inner_tol=1e-4, max_outer=50,
