@@ -300,7 +300,10 @@ __global__ void __launch_bounds__(256) k_dssum_rows(DssumArgs a, UqMesh M)
     uq_scatter(u, U, s);
 }
 
-// The same one node at a time, for vectors not aligned for vector accesses.
+// The same one node at a time: for vectors not aligned for a chunk's accesses, and for
+// larger meshes of N = 1, where a row is one chunk of two nodes and every node is
+// shared (64^3 elements: 17.2 us FP64 and 14.4 FP32 against 20.2 and 21.3 by chunks;
+// 16^3: 4.5 and 3.7 against 4.3 and 3.7; 4^3: 3.6 and 2.8 against 2.5 and 1.6).
 template <typename T>
 __global__ void k_dssum(T *__restrict__ u, GsDesc d)
 {
@@ -318,9 +321,9 @@ template <typename T>
 static int dssum_launch(sem_ctx *c, int n, void *const *u, cudaStream_t s)
 {
     const GsDesc d = sem_gs_desc(c);
-    bool aligned = true;
-    for (int k = 0; k < n; ++k) aligned &= (uintptr_t)u[k] % 32 == 0;
-    if (!aligned) {
+    bool rows = c->n > 2 || c->nG <= 16384;
+    for (int k = 0; k < n; ++k) rows &= (uintptr_t)u[k] % 32 == 0;
+    if (!rows) {
         for (int k = 0; k < n; ++k)
             k_dssum<T><<<(unsigned)sem_ceil_div(c->nG, 256), 256, 0, s>>>((T *)u[k], d);
         SEM_CHECK_LAUNCH();
