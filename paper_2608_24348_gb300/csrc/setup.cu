@@ -299,7 +299,7 @@ extern "C" void sem_destroy(sem_ctx *c)
     if (!c) return;
     cudaDeviceSynchronize();
     sem_pipe_destroy(c->pipe);
-    void *ps[] = {c->tab64, c->tab32, c->geo64, c->geo32, c->geodf, c->tabdf, c->tabdfeo, c->vert, c->jinv64, c->jinv32, c->err_dev,
+    void *ps[] = {c->tab64, c->geo64, c->geo32, c->geodf, c->tabdf, c->tabdfeo, c->vert, c->jinv64, c->jinv32, c->err_dev,
                   c->solve_dev, c->partials, c->stage[0], c->stage[1]};
     for (void *p : ps)
         if (p) cudaFree(p);
@@ -353,16 +353,20 @@ extern "C" int sem_setup(int N, int nelx, int nely, int nelz, const double exten
     gll_table(N, c->hxi, c->hw);
     deriv_table(N, c->hxi, c->hD);
     const int n = c->n;
-    double h64[2 * SEM_NPMAX + SEM_NPMAX * SEM_NPMAX];
+    const int ntab = 2 * n + n * n;
+    double h64[2 * (2 * SEM_NPMAX + SEM_NPMAX * SEM_NPMAX)];
     float h32[2 * SEM_NPMAX + SEM_NPMAX * SEM_NPMAX];
-    int ntab = 2 * n + n * n;
     for (int i = 0; i < n; ++i) { h64[i] = c->hxi[i]; h64[n + i] = c->hw[i]; }
     for (int i = 0; i < n * n; ++i) h64[2 * n + i] = c->hD[i];
     for (int i = 0; i < ntab; ++i) h32[i] = (float)h64[i];
-    SETUP_TRY(cudaMalloc(&c->tab64, sizeof(double) * ntab));
-    SETUP_TRY(cudaMalloc(&c->tab32, sizeof(float) * ntab));
-    SETUP_TRY(cudaMemcpy(c->tab64, h64, sizeof(double) * ntab, cudaMemcpyHostToDevice));
-    SETUP_TRY(cudaMemcpy(c->tab32, h32, sizeof(float) * ntab, cudaMemcpyHostToDevice));
+    // one allocation and one copy: the FP32 table right behind the FP64 one
+    memcpy(h64 + ntab, h32, sizeof(float) * ntab);
+    SETUP_TRY(cudaMalloc(&c->tab64, (sizeof(double) + sizeof(float)) * ntab));
+    c->tab32 = (float *)(c->tab64 + ntab);
+    SETUP_TRY(cudaMemcpy(c->tab64, h64, (sizeof(double) + sizeof(float)) * ntab, cudaMemcpyHostToDevice));
+    // (before the first kernel: the copy into constant memory waits for what is queued)
+    rc = sem_solve_upload_tables(c);
+    if (rc != SEM_OK) { sem_destroy(c); return rc; }
     size_t nv = (size_t)(nelx + 1) * (nely + 1) * (nelz + 1) * 3;
     SETUP_TRY(cudaMalloc(&c->vert, sizeof(double) * nv));
     if (vertices) {
@@ -382,8 +386,6 @@ extern "C" int sem_setup(int N, int nelx, int nely, int nelz, const double exten
     rc = sem_run_geometry(c, nullptr, false, s);
     if (rc != SEM_OK) { sem_destroy(c); return rc; }
     rc = sem_make_geo_df(c);
-    if (rc != SEM_OK) { sem_destroy(c); return rc; }
-    rc = sem_solve_upload_tables(c);
     if (rc != SEM_OK) { sem_destroy(c); return rc; }
     // volume = sum of B
     {
