@@ -197,7 +197,8 @@ SEM_API int sem_jacobi(sem_ctx *ctx, double h1, double h2, double *minv, void *s
  * ||r|| = sqrt(sum_local r^2 / mult); relative to ||b|| unless abs_tol != 0.
  * inner: the operator precision; SEM_F64 runs plain FP64 PCG, the other three
  * run FP64 iterative refinement around an inner PCG in that precision
- * (vectors FP32, dot products FP64) with relative tolerance inner_tol.
+ * (vectors FP32; dot products in FP64 or, over FP32 vectors, of exact products
+ * whose sums keep at least FP64's bits) with relative tolerance inner_tol.
  * SEM_F64 with a relative tol below 1e-11 runs on the native FP64 operator
  * (SEM_F64_NATIVE): the FP64-accurate operators on the FP32 pipes carry a
  * relative error of a few 1e-13 per application, the size of such a residual,

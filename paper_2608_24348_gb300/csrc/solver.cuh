@@ -65,6 +65,7 @@
 #include "ax_line32.cuh"
 #include "ax_tc.cuh"
 #include "common.cuh"
+#include "sum3.cuh"
 #include "tma.cuh"
 #include "uniq.cuh"
 
@@ -157,8 +158,8 @@ __device__ __forceinline__ void red_release_add_u32(unsigned *p, unsigned v)
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Phases whose sums are gathered in float pairs.
-__device__ __forceinline__ bool phase_pairs(int ph)
+// Phases whose sums are gathered in floats (Sum3).
+__device__ __forceinline__ bool phase_floats(int ph)
 {
     return ph == PH_A32 || ph == PH_C32 || ph == PH_INIT32;
 }
@@ -201,27 +202,11 @@ __device__ __forceinline__ void dot2_acc(dfacc &A, float a, float b)
     A.e = __fadd_rn(A.e, __fadd_rn(t, ep));
 }
 
-__device__ __forceinline__ double dfacc_value(dfacc A) { return (double)A.s + (double)A.e; }
-
 __device__ __forceinline__ double warp_sum(double v)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
-}
-
-// The sum of a warp's float pairs (two-sums, the errors gathered as in dot2_acc).
-__device__ __forceinline__ dfacc warp_sum_pair(dfacc A)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float b = __shfl_xor_sync(0xffffffffu, A.s, o), be = __shfl_xor_sync(0xffffffffu, A.e, o);
-        const float s = __fadd_rn(A.s, b), bv = __fsub_rn(s, A.s);
-        const float t = __fadd_rn(__fsub_rn(A.s, __fsub_rn(s, bv)), __fsub_rn(b, bv));
-        A.s = s;
-        A.e = __fadd_rn(__fadd_rn(A.e, be), t);
-    }
-    return A;
 }
 
 // The sum of a thread's values by halves: the additions of one level are
@@ -368,7 +353,7 @@ static __constant__ SolveTabs c_tabs[SEM_NPMAX + 1];
 // A32: p32 = z32 + beta p32, w32 <- A32 p32, <p32, w32>, by whole lines.
 template <int NP, int TH>
 __device__ __forceinline__ void phase_a32(const ProbDesc &P, double beta, int first, const Deal &deal,
-                                          unsigned char *smem, dfacc &dot)
+                                          unsigned char *smem, Sum3 &sum)
 {
     using G = GrpCfg<NP, TH>;
     constexpr int NP2 = NP * NP, NP3 = NP2 * NP;
@@ -400,6 +385,7 @@ __device__ __forceinline__ void phase_a32(const ProbDesc &P, double beta, int fi
         if (threadIdx.x % G::GT == 0) geo_prefetch<NP>(P.geo32, (int64_t)g * G::GE, G::GE, E, 4);
         const size_t off = (size_t)(active ? e : 0) * NP3 + th.tid;
         cp_async_wait_all();
+        dfacc dot = {0.f, 0.f};
         auto load = [&](int k) {
             float pn = sz[k * TH];
             if (!first) pn = fmaf(b32, sp[k * TH], pn);
@@ -412,6 +398,7 @@ __device__ __forceinline__ void phase_a32(const ProbDesc &P, double beta, int fi
         };
         ax_line32_element<NP>(load, store, P.geo32 + (size_t)(active ? e : 0) * 7 * NP3, h1, h2,
                               c_tabs[NP].l, slab, th.tid, active, [&] { fetch(g + stride); }, sync);
+        sum3_add(sum, dot.s, dot.e, 0.f);
     }
 }
 
@@ -625,9 +612,10 @@ __device__ __forceinline__ void elem_item_native(const ProbDesc &P, bool ax0, do
 // BF16, 2 FP16 (plain rounding); 3 FP16 x2, 4 BF16 x3 (split operands, N+1 <= 8).
 template <int NP>
 __device__ __forceinline__ void elem_item_tc(const ProbDesc &P, double beta, int first, int64_t g, int tc,
-                                             unsigned char *smem, dfacc &dot)
+                                             unsigned char *smem, Sum3 &sum)
 {
     const float b32 = (float)beta;
+    dfacc dot = {0.f, 0.f};
     auto load = [&](int64_t q) {
         float pn = __ldcg(P.w32 + q);
         if (!first) pn = fmaf(b32, __ldcg(P.p32 + q), pn);
@@ -644,6 +632,7 @@ __device__ __forceinline__ void elem_item_tc(const ProbDesc &P, double beta, int
         ax_tc_split_group<NP, false>(load, store, P.geo32, P.D32, (float)P.h1, (float)P.h2, P.E, g, smem);
     else
         ax_tc_group<NP>(load, store, P.geo32, P.D32, (float)P.h1, (float)P.h2, P.E, g, tc == 2, smem);
+    sum3_add(sum, dot.s, dot.e, 0.f);
 }
 
 // Whether the element phases of order NP in MODE are line phases (A32 always is).
@@ -656,7 +645,7 @@ constexpr bool line_mode()
 // This CTA's share of an element phase; returns the next problem's rot.
 template <int NP, int MODE, int TH>
 __device__ __forceinline__ unsigned phase_elem_np(const ProbDesc &P, int ph, double beta, int first,
-                                                  const Deal &deal, unsigned char *smem, double &acc, dfacc &dot)
+                                                  const Deal &deal, unsigned char *smem, double &acc, Sum3 &dot)
 {
     const bool ax0 = ph == PH_AX0;
     if constexpr (MODE == MODE_F64 && (solve_bfp<NP>() || solve_dfl<NP>())) {
@@ -694,14 +683,15 @@ __device__ __forceinline__ unsigned phase_elem_np(const ProbDesc &P, int ph, dou
 // of few iterations saves that last pass.
 constexpr int X_DIRECT = 4;
 
-// Chunk t of a unique phase.  v: FP64 sums; d: the sums of the FP32 phases, in
-// float pairs (converting them once a chunk cost more FP64 operations than an
-// FP64 phase has).
+// Chunk t of a unique phase.  v: FP64 sums; sum: the sums of the FP32 phases
+// (converting them to FP64 once a chunk cost more FP64 operations than an FP64
+// phase has).
 template <int NP, int MODE>
 __device__ __forceinline__ void uniq_item(const ProbDesc &P, const PState &S, int ph, unsigned t, double v[3],
-                                          dfacc d[2])
+                                          Sum3 sum[2])
 {
     constexpr int CH = UqCfg<NP>::CH;
+    dfacc d[2] = {{0.f, 0.f}, {0.f, 0.f}};  // the chunk's own
     constexpr bool MIXED = MODE == MODE_F32 || MODE == MODE_TC;
     const UqChunk U = uq_chunk<NP>(P.mesh, t);
     if constexpr (!MIXED) {
@@ -774,6 +764,8 @@ __device__ __forceinline__ void uniq_item(const ProbDesc &P, const PState &S, in
             uq_stv(P.r32 + U.f, r0, CH);
             uq_stv(P.d32 + U.f, dv, CH);
             uq_scatter(P.w32, U, s);
+            sum3_add(sum[0], d[0].s, d[0].e, 0.f);
+            sum3_add(sum[1], d[1].s, d[1].e, 0.f);
             return;
         }
         if (ph == PH_R64) {
@@ -809,6 +801,8 @@ __device__ __forceinline__ void uniq_item(const ProbDesc &P, const PState &S, in
             uq_stv(P.r32 + U.f, rv, CH);
             uq_stv(P.d32 + U.f, zero, CH);
             uq_scatter(P.w32, U, z);
+            sum3_add(sum[0], d[0].s, d[0].e, 0.f);
+            sum3_add(sum[1], d[1].s, d[1].e, 0.f);
             return;
         }
         if (ph == PH_UPD) {
@@ -1051,11 +1045,11 @@ struct SmemMax<MODE, TH, NP0, NPs...> {
 };
 
 // Static shared memory of the kernel (states, sums, reduction words).
-template <int MAXP, int TH, bool PAIRS>
+template <int MAXP, int TH, bool FLOATS>
 constexpr size_t solve_static_smem()
 {
     return MAXP * (sizeof(PState) + 3 * sizeof(double)) + 64 + TH / 8 +
-           (PAIRS && MAXP * (TH / 32) > TH ? MAXP * 3 * (TH / 32) : 3 * TH) * sizeof(double);
+           (FLOATS && MAXP * (TH / 32) > TH ? MAXP * 3 * (TH / 32) : 3 * TH) * sizeof(double);
 }
 
 // Threads of a CTA: one CTA that fills its multiprocessor for the line phases
@@ -1079,7 +1073,7 @@ template <int MODE, int TH, int NP0, int... NPs>
 struct PhaseDispatch<MODE, TH, NP0, NPs...> {
     // This CTA's share of P's phase; returns the next problem's rot.
     __device__ __forceinline__ static unsigned run(const ProbDesc &P, const PState &S, int kind, const Deal &deal,
-                                                   unsigned char *smem, double v[3], dfacc d[2])
+                                                   unsigned char *smem, double v[3], Sum3 d[2])
     {
         if constexpr (sizeof...(NPs) > 0)
             if (P.n != NP0) return PhaseDispatch<MODE, TH, NPs...>::run(P, S, kind, deal, smem, v, d);
@@ -1112,11 +1106,11 @@ __global__ void __launch_bounds__(TH, TH > SEM_SOLVE_THREADS ? 1 : 2)
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ PState s_st[MAXP];
     __shared__ double s_sum[MAXP][3];
-    // Sums of a problem's phase over the CTA: [value][thread], or, in an FP32
-    // launch of several problems, [problem][value][warp].
-    constexpr bool PAIRS = MODE == MODE_F32 || MODE == MODE_TC;
+    // Sums of a problem's phase over the CTA: [value][thread], or, in an FP32 launch
+    // (of several problems, or of more than 256 threads), [problem][value][warp].
+    constexpr bool FLOATS = MODE == MODE_F32 || MODE == MODE_TC;
     constexpr int NW = TH / 32;
-    constexpr int RED = PAIRS && MAXP * NW > TH ? MAXP * 3 * NW : 3 * TH;
+    constexpr int RED = FLOATS && MAXP * NW > TH ? MAXP * 3 * NW : 3 * TH;
     __shared__ double s_red[RED];
     __shared__ int s_fail;
     // Kept in shared memory so that no register holds them through an element
@@ -1159,7 +1153,7 @@ __global__ void __launch_bounds__(TH, TH > SEM_SOLVE_THREADS ? 1 : 2)
                 layout = want;
             }
             double v[3] = {0.0, 0.0, 0.0};
-            dfacc d[2] = {{0.f, 0.f}, {0.f, 0.f}};
+            Sum3 d[2] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
             if (kind != KIND_LOCAL) {
                 if (MAXP > 1) __syncwarp();
                 const Deal deal = {blockIdx.x, grid, MAXP == 1 ? 0u : s_rot[warp]};
@@ -1174,16 +1168,20 @@ __global__ void __launch_bounds__(TH, TH > SEM_SOLVE_THREADS ? 1 : 2)
             }
             const int nv = phase_nvals(s_st[p].phase);
             if (nv == 0) continue;
-            if (PAIRS && MAXP > 1 && np > 1) {
+            if (FLOATS && (np > 1 || TH > SEM_SOLVE_THREADS)) {
                 // no barrier between the problems of an FP32 launch: a warp sums
-                // its lanes' pairs and leaves the values for the end of the step
-                const bool pairs = phase_pairs(s_st[p].phase);
+                // its lanes' values and leaves the sums for the end of the step
+                if (phase_floats(s_st[p].phase)) {
+                    const double t = warp_sum3(d, lane);
+                    if (lane % 16 == 0 && (int)lane / 16 < nv) s_red[(p * 3 + lane / 16) * NW + warp] = t;
+                } else {
 #pragma unroll
-                for (int k = 0; k < 2; ++k)
-                    if (k < nv) {
-                        const double t = pairs ? dfacc_value(warp_sum_pair(d[k])) : warp_sum(v[k]);
-                        if (lane == 0) s_red[(p * 3 + k) * NW + warp] = t;
-                    }
+                    for (int k = 0; k < 2; ++k)
+                        if (k < nv) {
+                            const double t = warp_sum(v[k]);
+                            if (lane == 0) s_red[(p * 3 + k) * NW + warp] = t;
+                        }
+                }
                 continue;
             }
             // one warp per value sums the CTA's TH in a fixed order
@@ -1191,7 +1189,7 @@ __global__ void __launch_bounds__(TH, TH > SEM_SOLVE_THREADS ? 1 : 2)
             for (int k = 0; k < 3; ++k)
                 if (k < nv)
                     s_red[k * TH + threadIdx.x] =
-                        PAIRS && k < 2 && phase_pairs(s_st[p].phase) ? dfacc_value(d[k]) : v[k];
+                        FLOATS && k < 2 && phase_floats(s_st[p].phase) ? sum3_value(d[k]) : v[k];
             __syncthreads();
             if ((int)warp < nv) {
                 double t[NW];
@@ -1204,7 +1202,7 @@ __global__ void __launch_bounds__(TH, TH > SEM_SOLVE_THREADS ? 1 : 2)
         }
         if (all_done) break;
 
-        if (PAIRS && MAXP > 1 && np > 1) {
+        if (FLOATS && (np > 1 || TH > SEM_SOLVE_THREADS)) {
             __syncthreads();
             for (int pk = warp; pk < np * 3; pk += NW) {
                 const int p = pk / 3, k = pk - 3 * p;
