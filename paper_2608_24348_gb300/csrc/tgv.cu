@@ -635,14 +635,25 @@ __global__ void __launch_bounds__(VelCfg<NP>::TH) k_tgv_vel(VArgs a, const __gri
 // element's largest sum_a |U_a| / dxi_a over its nodes (part[2][e]; U_a = sum_c
 // (dr_a/dx_c) u_c, dxi_a the GLL gap at the node's index along a; the CFL number
 // per unit step, Sec. 3).  Gradients, vorticity and both integrands in float
-// pairs (jinv, geo, D as pairs), the sums over an element in FP64.
+// pairs (jinv, geo, D as pairs), the sums over an element and the CFL number in FP64.
 //
 // Bound: FP32 issue and HBM (13 words a node).  The nine derivatives run by whole
 // folded lines (ax_dfl.cuh), and only the six products that the vorticity needs
 // are formed; a node at a time, with all nine: 1.73 ms at 32^3, N = 7, now 1.07.
 struct GapInv {
-    dfp v[SEM_NPMAX];
+    double v[SEM_NPMAX];
 };
+
+// FP32 -> FP64 on the integer pipe (a conversion takes the FP64 pipe, as the three
+// additions and products a node do): exact for zero, normal numbers, infinities and
+// NaN; subnormals give zero.
+__device__ __forceinline__ double widen(float f)
+{
+    const unsigned u = __float_as_uint(f), e = u >> 23 & 0xffu;
+    const unsigned hi = (u & 0x80000000u) | (e == 0xffu ? 0x7ff00000u : e == 0u ? 0u : (e + 896u) << 20) |
+                        (e == 0u ? 0u : (u & 0x7fffffu) >> 3);
+    return __hiloint2double((int)hi, e == 0u ? 0 : (int)(u << 29));
+}
 
 template <int NP>
 struct DiagCfg {
@@ -697,16 +708,15 @@ __global__ void __launch_bounds__(DiagCfg<NP>::TH)
             const dfp bm = geo[(e * 7 + 6) * N3 + pn];
             const dfp uu[3] = {su[o], su[SL + o], su[2 * SL + o]};
             const int ia[3] = {i, j, k};
-            dfacc cn = {0.f, 0.f};
+            double cn = 0.0;  // (FP64: the CFL-controlled step size is made from it)
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 dfacc U = df_mul(J[a * 3], uu[0]);
                 df_mad(U, J[a * 3 + 1], uu[1]);
                 df_mad(U, J[a * 3 + 2], uu[2]);
-                const float s = __fadd_rn(U.s, U.e), r = __fsub_rn(U.e, __fsub_rn(s, U.s));
-                df_mad(cn, ig.v[ia[a]], s < 0.f ? dfp{-s, -r} : dfp{s, r});
+                cn = fma(fabs(widen(U.s) + widen(U.e)), ig.v[ia[a]], cn);
             }
-            cmax = fmax(cmax, df_widen(cn.s) + df_widen(cn.e));
+            cmax = fmax(cmax, cn);
             // component du_c/dx_d - du_d/dx_c
             auto curl = [&](int c, int d) {
                 dfacc w = {0.f, 0.f};
@@ -1059,9 +1069,7 @@ static GapInv gap_inv(const sem_ctx *c)
     for (int i = 0; i <= N; ++i) {
         const double l = i > 0 ? c->hxi[i] - c->hxi[i - 1] : 1e300;
         const double r = i < N ? c->hxi[i + 1] - c->hxi[i] : 1e300;
-        const double v = 1.0 / (l < r ? l : r);
-        const float h = (float)v;
-        g.v[i] = {h, (float)(v - (double)h)};
+        g.v[i] = 1.0 / (l < r ? l : r);
     }
     return g;
 }
