@@ -34,6 +34,7 @@
 #include "common.cuh"
 #include "df64.cuh"
 #include "gs.cuh"
+#include "quot.cuh"
 #include "tma.cuh"
 #include "uniq.cuh"
 
@@ -436,20 +437,10 @@ __device__ __forceinline__ void ld_fsv(const void *p, size_t q, int s32, double 
 }
 
 // k[0] x + k[1] y + k[2] z over the levels of a history; the order is written out
-// because the step's results follow its last bit (see div_r).
+// because the step's results follow its last bit (see quot.cuh).
 __device__ __forceinline__ double sum3(const double (&k)[3], double x, double y, double z)
 {
     return fma(k[2], z, fma(k[0], x, k[1] * y));
-}
-
-// a / b from r = 1 / b rounded: one residual step restores the quotient's last
-// bit (Markstein, IBM J. Res. Dev. 34, 1990), in three operations.  The steps
-// must not differ from a divided form by even that bit: the loosely stopped
-// solves downstream amplify a last-bit change of the velocity by 1e6 and more.
-__device__ __forceinline__ double div_r(double a, double b, double r)
-{
-    const double q = a * r;
-    return fma(fma(-q, b, a), r, q);
 }
 
 struct FArgs {
