@@ -134,21 +134,50 @@ static int launch_tma(const sem_ctx *c, const float *u, float *w, float h1, floa
     }
 }
 
-// The line operator (ax_line32.cuh): 256 threads, the next element group's u
-// copied into shared memory by asynchronous copies (every thread its own
-// column), groups synchronised by themselves.  Bound: FP32 issue and HBM alike
-// (36 bytes a node); 0.1055 ms at 32^3 elements, N = 7 (0.1209 by the staged form
-// below, 0.089 the bytes alone).
+// The line operator (ax_line32.cuh): the next element group's u copied into shared
+// memory by asynchronous copies (every thread its own column), groups synchronised
+// by themselves.  Bound: FP32 issue and HBM alike (36 bytes a node); 0.1055 ms at
+// 32^3 elements, N = 7 (0.1209 by the staged form above, 0.089 the bytes alone).
+//
+// Blocks of 256 threads, or of the whole warps of one element for N >= 11, whose
+// columns fill 256 threads badly.  Registers decide between the latency of one
+// element (a whole line and its result want NP^2 / 2 or so) and the elements in
+// flight: blocks an SM by order, measured at one to four (us; in brackets direct
+// loads or, N = 7 and 9, the staged form, which the smallest meshes took before):
+//  - N = 8: three, 77.6 at 13824 elements (two 93.7, four 83.3), 5.2 at 252 (four 6.4) [145, 5.5]
+//  - N = 9: three, 113 at 13824 (two 132, four 136) [145]
+//  - N = 10: two, 90.2 at 8000 (one 143, three 97.5), 5.2 at 125 [189, 5.7]
+//  - N = 11: three blocks of 160, 132 at 8000 (256 threads, one block: 305) [198]
+//  - N = 12: two blocks of 192, 109 at 3840 (256 threads, one block: 176) [148]
+//  - N = 13: two blocks of 224 above six elements an SM, 90.8 at 1872 (one 105); one
+//    below, 31.6 at 648 (two 34.2) [144, 29.3]
+//  - others: four, or one (N >= 14: 128 registers spill).
+// A mesh that one block an SM holds (two at N = 9) takes two blocks' registers at
+// N = 2, 6, 7 and 9, since only its latency counts: N = 2, 36 elements 2.5 (four 2.7)
+// [2.6]; N = 6, 648 elements 4.4 (four 4.9) [4.4]; N = 7, 36 elements 3.6 (3.8) [3.6];
+// N = 9, 252 elements 5.3 (three 6.0, four 7.3) [5.4].  Direct loads stay ahead at N = 2
+// above 4000 elements (15.0 against 16.5 at 65536) and N = 13 below 900 (29.3 against
+// 31.6 at 648).  The staged form's and the direct loads' error is three times that of
+// whole lines (1.2e-7 against 4.2e-8 of the result at N = 7).
 template <int NP>
 struct L32Shape {
     static constexpr int NP2 = NP * NP;
-    static constexpr int GT = NP <= 4 ? 32 : NP == 8 ? 64 : (NP == 5 || NP == 6 || NP == 10 || NP == 11) ? 128 : 256;
-    static constexpr int GE = GT / NP2, NG = 256 / GT, NE = NG * GE;
-    static constexpr size_t SMEM = sizeof(float) * ((size_t)NE * 3 * Line32Cfg<NP>::SLAB + NP * 256);
+    static constexpr int GT = NP <= 4    ? 32
+                              : NP == 8  ? 64
+                              : NP >= 12 ? (NP2 + 31) / 32 * 32
+                              : (NP == 5 || NP == 6 || NP == 10 || NP == 11) ? 128 : 256;
+    static constexpr int TB = NP >= 12 ? GT : 256;
+    static constexpr int GE = GT / NP2, NG = TB / GT, NE = NG * GE;
+    static constexpr size_t SMEM = sizeof(float) * ((size_t)NE * 3 * Line32Cfg<NP>::SLAB + NP * TB);
+    // blocks an SM (registers), for large meshes and for small ones
+    static constexpr int MINB = NP == 9 || NP == 10 || NP == 12 ? 3 : NP == 11 || NP == 13 || NP == 14 ? 2 : NP >= 15 ? 1 : 4;
+    static constexpr int MINB_SMALL = NP == 3 || NP == 7 || NP == 8 || NP == 10 ? 2 : NP == 14 ? 1 : MINB;
+    // the largest small mesh, in elements an SM: a block's worth, N = 9 two blocks', N = 13 six
+    static constexpr int SMALL = NP == 14 ? 6 : NP == 10 ? 4 : NE;
 };
 
-template <int NP>
-__global__ void __launch_bounds__(256, NP <= 10 ? 4 : 1)
+template <int NP, int MINB>
+__global__ void __launch_bounds__(L32Shape<NP>::TB, MINB)
     k_ax_line32(const float *__restrict__ u, float *__restrict__ w, const float *__restrict__ geo,
                 const __grid_constant__ LineTab32 T, float h1, float h2, int64_t E)
 {
@@ -160,7 +189,7 @@ __global__ void __launch_bounds__(256, NP <= 10 ? 4 : 1)
     float *slab = reinterpret_cast<float *>(smem) + (size_t)(grp * S::GE + ge) * 3 * Line32Cfg<NP>::SLAB;
     float *su = reinterpret_cast<float *>(smem) + (size_t)S::NE * 3 * Line32Cfg<NP>::SLAB + threadIdx.x;
     auto sync = [&] {
-        if constexpr (S::GT == 256)
+        if constexpr (S::GT == S::TB)
             __syncthreads();
         else if constexpr (S::GT == 32)
             __syncwarp();
@@ -172,7 +201,7 @@ __global__ void __launch_bounds__(256, NP <= 10 ? 4 : 1)
         const int64_t e = g * S::GE + ge;
         if (g < groups && tid >= 0 && e < E) {
 #pragma unroll
-            for (int k = 0; k < NP; ++k) cp_async4(su + k * 256, u + e * NP3 + k * NP2 + tid);
+            for (int k = 0; k < NP; ++k) cp_async4(su + k * S::TB, u + e * NP3 + k * NP2 + tid);
         }
     };
     int64_t g = (int64_t)grp * gridDim.x + blockIdx.x;
@@ -184,21 +213,21 @@ __global__ void __launch_bounds__(256, NP <= 10 ? 4 : 1)
             l2_prefetch_span(geo, e0 * 7 * NP3 * 4, (e0 + S::GE < E ? e0 + S::GE : E) * 7 * NP3 * 4);
         float *we = w + (active ? e : 0) * NP3 + tid;
         cp_async_wait_all();
-        auto load = [&](int k) { return su[k * 256]; };
+        auto load = [&](int k) { return su[k * S::TB]; };
         auto store = [&](int k, float v, float) { we[k * NP2] = v; };
         ax_line32_element<NP>(load, store, geo + (active ? e : 0) * 7 * NP3, h1, h2, T, slab, tid, active,
                               [&] { fetch(g + stride); }, sync);
     }
 }
 
-template <int NP>
-static int launch_line32(const sem_ctx *c, const float *u, float *w, float h1, float h2, cudaStream_t s)
+template <int NP, int MINB>
+static int launch_line32_regs(const sem_ctx *c, const float *u, float *w, float h1, float h2, cudaStream_t s)
 {
     using S = L32Shape<NP>;
     static std::atomic<unsigned> attr{0};
-    SEM_CUDA(sem_smem_attr(k_ax_line32<NP>, S::SMEM, attr));
+    SEM_CUDA(sem_smem_attr(k_ax_line32<NP, MINB>, S::SMEM, attr));
     int per_sm = 0;
-    SEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ax_line32<NP>, 256, S::SMEM));
+    SEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ax_line32<NP, MINB>, S::TB, S::SMEM));
     if (per_sm < 1) return SEM_ERR_ARG;
     const int64_t groups = sem_ceil_div(c->E, S::GE);
     int64_t grid = (int64_t)per_sm * c->num_sms;
@@ -206,9 +235,20 @@ static int launch_line32(const sem_ctx *c, const float *u, float *w, float h1, f
     LineTab32 T;
     memset(&T, 0, sizeof(T));
     for (int t = 0; t < NP * NP; ++t) T.d[t] = (float)c->hD[t];
-    k_ax_line32<NP><<<(unsigned)grid, 256, S::SMEM, s>>>(u, w, c->geo32, T, h1, h2, c->E);
+    k_ax_line32<NP, MINB><<<(unsigned)grid, S::TB, S::SMEM, s>>>(u, w, c->geo32, T, h1, h2, c->E);
     SEM_CHECK_LAUNCH();
     return SEM_OK;
+}
+
+template <int NP>
+static int launch_line32(const sem_ctx *c, const float *u, float *w, float h1, float h2, cudaStream_t s)
+{
+    using S = L32Shape<NP>;
+    if constexpr (S::MINB_SMALL != S::MINB)
+        // (of the whole mesh, so that a call on host buffers, in chunks, does the same)
+        if ((int64_t)c->nelx * c->nely * c->nelz <= (int64_t)S::SMALL * c->num_sms)
+            return launch_line32_regs<NP, S::MINB_SMALL>(c, u, w, h1, h2, s);
+    return launch_line32_regs<NP, S::MINB>(c, u, w, h1, h2, s);
 }
 
 // Variants of the FP32 operator (see sem_tune_ax): 0 whole lines, 1 staged
