@@ -321,17 +321,21 @@ template <typename T>
 static int dssum_launch(sem_ctx *c, int n, void *const *u, cudaStream_t s)
 {
     const GsDesc d = sem_gs_desc(c);
-    bool rows = c->n > 2 || c->nG <= 16384;
-    for (int k = 0; k < n; ++k) rows &= (uintptr_t)u[k] % 32 == 0;
-    if (!rows) {
-        for (int k = 0; k < n; ++k)
-            k_dssum<T><<<(unsigned)sem_ceil_div(c->nG, 256), 256, 0, s>>>((T *)u[k], d);
-        SEM_CHECK_LAUNCH();
-        return SEM_OK;
+    uintptr_t at = 0;
+    for (int k = 0; k < n; ++k) at |= (uintptr_t)u[k];
+    if (c->n > 2 || c->nG <= 16384) {
+        DssumArgs a = {{u[0], n > 1 ? u[1] : nullptr, n > 2 ? u[2] : nullptr}};
+        const UqMesh M = uq_mesh(d);
+        SEM_DISPATCH_NP(c->n, {
+            if (at % (sizeof(T) * uq_width<NP>()) == 0) {
+                k_dssum_rows<NP, T><<<dim3((uq_units<NP>(M) + 255) / 256, n), 256, 0, s>>>(a, M);
+                SEM_CHECK_LAUNCH();
+                return SEM_OK;
+            }
+        });
     }
-    DssumArgs a = {{u[0], n > 1 ? u[1] : nullptr, n > 2 ? u[2] : nullptr}};
-    const UqMesh M = uq_mesh(d);
-    SEM_DISPATCH_NP(c->n, k_dssum_rows<NP, T><<<dim3((uq_units<NP>(M) + 255) / 256, n), 256, 0, s>>>(a, M));
+    for (int k = 0; k < n; ++k)
+        k_dssum<T><<<(unsigned)sem_ceil_div(c->nG, 256), 256, 0, s>>>((T *)u[k], d);
     SEM_CHECK_LAUNCH();
     return SEM_OK;
 }

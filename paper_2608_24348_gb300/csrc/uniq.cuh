@@ -74,6 +74,16 @@ struct UqCfg {
     static constexpr int NC = NP / CH;  // chunks a row
 };
 
+// Values that an access to a chunk takes at once (uq_ldv, uq_stv): a vector has to
+// be aligned to as many.  An E-vector's offset into a larger array is a multiple of
+// its length, which for even N+1 is a multiple of this, but for odd N+1 may be odd.
+template <int NP>
+__host__ __device__ constexpr int uq_width()
+{
+    constexpr int CH = UqCfg<NP>::CH;
+    return CH == 4 || CH == 2 ? CH : 1;
+}
+
 // The copies of a chunk: offset f of its first node in the first row (the
 // owner's), distances dy, dz to the rows of the neighbours that share it, and
 // distance dl from f to the left neighbour's copy of that node (only the first
