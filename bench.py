@@ -373,7 +373,11 @@ def batched_section(sem, inputs, stream, peak_gbs):
     ms = e0.elapsed_time(e1)
     nodes = sum(c.nL for c in ctxs)
     work = sum(i["iters"] * c.nL for i, c in zip(infos, ctxs))
-    gbs = 84.0 * work / (ms * 1e-3) / 1e9
+    gbs = 72.0 * work / (ms * 1e-3) / 1e9  # an FP32 inner iteration moves 72 bytes a node
+    # the launch's shape: 768 threads, 256 where a problem takes the tensor cores; an
+    # order's elements go to groups of GT threads, as many as fit (8 a block by warps there)
+    threads = 256 if any(t["path"] for t in tuned.values()) else 768
+    group = {5: 128, 7: 64, 9: 128}
     out = {"workload": "64 uneven periodic Poisson problems, E in {8^3..24^3}, N in {5,7,9}, "
                        "FP32-accurate inner (per-order path chosen by the tuner) / FP64 refinement "
                        "to 1e-10, one persistent launch",
@@ -381,10 +385,11 @@ def batched_section(sem, inputs, stream, peak_gbs):
            "status_all_ok": all(i["status"] == 0 for i in infos),
            "gdofs_iter": work / (ms * 1e-3) / 1e9, "hbm_gbs": gbs, "hbm_frac": gbs / peak_gbs,
            "tile": {str(N): {"inner_path": "fp16x2_tensor_cores" if t["path"] else "fp32_cuda_cores",
-                             "elements_per_block": 8 if t["path"] else 256 // (N + 1) ** 2,
+                             "elements_per_block": 8 if t["path"] else
+                             threads // group[N] * (group[N] // (N + 1) ** 2),
                              "ms_per_inner_iter": t["ms_per_iter"]}
                     for N, t in sorted(tuned.items())},
-           "threads_per_block": 256}
+           "threads_per_block": threads}
     for c in ctxs:
         c.close()
     return out

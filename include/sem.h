@@ -291,8 +291,8 @@ SEM_API int sem_pcg_solve_noalloc(int N, int nelx, int nely, int nelz, const int
 
 /* Autotuner of the inner path of refinement for the context's order N.  The
  * candidates are the two FP32-accurate inner operators: 0 = the FP32
- * CUDA-core operator (256/(N+1)^2 elements per 256-thread block, slabs in
- * shared memory per element) and 1 = the split-operand FP16 tensor-core
+ * CUDA-core operator (whole lines; groups of one to eight warps, of one or more
+ * elements, in a block of 768 threads) and 1 = the split-operand FP16 tensor-core
  * operator (SEM_F16X2_TC: one element per warp, 8 per block; N <= 7 only).
  * Each runs `iters` inner PCG iterations (a Helmholtz problem on the
  * context's mesh, one persistent launch) after one untimed run; ms (NULL or

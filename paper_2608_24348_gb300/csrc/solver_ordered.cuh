@@ -9,8 +9,10 @@
 // by 2e-9 to 8e-9 (N = 7, 24^3 and 32^3 elements; 8e-8 at N = 8).  The solver of
 // solver.cuh is faster (5.4 ms a launch against 6.8 at 32^3, N = 7; half the
 // time at 16^3) but sums in another order; runs that are to repeat to 1e-9 therefore keep this one.
-// Solves whose tolerance ends the iteration on the solution itself, and steps
-// with GMRES, whose iterates agree to 1e-10 either way, use solver.cuh.
+// Every FP64 solve of such a step takes this solver, whatever its tolerance, but a
+// relative one below 1e-11 (native FP64 operator); where the tolerance ends the
+// iteration on the solution itself, the iterates agree to 1e-10 with either solver,
+// and this one costs up to twice the time.  Steps with GMRES use solver.cuh.
 //
 // Work items: groups of NE elements, chunks of 256 unique nodes on SEM_UQ_ROWS
 // rows, chunks of 256 local nodes; they are dealt to the CTAs in turn.  The last

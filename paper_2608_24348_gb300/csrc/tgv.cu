@@ -630,7 +630,8 @@ __global__ void __launch_bounds__(VelCfg<NP>::TH) k_tgv_vel(VArgs a, const __gri
 //
 // Bound: FP32 issue and HBM (13 words a node).  The nine derivatives run by whole
 // folded lines (ax_dfl.cuh), and only the six products that the vorticity needs
-// are formed; a node at a time, with all nine: 1.73 ms at 32^3, N = 7, now 1.07.
+// are formed; a node at a time, with all nine: 1.73 ms at 32^3, N = 7, now 1.17
+// (1.07 with the CFL number in float pairs as well).
 struct GapInv {
     double v[SEM_NPMAX];
 };
